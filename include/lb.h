@@ -78,12 +78,17 @@ enum { LB_HOST = 0, LB_DEVICE = 1 };
 
 /* Step kernels selectable with lb_set_kernel(). */
 enum {
-    LB_KERNEL_AUTO = 0,     /* library default, the fastest measured on GB300:
-                               LB_KERNEL_BULK (3 slots, clusters of 2, 16
-                               planes) for FP32-shifted 7-point BGK steps on
-                               rows of 256 sites with ny even, else
-                               LB_KERNEL_TWO_PASS                            */
-    LB_KERNEL_TWO_PASS = 1, /* phi pass + collide/stream pass (phi buffer)     */
+    LB_KERNEL_AUTO = 0,     /* library default, the fastest measured on GB300.
+                               FP32-shifted with tau_g = 1, more than 2^18
+                               sites and rows of 12 or more: within one
+                               lb_step call g is kept as its equilibrium's
+                               moments, and written in full by the last step.
+                               Else LB_KERNEL_BULK (3 slots, clusters of 2,
+                               16 planes) for FP32-shifted 7-point BGK steps
+                               with tau_g != 1 on rows of 256 sites with ny
+                               even, else LB_KERNEL_TWO_PASS                 */
+    LB_KERNEL_TWO_PASS = 1, /* phi pass + collide/stream pass (phi buffer);
+                               with tau_g = 1 the second does not read g     */
     LB_KERNEL_FUSED = 2,    /* single pass, phi halo staged in shared memory   */
     LB_KERNEL_STAGED = 3,   /* single pass, planes staged by asynchronous
                                copies into a 3-buffer shared-memory pipeline   */

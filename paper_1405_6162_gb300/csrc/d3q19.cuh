@@ -44,6 +44,14 @@ __device__ __forceinline__ void relax_pair(T c, T &fp, T &fm, T s, T a)
     fm = fmadd_sum(c, fm, s, -a);
 }
 
+// fp = s + a, fm = s - a: the values of an opposite pair at equilibrium
+template <typename T>
+__device__ __forceinline__ void equilibrium_pair(T &fp, T &fm, T s, T a)
+{
+    fp = s + a;
+    fm = s - a;
+}
+
 template <typename T>
 __device__ __forceinline__ void store(T *p, T v)
 {
@@ -74,6 +82,9 @@ __host__ __device__ constexpr double weight(int i) {
 // x / 2 (exact in binary floating point)
 __device__ __forceinline__ float half(float x) { return 0.5f * x; }
 __device__ __forceinline__ double half(double x) { return 0.5 * x; }
+// 2 x (exact)
+__device__ __forceinline__ float twice(float x) { return 2.0f * x; }
+__device__ __forceinline__ double twice(double x) { return 2.0 * x; }
 
 // Relaxation and free-energy parameters in the arithmetic type T.  The
 // relaxation constants fold omega = 1/tau into the lattice weights so that
@@ -235,22 +246,42 @@ __device__ __forceinline__ void collide_f(const Coll<T>& p, T (&f)[Q], T phi, T 
 }
 
 // In-place BGK collision of g at one site with velocity u and chemical
-// potential mu.
-template <typename T>
+// potential mu.  GEQ (tau_g = 1, so 1 - omega_g = 0): g* is the equilibrium,
+// g comes in undefined and the products with 1 - omega_g are left out -- the
+// same values, since 0 * g adds nothing to a finite sum and a g that is not
+// finite reaches g* through phi = sum g.
+template <typename T, bool GEQ = false>
 __device__ __forceinline__ void collide_g(const Coll<T>& p, T (&g)[Q], T phi, T ux, T uy, T uz, T mu)
 {
-    const T third = T(1.0 / 3.0), h = T(4.5);
     // ---- g: omega_g geq_i = omega_g w_i [phi + 3 phi c.u + 9/2 (phi (c.u)^2 - phi u^2/3 + (Gamma mu - phi/3)(c^2 - 1))]
     const T cg = p.cg;
     const T px = phi * ux, py = phi * uy, pz = phi * uz;
-    const T gm = p.gamma * mu - phi * third;
+    // 9/2 (Gamma mu - phi/3).  As the sum of 9 Gamma/2 mu and -3/2 phi it has
+    // no factor 1/3, whose float rounding enters every step with the same sign
+    // (tau_g = 1: phi's FP32 error after 200 spinodal steps is a third without
+    // it).  The other paths keep the factor: the sum changed their register
+    // allocation for the worse (double-float 3 %, FP32 with tau_g != 1 0.6 %).
+    T gm;
+    if constexpr (GEQ && sizeof(T) == sizeof(float))
+        gm = (T(4.5) * p.gamma) * mu - T(1.5) * phi;
+    else
+        gm = T(4.5) * (p.gamma * mu - phi * T(1.0 / 3.0));
     const T bg = phi - T(1.5) * (px * ux + py * uy + pz * uz);   // phi - 9/2 phi u^2 / 3
-    g[0] = fmadd(cg, g[0], p.g0 * (bg - h * gm));
-    const T G1 = p.g1 * bg, G2 = p.g2 * (bg + h * gm);
+    if constexpr (GEQ)
+        g[0] = p.g0 * (bg - gm);
+    else
+        g[0] = fmadd(cg, g[0], p.g0 * (bg - gm));
+    auto relax = [&](T &gp, T &gmi, T s, T a) {
+        if constexpr (GEQ)
+            equilibrium_pair(gp, gmi, s, a);
+        else
+            relax_pair(cg, gp, gmi, s, a);
+    };
+    const T G1 = p.g1 * bg, G2 = p.g2 * (bg + gm);
 #define LBK_GFACE(IP, IM, PA, UA)                                   \
     {                                                               \
         const T s_ = fmadd(p.g1h, PA * UA, G1), a_ = p.g1t * PA;    \
-        relax_pair(cg, g[IP], g[IM], s_, a_);                       \
+        relax(g[IP], g[IM], s_, a_);                                \
     }
     LBK_GFACE(1, 2, px, ux)
     LBK_GFACE(3, 4, py, uy)
@@ -260,7 +291,7 @@ __device__ __forceinline__ void collide_g(const Coll<T>& p, T (&g)[Q], T phi, T 
     {                                                               \
         const T pc_ = PC, cu_ = CU;                                 \
         const T s_ = fmadd(p.g2h, pc_ * cu_, G2), a_ = p.g2t * pc_; \
-        relax_pair(cg, g[IP], g[IM], s_, a_);                       \
+        relax(g[IP], g[IM], s_, a_);                                \
     }
     LBK_GEDGE(7, 8, px + py, ux + uy)
     LBK_GEDGE(9, 10, px - py, ux - uy)
@@ -303,9 +334,8 @@ struct Mrt {
     T hFx, hFy, hFz;   // F/2
 };
 
-// In-place multiple-relaxation-time collision of f with a Guo body force,
-// then the BGK collision of g with the force-corrected velocity
-// u = (j + F/2)/rho.  With N = sum (f - feq) c c (= Pi - R/3 I - S in the
+// In-place multiple-relaxation-time collision of f with a Guo body force;
+// also returns the force-corrected velocity u = (j + F/2)/rho and mu.  With N = sum (f - feq) c c (= Pi - R/3 I - S in the
 // shifted form), G = u F + F u, each split into bulk (trace/3 I) and shear
 // (traceless) parts,
 //   X  = (1 - w_s) N_s + (1 - w_b) N_b + (1 - w_s/2) G_s + (1 - w_b/2) G_b,
@@ -315,8 +345,8 @@ struct Mrt {
 //   S' = w_gh S + X - (1 - w_gh) N,
 // which is BGK when the three rates are equal and F = 0.
 template <typename T, bool SH>
-__device__ __forceinline__ void collide_mrt(const Coll<T>& p, const Mrt<T>& m, T (&f)[Q], T (&g)[Q],
-                                            T phi, T dx, T dy, T dz, T lap)
+__device__ __forceinline__ void collide_mrt_f(const Coll<T>& p, const Mrt<T>& m, T (&f)[Q], T phi, T dx, T dy,
+                                              T dz, T lap, T& ux, T& uy, T& uz, T& mu)
 {
     T R, jx, jy, jz;
     density_moments(f, R, jx, jy, jz);
@@ -324,9 +354,11 @@ __device__ __forceinline__ void collide_mrt(const Coll<T>& p, const Mrt<T>& m, T
     const T rho = SH ? p.rho0 + R : R;
     const T rinv = T(1) / rho;
     const T Jx = jx + m.hFx, Jy = jy + m.hFy, Jz = jz + m.hFz;   // rho u
-    const T ux = Jx * rinv, uy = Jy * rinv, uz = Jz * rinv;
+    ux = Jx * rinv;
+    uy = Jy * rinv;
+    uz = Jz * rinv;
     const T phi2 = phi * phi;
-    const T mu = phi * (p.A + p.B * phi2) - p.kappa * lap;
+    mu = phi * (p.A + p.B * phi2) - p.kappa * lap;
     const T pb = phi2 * (T(0.5) * p.A + T(0.75) * p.B * phi2)
                - p.kappa * (phi * lap + T(0.5) * (dx * dx + dy * dy + dz * dz));
     // S = P + rho u u
@@ -395,6 +427,15 @@ __device__ __forceinline__ void collide_mrt(const Coll<T>& p, const Mrt<T>& m, T
     LBK_MEDGES(11, 12, 13, 14, Spxx, Spzz, Spxz, Jpx, Jpz)
     LBK_MEDGES(15, 16, 17, 18, Spyy, Spzz, Spyz, Jpy, Jpz)
 #undef LBK_MEDGES
+}
+
+// collide_mrt_f, then the collision of g with the force-corrected velocity
+template <typename T, bool SH>
+__device__ __forceinline__ void collide_mrt(const Coll<T>& p, const Mrt<T>& m, T (&f)[Q], T (&g)[Q],
+                                            T phi, T dx, T dy, T dz, T lap)
+{
+    T ux, uy, uz, mu;
+    collide_mrt_f<T, SH>(p, m, f, phi, dx, dy, dz, lap, ux, uy, uz, mu);
     collide_g<T>(p, g, phi, ux, uy, uz, mu);
 }
 

@@ -185,6 +185,9 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b)
 // x / 2: both parts halved, exactly (barring underflow)
 __device__ __forceinline__ df64 half(df64 a) { return df64(0.5f * a.hi, 0.5f * a.lo); }
 
+// 2 x (exact)
+__device__ __forceinline__ df64 twice(df64 a) { return df64(2.0f * a.hi, 2.0f * a.lo); }
+
 // a / b: a float quotient refined twice by the residual a - q b
 __device__ __forceinline__ df64 operator/(df64 a, df64 b)
 {
@@ -255,6 +258,20 @@ __device__ __forceinline__ void relax_pair(df64 c, df64 &fp, df64 &fm, df64 s, d
     two_sum(p, s1, sum, t2);
     const unsigned long long t = add(add(t1, t2), add(e, add(sl, al)));
     // fast two-sum of (sum, t)
+    const unsigned long long rh = add(sum, t);
+    const unsigned long long rl = sub(t, sub(rh, sum));
+    unpack(rh, fp.hi, fm.hi);
+    unpack(rl, fp.lo, fm.lo);
+}
+
+// fp = s + a, fm = s - a, each operator+'s float sequence, both through one
+// pass of paired FP32 instructions
+__device__ __forceinline__ void equilibrium_pair(df64 &fp, df64 &fm, df64 s, df64 a)
+{
+    using namespace px2;
+    unsigned long long sum, e;
+    two_sum(pack(s.hi, s.hi), pack(a.hi, -a.hi), sum, e);
+    const unsigned long long t = add(e, add(pack(s.lo, s.lo), pack(a.lo, -a.lo)));
     const unsigned long long rh = add(sum, t);
     const unsigned long long rl = sub(t, sub(rh, sum));
     unpack(rh, fp.hi, fm.hi);

@@ -157,16 +157,16 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kBatchMaxThreads64 : kBatchMa
                 const LatDesc<T> &L = lats[it.x];
                 const long long s = (long long)it.y * blockDim.x + threadIdx.x;
                 if (s < L.N)
-                    t1_collide_site<T, SH, 7>(L.f[a], const_cast<T *>(L.g[a]), const_cast<T *>(L.f[1 - a]), L.p,
-                                              L.nx, L.ny, L.nz, L.S, (int)s);
+                    t1_collide_site<T, SH, 7>(L.f[a], L.g[a], quads(const_cast<T *>(L.g[a]), L.S),
+                                              const_cast<T *>(L.f[1 - a]), L.p, L.nx, L.ny, L.nz, L.S, (int)s);
             }
             if ((int)blockIdx.x == skip_cta) return;   // test hook: this CTA never arrives
             if (!grid_sync(bar, G.m, timeout_ns, err, &s_fail)) return;
             for (int w = G.to + r; w < tend; w += G.m) {
                 const int4 it = work_t1[w];   // (lattice, x block, warp group, z run)
                 const LatDesc<T> &L = lats[it.x];
-                t1_phi_tile<T, KY>(L.g[a], const_cast<T *>(L.g[1 - a]), L.nx, L.ny, L.nz, L.kzc, L.S, it.y,
-                                   (it.z * warps + warp) * KY, it.w, lane);
+                t1_phi_tile<T, KY>(L.g[a], quads(L.g[a], L.S), const_cast<T *>(L.g[1 - a]), L.nx, L.ny, L.nz, L.kzc,
+                                   it.y, (it.z * warps + warp) * KY, it.w, lane);
             }
             if (!grid_sync(bar, G.m, timeout_ns, err, &s_fail)) return;
         }

@@ -564,12 +564,14 @@ static int run_bulk(lb_ctx *c, int nsteps)
 // the shape the library default uses: 3 slots, clusters of 2, 16 planes per
 // CTA (the fastest measured at 256^3 FP32-shifted on GB300), on rows of 256
 // sites (eight warps a CTA; at 128^3, four warps a CTA, the two-pass step is
-// faster: 17.4 against 14.2 GLUPS)
+// faster: 17.4 against 14.2 GLUPS) and tau_g != 1: with tau_g = 1 g need not
+// be read by the collision, and 50 steps of 256^3 take 530 us each
+// (lb_taug1.cu) against 902 here, a single one 777
 constexpr int kAutoSlots = 3, kAutoCluster = 2, kAutoPlanes = 16;
 
 bool auto_uses_bulk(const lb_ctx *c)
 {
-    return c->p.precision == LB_FP32_SHIFTED && c->npts == 7 && !uses_mrt(c) && c->p.nx == kBulkMaxRow &&
+    return !g_is_equilibrium(c->p) && c->p.precision == LB_FP32_SHIFTED && c->npts == 7 && !uses_mrt(c) && c->p.nx == kBulkMaxRow &&
            bulk_validate(c->p, kAutoSlots, kAutoCluster, kAutoPlanes) == LB_OK;
 }
 

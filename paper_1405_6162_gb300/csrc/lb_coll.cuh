@@ -7,6 +7,11 @@
 
 namespace lbk {
 
+// tau_g = 1: the collision of g returns its equilibrium, whatever g was
+// (1 - omega_g = 0 in every arithmetic type), so the passes that would only
+// multiply g by that zero need not read it
+inline bool g_is_equilibrium(const lb_params &p) { return p.tau_g == 1.0; }
+
 // Parameters of the step in the arithmetic type T (constants formed in
 // double, rounded once).
 template <typename T>

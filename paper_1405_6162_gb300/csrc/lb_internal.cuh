@@ -117,6 +117,10 @@ int two_pass_validate(int block_x, int block_y, int z_chunk);   // threads per C
 // of N doubles supplied by the caller)
 int launch_two_pass_fp64_raw(const lb_params &p, const double *fa, const double *ga, double *phi, double *fb,
                              double *gb, long long S, cudaStream_t stream);
+// the FP32-shifted passes of a step with tau_g = 1: phi of the stored g, and
+// the collide/stream pass that does not read g
+cudaError_t launch_phi_pull(lb_ctx *c, const float *ga, float *phi);
+cudaError_t launch_collide_geq(lb_ctx *c, const float *fa, const float *phi, float *fb, float *gb);
 int launch_moments(lb_ctx *c, double *rho, double *u, double *phi);
 int launch_get_state(lb_ctx *c, double *f, double *g);
 int launch_set_state(lb_ctx *c, const double *f, const double *g);
@@ -148,6 +152,11 @@ int taug1_validate(const lb_params &p, int block_x, int block_y, int z_chunk);
 int taug1_convert(lb_ctx *c, int to_reduced);
 int taug1_g_rows(lb_ctx *c, int i0, int i1, double *out);
 int taug1_phi_out(lb_ctx *c, double *out);
+
+// LB_KERNEL_AUTO with tau_g = 1, FP32-shifted: steps that keep g as its
+// equilibrium's moments within a call
+bool auto_uses_geq(const lb_ctx *c);
+int launch_step_geq(lb_ctx *c, int nsteps);
 
 // masked copies (lb_masked.cu)
 size_t masked_scratch_ints(long long N);

@@ -9,6 +9,8 @@
 // sites are consecutive in memory).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "d3q19.cuh"
 #include "lb_internal.cuh"
 #include "lb_pdl.cuh"
@@ -48,7 +50,11 @@ __global__ void __launch_bounds__(256) k_phi_pull(const T *__restrict__ ga, T *_
 
 // CTAs per SM the register budget of the collide/stream kernel must allow
 // (measured: FP64 is bound by the FP64 pipe at 2 or 3; an allowance of 1
-// lets ptxas spend 152 registers and loses 11 %; FP32 is DRAM-bound)
+// lets ptxas spend 152 registers and loses 11 %; FP32 is DRAM-bound).
+// Double-float with g unread (GEQ): without g's 38 words in flight 96
+// registers do, in CTAs of 128 threads five to an SM -- 221 us a step at
+// 144x120x100 against 255 with two CTAs of 256 and 240 with g read
+// (arithmetic-bound either way: the 20 warps are what hides its latency).
 #ifndef LBK_K2_MINB64
 #define LBK_K2_MINB64 2
 #endif
@@ -61,11 +67,17 @@ __global__ void __launch_bounds__(256) k_phi_pull(const T *__restrict__ ga, T *_
 #ifndef LBK_K2_MINB32W
 #define LBK_K2_MINB32W 3   // FP32 with the 19- / 27-point stencils
 #endif
-#define LBK_K2_MINB(T, NP) \
-    (is_df64<T>::value ? LBK_K2_MINBDF : sizeof(T) == 8 ? LBK_K2_MINB64 : NP > 7 ? LBK_K2_MINB32W : LBK_K2_MINB32)
+#ifndef LBK_K2_MINBDFG
+#define LBK_K2_MINBDFG 5   // double-float, GEQ (of 128 threads)
+#endif
+#define LBK_K2_MAXT(T, GEQ) (is_df64<T>::value && (GEQ) ? 128 : 256)
+#define LBK_K2_MINB(T, NP, GEQ)                                                                        \
+    (is_df64<T>::value ? ((GEQ) ? LBK_K2_MINBDFG : LBK_K2_MINBDF) : sizeof(T) == 8 ? LBK_K2_MINB64   \
+                                                                  : NP > 7 ? LBK_K2_MINB32W : LBK_K2_MINB32)
 
-template <typename T, bool SH, int NP = 7>
-__global__ void __launch_bounds__(256, LBK_K2_MINB(T, NP)) k_collide_pull(const T *__restrict__ fa, const T *__restrict__ ga,
+// GEQ: tau_g = 1, g is not read (collide_site)
+template <typename T, bool SH, int NP, bool GEQ>
+__global__ void __launch_bounds__(LBK_K2_MAXT(T, GEQ), LBK_K2_MINB(T, NP, GEQ)) k_collide_pull(const T *__restrict__ fa, const T *__restrict__ ga,
                                                       const T *__restrict__ phi,
                                                       T *__restrict__ fb, T *__restrict__ gb,
                                                       Coll<T> p, int nx, int ny, int nz, long long S)
@@ -75,12 +87,12 @@ __global__ void __launch_bounds__(256, LBK_K2_MINB(T, NP)) k_collide_pull(const 
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
     const Nbr n(s, nx, ny, nz);
-    collide_site<T, SH, NP>(fa, ga, phi, fb, gb, p, n, s, S);
+    collide_site<T, SH, NP, GEQ>(fa, ga, phi, fb, gb, p, n, s, S);
 }
 
 // multiple-relaxation-time collision of f with a Guo body force (collide_mrt)
-template <typename T, bool SH, int NP>
-__global__ void __launch_bounds__(256, LBK_K2_MINB(T, NP))
+template <typename T, bool SH, int NP, bool GEQ>
+__global__ void __launch_bounds__(LBK_K2_MAXT(T, GEQ), LBK_K2_MINB(T, NP, GEQ))
 k_collide_pull_mrt(const T *__restrict__ fa, const T *__restrict__ ga, const T *__restrict__ phi,
                    T *__restrict__ fb, T *__restrict__ gb, Coll<T> p, Mrt<T> m, int nx, int ny, int nz,
                    long long S)
@@ -90,22 +102,7 @@ k_collide_pull_mrt(const T *__restrict__ fa, const T *__restrict__ ga, const T *
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
     const Nbr n(s, nx, ny, nz);
-    T f[Q], g[Q];
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-        const size_t o = (size_t)i * S + n.src(i);
-        f[i] = fa[o];
-        g[i] = ga[o];
-    }
-    const T ph = phi[s];
-    T dx, dy, dz, lap;
-    stencil_np<NP, T>(phi, n, ph, dx, dy, dz, lap);
-    collide_mrt<T, SH>(p, m, f, g, ph, dx, dy, dz, lap);
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-        fb[(size_t)i * S + s] = f[i];
-        gb[(size_t)i * S + s] = g[i];
-    }
+    collide_site<T, SH, NP, GEQ>(fa, ga, phi, fb, gb, p, n, s, S, &m);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -114,40 +111,44 @@ static inline unsigned grid_for(long long N, int tpb) { return (unsigned)((N + t
 
 // the phi pass with V sites per thread
 template <typename T>
-static cudaError_t launch_phi(lb_ctx *c, const T *ga, int tpb, int vvl)
+static cudaError_t launch_phi(lb_ctx *c, const T *ga, T *phi, int tpb, int vvl)
 {
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     const unsigned grid = grid_for(c->N, tpb * vvl);
-    if (vvl == 4) return launch_pdl(k_phi_pull<T, 4>, grid, tpb, c->stream, ga, (T *)c->phi, nx, ny, nz, c->S);
-    if (vvl == 2) return launch_pdl(k_phi_pull<T, 2>, grid, tpb, c->stream, ga, (T *)c->phi, nx, ny, nz, c->S);
-    return launch_pdl(k_phi_pull<T, 1>, grid, tpb, c->stream, ga, (T *)c->phi, nx, ny, nz, c->S);
+    if (vvl == 4) return launch_pdl(k_phi_pull<T, 4>, grid, tpb, c->stream, ga, phi, nx, ny, nz, c->S);
+    if (vvl == 2) return launch_pdl(k_phi_pull<T, 2>, grid, tpb, c->stream, ga, phi, nx, ny, nz, c->S);
+    return launch_pdl(k_phi_pull<T, 1>, grid, tpb, c->stream, ga, phi, nx, ny, nz, c->S);
+}
+
+// the collide/stream pass from level fa, ga (and phi of the state) to fb, gb
+template <typename T, bool SH, int NP, bool GEQ>
+static cudaError_t launch_collide(lb_ctx *c, const T *fa, const T *ga, const T *phi, T *fb, T *gb, int tpb)
+{
+    const auto p = make_coll<T>(c->p);
+    tpb = std::min(tpb, LBK_K2_MAXT(T, GEQ));
+    const unsigned grid = grid_for(c->N, tpb);
+    const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
+    if (uses_mrt(c))
+        return launch_pdl(k_collide_pull_mrt<T, SH, NP, GEQ>, grid, tpb, c->stream, fa, ga, phi, fb, gb, p,
+                          make_mrt<T>(c), nx, ny, nz, c->S);
+    return launch_pdl(k_collide_pull<T, SH, NP, GEQ>, grid, tpb, c->stream, fa, ga, phi, fb, gb, p, nx, ny, nz, c->S);
 }
 
 template <typename T, bool SH, int NP>
 static int two_pass(lb_ctx *c, int nsteps)
 {
-    const auto p = make_coll<T>(c->p);
-    const bool mrt = uses_mrt(c);
-    const auto m = make_mrt<T>(c);
     // launch shape: threads per CTA of both passes, sites per thread of the
     // phi pass (lb_set_kernel's block_x, block_y; 0 = 256 and 1)
     const int tpb = c->block_x ? c->block_x : 256;
     const int vvl = c->block_y ? c->block_y : 1;
-    const unsigned grid = grid_for(c->N, tpb);
-    const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     for (int t = 0; t < nsteps; t++) {
         const int a = c->buf.cur, b = 1 - a;
-        const T *fa = (const T *)c->buf.f[a], *ga = (const T *)c->buf.g[a];
+        const T *fa = (const T *)c->buf.f[a], *ga = (const T *)c->buf.g[a], *phi = (const T *)c->phi;
         T *fb = (T *)c->buf.f[b], *gb = (T *)c->buf.g[b];
-        cudaError_t e = launch_phi<T>(c, ga, tpb, vvl);
-        if (e == cudaSuccess) {
-            if (mrt)
-                e = launch_pdl(k_collide_pull_mrt<T, SH, NP>, grid, tpb, c->stream, fa, ga, (const T *)c->phi, fb, gb,
-                               p, m, nx, ny, nz, c->S);
-            else
-                e = launch_pdl(k_collide_pull<T, SH, NP>, grid, tpb, c->stream, fa, ga, (const T *)c->phi, fb, gb, p,
-                               nx, ny, nz, c->S);
-        }
+        cudaError_t e = launch_phi<T>(c, ga, (T *)c->phi, tpb, vvl);
+        if (e == cudaSuccess)
+            e = g_is_equilibrium(c->p) ? launch_collide<T, SH, NP, true>(c, fa, ga, phi, fb, gb, tpb)
+                                       : launch_collide<T, SH, NP, false>(c, fa, ga, phi, fb, gb, tpb);
         int rc = e != cudaSuccess ? cuda_status(e) : check_launch();
         if (rc) return rc;
         c->buf.cur = b;
@@ -162,8 +163,27 @@ int launch_two_pass_fp64_raw(const lb_params &prm, const double *fa, const doubl
     const long long N = (long long)prm.nx * prm.ny * prm.nz;
     const unsigned grid = grid_for(N, 256);
     k_phi_pull<double, 1><<<grid, 256, 0, stream>>>(ga, phi, prm.nx, prm.ny, prm.nz, S);
-    k_collide_pull<double, false><<<grid, 256, 0, stream>>>(fa, ga, phi, fb, gb, p, prm.nx, prm.ny, prm.nz, S);
+    if (g_is_equilibrium(prm))
+        k_collide_pull<double, false, 7, true><<<grid, 256, 0, stream>>>(fa, ga, phi, fb, gb, p, prm.nx, prm.ny,
+                                                                         prm.nz, S);
+    else
+        k_collide_pull<double, false, 7, false><<<grid, 256, 0, stream>>>(fa, ga, phi, fb, gb, p, prm.nx, prm.ny,
+                                                                          prm.nz, S);
     return check_launch();
+}
+
+cudaError_t launch_phi_pull(lb_ctx *c, const float *ga, float *phi)
+{
+    return launch_phi<float>(c, ga, phi, c->block_x ? c->block_x : 256, c->block_y ? c->block_y : 1);
+}
+
+cudaError_t launch_collide_geq(lb_ctx *c, const float *fa, const float *phi, float *fb, float *gb)
+{
+    const int tpb = c->block_x ? c->block_x : 256;
+    const float *no_g = nullptr;
+    if (c->npts == 19) return launch_collide<float, true, 19, true>(c, fa, no_g, phi, fb, gb, tpb);
+    if (c->npts == 27) return launch_collide<float, true, 27, true>(c, fa, no_g, phi, fb, gb, tpb);
+    return launch_collide<float, true, 7, true>(c, fa, no_g, phi, fb, gb, tpb);
 }
 
 template <typename T, bool SH>

@@ -102,12 +102,13 @@ __device__ __forceinline__ T phi_site(const T *__restrict__ ga, const Nbr &n, lo
 }
 
 // Pull f and g to site s, collide with the NP-point phi stencil, write the
-// post-collision values at s.
-template <typename T, bool SH, int NP = 7>
+// post-collision values at s.  GEQ (tau_g = 1): g is not read, its result
+// depends on it through phi alone.  With m the collision of f is collide_mrt.
+template <typename T, bool SH, int NP = 7, bool GEQ = false>
 __device__ __forceinline__ void collide_site(const T *__restrict__ fa, const T *__restrict__ ga,
                                              const T *__restrict__ phi, T *__restrict__ fb,
                                              T *__restrict__ gb, const Coll<T> &p, const Nbr &n, long long s,
-                                             long long S)
+                                             long long S, const Mrt<T> *m = nullptr)
 {
     T f[Q], g[Q];
     const T ph = phi[s];
@@ -120,14 +121,31 @@ __device__ __forceinline__ void collide_site(const T *__restrict__ fa, const T *
     for (int i = 0; i < Q; i++) {
         const size_t o = (size_t)i * S + n.src(i);
         f[i] = fa[o];
-        g[i] = ga[o];
+        if constexpr (!GEQ) g[i] = ga[o];
     }
     if constexpr (NP != 27) stencil_np<NP, T>(phi, n, ph, dx, dy, dz, lap);
-    collide<T, SH>(p, f, g, ph, dx, dy, dz, lap);
+    if constexpr (GEQ) {
+        // f's values are stored, and their registers free, before g's are formed
+        T ux, uy, uz, mu;
+        if (m)
+            collide_mrt_f<T, SH>(p, *m, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
+        else
+            collide_f<T, SH>(p, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        fb[(size_t)i * S + s] = f[i];
-        gb[(size_t)i * S + s] = g[i];
+        for (int i = 0; i < Q; i++) fb[(size_t)i * S + s] = f[i];
+        collide_g<T, true>(p, g, ph, ux, uy, uz, mu);
+#pragma unroll
+        for (int i = 0; i < Q; i++) gb[(size_t)i * S + s] = g[i];
+    } else {
+        if (m)
+            collide_mrt<T, SH>(p, *m, f, g, ph, dx, dy, dz, lap);
+        else
+            collide<T, SH>(p, f, g, ph, dx, dy, dz, lap);
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            fb[(size_t)i * S + s] = f[i];
+            gb[(size_t)i * S + s] = g[i];
+        }
     }
 }
 

@@ -10,10 +10,11 @@
 
 namespace lbk {
 
-// a source site's moments expanded for geq: base by c^2 (0, 1, 2), 3 phi, 9/2 phi, u
+// a source site's moments expanded for geq: base by c^2 (0, 1, 2), 3 phi,
+// 9/2 phi, u, u^2
 template <typename T>
 struct Eq {
-    T b0, b1, b2, a3, a45, ux, uy, uz;
+    T b0, b1, b2, a3, a45, ux, uy, uz, u2;
 };
 
 template <typename T>
@@ -29,13 +30,15 @@ __device__ __forceinline__ Eq<T> make_eq(T phi, T gmh, T ux, T uy, T uz)
     e.ux = ux;
     e.uy = uy;
     e.uz = uz;
+    e.u2 = u2;
     return e;
 }
 
+// gmh = 9/2 (Gamma mu - phi/3), without a factor 1/3 (collide_g)
 template <typename T>
 __device__ __forceinline__ T gmh_of(T phi, T mu, T gamma)
 {
-    return T(4.5) * (gamma * mu - phi * T(1.0 / 3.0));
+    return (T(4.5) * gamma) * mu - T(1.5) * phi;
 }
 
 // c_i . u with the zero components left out; i a literal after inlining
@@ -73,10 +76,36 @@ __device__ __forceinline__ T geq_eq(int i, const Eq<T> &e)
     return T(weight(i)) * add_px(base, cu * add_px(e.a3, e.a45 * cu));
 }
 
-// The phi pass's form of the equilibria.  For an opposite pair (i, i + 1;
+// The phi pass sums the 18 moving equilibria of the sources around a site in
+// units of 1/36, the weights being the integers 2 (faces) and 1 (edges), and
+// takes the rest value as what the site's own 18 leave of its phi:
+//   phi(t+1) = phi + (U - 12 t) / 36,
+//   U = sum_{i>0} 36 geq_i(x - c_i),
+//   12 t = sum_{i>0} 36 geq_i(x),  t = b1 + b2 + 9/2 phi u^2.
+// The U of all sites add up to their 12 t but for unbiased rounding, so phi
+// is conserved like that of the general step, whose g*_0 takes up the rounding
+// of the other 18 (d3q19.cuh).  With the rest value formed from its own
+// weight instead, phi's FP32 error against FP64 grew by about 5e-9 of phi a
+// step, to 1.9 times the general step's after 200 steps.
+template <typename T>
+__device__ __forceinline__ T moving_sum(const Eq<T> &e)
+{
+    return (e.b1 + e.b2) + e.a45 * e.u2;
+}
+
+// 36 geq_i of a moving direction; i a literal after inlining.  The face
+// weight multiplies the class terms, which is exact.
+template <typename T>
+__device__ __forceinline__ T geq36(int i, const Eq<T> &e)
+{
+    const T cu = cdot(i, e.ux, e.uy, e.uz);
+    return i <= 6 ? twice(e.b1 + cu * (e.a3 + e.a45 * cu)) : e.b2 + cu * (e.a3 + e.a45 * cu);
+}
+
+// The phi pass's form for double-float.  For an opposite pair (i, i + 1;
 // i odd, c_{i+1} = -c_i) with cu = c_i . u,
-//   geq_i = S + A,  geq_{i+1} = S - A,  S = w (b + 9/2 phi cu^2),  A = 3 w phi cu,
-// w and b those of the pair's weight class, so that a pair costs one S and
+//   36 geq_i = S + A,  36 geq_{i+1} = S - A,  S = W (b + 9/2 phi cu^2),  A = 3 W phi cu,
+// W and b those of the pair's weight class, so that a pair costs one S and
 // one A.  The class terms are formed once per source site.
 static_assert(cx(2) == -cx(1) && cy(4) == -cy(3) && cz(6) == -cz(5) && cx(8) == -cx(7) && cy(8) == -cy(7) &&
                   cy(10) == -cy(9) && cz(12) == -cz(11) && cz(14) == -cz(13) && cy(16) == -cy(15) &&
@@ -85,8 +114,7 @@ static_assert(cx(2) == -cx(1) && cy(4) == -cy(3) && cz(6) == -cz(5) && cx(8) == 
 
 template <typename T>
 struct EqPair {
-    T r0;                       // geq_0
-    T wb[2], wq[2], wa[2];      // per class (faces, edges): w b, 9/2 w phi, 3 w phi
+    T wb[2], wq[2], wa[2];      // per class (faces, edges): W b, 9/2 W phi, 3 W phi
     T ux, uy, uz;
 };
 
@@ -94,14 +122,12 @@ template <typename T>
 __device__ __forceinline__ EqPair<T> pair_form(const Eq<T> &e)
 {
     EqPair<T> p;
-    p.r0 = geq_eq(0, e);
-    const T w1 = T(weight(1)), w2 = T(weight(7));
-    p.wb[0] = w1 * e.b1;
-    p.wb[1] = w2 * e.b2;
-    p.wq[0] = w1 * e.a45;
-    p.wq[1] = w2 * e.a45;
-    p.wa[0] = w1 * e.a3;
-    p.wa[1] = w2 * e.a3;
+    p.wb[0] = twice(e.b1);
+    p.wb[1] = e.b2;
+    p.wq[0] = twice(e.a45);
+    p.wq[1] = e.a45;
+    p.wa[0] = twice(e.a3);
+    p.wa[1] = e.a3;
     p.ux = e.ux;
     p.uy = e.uy;
     p.uz = e.uz;
@@ -177,9 +203,9 @@ __device__ __forceinline__ df64 shfl_down1(df64 v)
 
 // the quads start at component 1 (S is a multiple of 64 elements, so they are aligned)
 template <typename T>
-__device__ __forceinline__ const T *quads(const T *g, long long S) { return g + S; }
+__host__ __device__ __forceinline__ const T *quads(const T *g, long long S) { return g + S; }
 template <typename T>
-__device__ __forceinline__ T *quads(T *g, long long S) { return g + S; }
+__host__ __device__ __forceinline__ T *quads(T *g, long long S) { return g + S; }
 
 // moments of site src stored in the reduced form
 template <typename T>
@@ -190,15 +216,15 @@ __device__ __forceinline__ Eq<T> load_eq(const T *__restrict__ g, long long S, l
     return make_eq(g[src], v[0], v[1], v[2], v[3]);
 }
 
-// The collide pass at site s: pull f, the NP-point stencil of phi(t) from
-// component 0 of level a, the general collision's f part; write f* and the
-// quad (gmh, u) of (s, t) into level a.
+// The collide pass at site s: pull f, the NP-point stencil of phi(t), the
+// general collision's f part (collide_mrt's with m); write f* and the quad
+// (gmh, u) of (s, t).
 template <typename T, bool SH, int NP>
-__device__ __forceinline__ void t1_collide_site(const T *__restrict__ fa, T *__restrict__ ga, T *__restrict__ fb,
-                                                const Coll<T> &p, int nx, int ny, int nz, long long S, int s)
+__device__ __forceinline__ void t1_collide_site(const T *__restrict__ fa, const T *__restrict__ phi,
+                                                T *__restrict__ quad, T *__restrict__ fb, const Coll<T> &p, int nx,
+                                                int ny, int nz, long long S, int s, const Mrt<T> *m = nullptr)
 {
     const Nbr n(s, nx, ny, nz);
-    const T *phi = ga;
     T f[Q];
 #pragma unroll
     for (int i = 0; i < Q; i++) f[i] = fa[(size_t)i * S + n.src(i)];
@@ -207,10 +233,13 @@ __device__ __forceinline__ void t1_collide_site(const T *__restrict__ fa, T *__r
     stencil_np<NP, T>(phi, n, ph, dx, dy, dz, lap);
     // the general collision's f part; g's result is its equilibrium, kept as moments
     T ux, uy, uz, mu;
-    collide_f<T, SH>(p, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
+    if (m)
+        collide_mrt_f<T, SH>(p, *m, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
+    else
+        collide_f<T, SH>(p, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
 #pragma unroll
     for (int i = 0; i < Q; i++) fb[(size_t)i * S + s] = f[i];
-    Quad<T>::store(quads(ga, S), s, gmh_of(ph, mu, p.gamma), ux, uy, uz);
+    Quad<T>::store(quad, s, gmh_of(ph, mu, p.gamma), ux, uy, uz);
 }
 
 constexpr int kPhiOut = 30;    // output columns per warp
@@ -238,11 +267,11 @@ __device__ __forceinline__ int wrap_up(int v, int n)
 
 // raw moments (phi, gmh, u) of site o
 template <typename T>
-__device__ __forceinline__ void t1_load_site(const T *__restrict__ ga, const T *__restrict__ q0, int o, T (&d)[5])
+__device__ __forceinline__ void t1_load_site(const T *__restrict__ phi, const T *__restrict__ q0, int o, T (&d)[5])
 {
     T v[4];
     Quad<T>::load(q0, o, v);
-    d[0] = ga[o], d[1] = v[0], d[2] = v[1], d[3] = v[2], d[4] = v[3];
+    d[0] = phi[o], d[1] = v[0], d[2] = v[1], d[3] = v[2], d[4] = v[3];
 }
 
 // The phi pass for the tile of one warp: x columns bx*30 - 1 .. bx*30 + 30
@@ -253,8 +282,9 @@ __device__ __forceinline__ void t1_load_site(const T *__restrict__ ga, const T *
 // j + 1, so a plane of arithmetic covers each load's latency and one plane
 // of raw moments is held.  Site offsets fit an int (N < 2^31).
 template <typename T, int KY>
-__device__ __forceinline__ void t1_phi_tile(const T *__restrict__ ga, T *__restrict__ gb, int nx, int ny, int nz,
-                                            int kzc, long long S, int bx, int y0, int bz, int lane)
+__device__ __forceinline__ void t1_phi_tile(const T *__restrict__ phi, const T *__restrict__ q0,
+                                            T *__restrict__ phi_out, int nx, int ny, int nz, int kzc, int bx, int y0,
+                                            int bz, int lane)
 {
     if (y0 >= ny) return;   // uniform over the warp
     const int z0 = bz * kzc;
@@ -272,12 +302,14 @@ __device__ __forceinline__ void t1_phi_tile(const T *__restrict__ ga, T *__restr
     for (int q = 0; q < 3; q++)
 #pragma unroll
         for (int a = 0; a < KY; a++) acc[q][a] = acc_r[q][a] = acc_l[q][a] = T(0);
-    const T *q0 = quads(ga, S);
+    T own[KY];   // phi of the last source plane, the one whose outputs the current plane completes
+#pragma unroll
+    for (int a = 0; a < KY; a++) own[a] = T(0);
     T raw[KY + 2][5];
     // source plane 0 of the run
     int zl = wrap_up(z0 - 1 + nz, nz) * plane;   // offset of the next plane to load
 #pragma unroll
-    for (int r = 0; r < KY + 2; r++) t1_load_site(ga, q0, zl + yoff[r], raw[r]);
+    for (int r = 0; r < KY + 2; r++) t1_load_site(phi, q0, zl + yoff[r], raw[r]);
     zl += plane;
     if (zl == plane * nz) zl = 0;
     for (int j0 = 0; j0 < nzc + 2; j0 += 3) {
@@ -293,21 +325,23 @@ __device__ __forceinline__ void t1_phi_tile(const T *__restrict__ ga, T *__restr
                 const int q = (k + 2 + cz(i)) % 3;
                 return cx(i) == 0 ? acc[q][oy] : cx(i) > 0 ? acc_r[q][oy] : acc_l[q][oy];
             };
+            T own_j[KY];
 #pragma unroll
             for (int ry = -1; ry <= KY; ry++) {
                 T (&c5)[5] = raw[ry + 1];
                 const Eq<T> e = make_eq(c5[0], c5[1], c5[2], c5[3], c5[4]);
-                if (more) t1_load_site(ga, q0, zl + yoff[ry + 1], c5);
+                if (ry >= 0 && ry < KY) {
+                    own_j[ry] = c5[0];
+                    T &a = acc[(k + 2) % 3][ry];
+                    a = fmadd(T(-12), moving_sum(e), a);
+                }
+                if (more) t1_load_site(phi, q0, zl + yoff[ry + 1], c5);
                 if constexpr (is_df64<T>::value) {
                     // double-float: the pair form (measured: 7.59 against 6.21
                     // GLUPS at 256^3; in float and double the compiler already
                     // shares c.u between opposite directions, and the pair
                     // form's longer-lived class terms cost occupancy there)
                     const EqPair<T> ep = pair_form(e);
-                    if (ry >= 0 && ry < KY) {
-                        T &a = slot(0, ry);
-                        a = add_px(a, ep.r0);
-                    }
 #pragma unroll
                     for (int i = 1; i < Q; i += 2) {
                         const int op = ry + cy(i), om = ry - cy(i);   // output rows of i and i + 1
@@ -327,11 +361,11 @@ __device__ __forceinline__ void t1_phi_tile(const T *__restrict__ ga, T *__restr
                     }
                 } else {
 #pragma unroll
-                    for (int i = 0; i < Q; i++) {
+                    for (int i = 1; i < Q; i++) {
                         const int oy = ry + cy(i);
                         if (oy < 0 || oy >= KY) continue;
                         T &a = slot(i, oy);
-                        a += geq_eq(i, e);
+                        a += geq36(i, e);
                     }
                 }
             }
@@ -339,7 +373,7 @@ __device__ __forceinline__ void t1_phi_tile(const T *__restrict__ ga, T *__restr
                 zl += plane;
                 if (zl == plane * nz) zl = 0;
             }
-            // output plane j - 2 (slot (k + 1) mod 3) is complete
+            // output plane j - 2 (slot (k + 1) mod 3) is complete: U - 12 t
             const int qd = (k + 1) % 3;
             const int oz = j - 2;
 #pragma unroll
@@ -347,8 +381,10 @@ __device__ __forceinline__ void t1_phi_tile(const T *__restrict__ ga, T *__restr
                 const T from_left = shfl_up1(acc_r[qd][a]);
                 const T from_right = shfl_down1(acc_l[qd][a]);
                 if (out_x && oz >= 0 && y0 + a < ny)
-                    gb[yoff[a + 1] + (z0 + oz) * plane] = add_px(acc[qd][a], add_px(from_left, from_right));
+                    phi_out[yoff[a + 1] + (z0 + oz) * plane] =
+                        fmadd(T(1.0 / 36.0), add_px(acc[qd][a], add_px(from_left, from_right)), own[a]);
                 acc[qd][a] = acc_r[qd][a] = acc_l[qd][a] = T(0);
+                own[a] = own_j[a];
             }
         }
     }

@@ -34,6 +34,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <utility>
 
 #include "d3q19.cuh"
 #include "lb_internal.cuh"
@@ -49,26 +50,40 @@ constexpr int kT1Threads = 256;
 
 template <typename T, bool SH, int NP>
 __global__ void __launch_bounds__(kT1Threads, sizeof(T) == 8 ? 2 : 3)
-k_t1_collide(const T *__restrict__ fa, T *__restrict__ ga /* level a: phi in, (gmh, u) out */, T *__restrict__ fb,
+k_t1_collide(const T *__restrict__ fa, const T *__restrict__ phi, T *__restrict__ quad, T *__restrict__ fb,
              Coll<T> p, int nx, int ny, int nz, long long S)
 {
     pdl_wait_then_release();
     const long long N = (long long)nx * ny * nz;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
-    t1_collide_site<T, SH, NP>(fa, ga, fb, p, nx, ny, nz, S, s);
+    t1_collide_site<T, SH, NP>(fa, phi, quad, fb, p, nx, ny, nz, S, s);
+}
+
+// the same with the multiple-relaxation-time collision or a body force
+template <typename T, bool SH, int NP>
+__global__ void __launch_bounds__(kT1Threads, sizeof(T) == 8 ? 2 : 3)
+k_t1_collide_mrt(const T *__restrict__ fa, const T *__restrict__ phi, T *__restrict__ quad, T *__restrict__ fb,
+                 Coll<T> p, Mrt<T> m, int nx, int ny, int nz, long long S)
+{
+    pdl_wait_then_release();
+    const long long N = (long long)nx * ny * nz;
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= N) return;
+    t1_collide_site<T, SH, NP>(fa, phi, quad, fb, p, nx, ny, nz, S, s, &m);
 }
 
 constexpr int kPhiWarps = 4;      // default warps per block, stacked in y
 constexpr int kPhiMaxWarps = 8;
 
 template <typename T, int KY>
-__global__ void __launch_bounds__(32 * kPhiMaxWarps) k_t1_phi(const T *__restrict__ ga, T *__restrict__ gb, int nx,
-                                                               int ny, int nz, int kzc, long long S)
+__global__ void __launch_bounds__(32 * kPhiMaxWarps) k_t1_phi(const T *__restrict__ phi,
+                                                               const T *__restrict__ quad, T *__restrict__ phi_out,
+                                                               int nx, int ny, int nz, int kzc)
 {
     pdl_wait_then_release();
-    t1_phi_tile<T, KY>(ga, gb, nx, ny, nz, kzc, S, blockIdx.x, (blockIdx.y * blockDim.y + threadIdx.y) * KY,
-                       blockIdx.z, threadIdx.x);
+    t1_phi_tile<T, KY>(phi, quad, phi_out, nx, ny, nz, kzc, blockIdx.x,
+                       (blockIdx.y * blockDim.y + threadIdx.y) * KY, blockIdx.z, threadIdx.x);
 }
 
 // g state of the reduced form as post-streaming FP64 rows [i0, i1):
@@ -198,27 +213,59 @@ int phi_z_run(lb_ctx *c, long long columns, int bps, int *kzc)
     return LB_OK;
 }
 
+// The two passes of the reduced form for context c: the launch shapes of its
+// phi pass (warps per CTA, z run) worked out once.
+template <typename T, bool SH, int NP, int KY>
+struct T1Passes {
+    lb_ctx *c;
+    dim3 pgrid, pblock;
+    int kzc = 0;
+
+    int plan(lb_ctx *ctx, int block_warps)
+    {
+        c = ctx;
+        const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
+        const int warps = block_warps ? block_warps : kPhiWarps;
+        const unsigned gx = (nx + kPhiOut - 1) / kPhiOut, gy = (ny + KY * warps - 1) / (KY * warps);
+        static std::atomic<int> cache[kPhiMaxWarps + 1];
+        int bps = 0;
+        int rc = blocks_per_sm(k_t1_phi<T, KY>, 32 * warps, 0, cache[warps], &bps);
+        if (!rc) rc = phi_z_run(c, (long long)gx * gy, bps, &kzc);
+        pgrid = dim3(gx, gy, (nz + kzc - 1) / (kzc ? kzc : 1));
+        pblock = dim3(32, warps);
+        return rc;
+    }
+    // f of the step into fb, the quads of (mu, u); phi is phi(t)
+    cudaError_t collide(const T *fa, const T *phi, T *quad, T *fb) const
+    {
+        const unsigned grid = grid_of(c->N);
+        const auto p = make_coll<T>(c->p);
+        const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
+        if (uses_mrt(c))
+            return launch_pdl(k_t1_collide_mrt<T, SH, NP>, grid, kT1Threads, c->stream, fa, phi, quad, fb, p,
+                              make_mrt<T>(c), nx, ny, nz, c->S);
+        return launch_pdl(k_t1_collide<T, SH, NP>, grid, kT1Threads, c->stream, fa, phi, quad, fb, p, nx, ny, nz,
+                          c->S);
+    }
+    // phi(t + 1) from phi(t) and the quads
+    cudaError_t next_phi(const T *phi, const T *quad, T *phi_out) const
+    {
+        return launch_pdl(k_t1_phi<T, KY>, pgrid, pblock, c->stream, phi, quad, phi_out, c->p.nx, c->p.ny, c->p.nz,
+                          kzc);
+    }
+};
+
 template <typename T, bool SH, int NP, int KY>
 int run_t1(lb_ctx *c, int nsteps)
 {
-    const auto p = make_coll<T>(c->p);
-    const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
-    const unsigned grid = grid_of(c->N);
-    const int warps = c->block_y ? c->block_y : kPhiWarps;
-    const unsigned gx = (nx + kPhiOut - 1) / kPhiOut, gy = (ny + KY * warps - 1) / (KY * warps);
-    static std::atomic<int> cache[kPhiMaxWarps + 1];
-    int bps = 0, kzc = 0;
-    int rc = blocks_per_sm(k_t1_phi<T, KY>, 32 * warps, 0, cache[warps], &bps);
-    if (!rc) rc = phi_z_run(c, (long long)gx * gy, bps, &kzc);
+    T1Passes<T, SH, NP, KY> pass;
+    int rc = pass.plan(c, c->block_y);
     if (rc) return rc;
-    const dim3 pgrid(gx, gy, (nz + kzc - 1) / kzc), pblock(32, warps);
     for (int t = 0; t < nsteps; t++) {
         const int a = c->buf.cur, b = 1 - a;
-        cudaError_t e = launch_pdl(k_t1_collide<T, SH, NP>, grid, kT1Threads, c->stream, (const T *)c->buf.f[a],
-                                   (T *)c->buf.g[a], (T *)c->buf.f[b], p, nx, ny, nz, c->S);
-        if (e == cudaSuccess)
-            e = launch_pdl(k_t1_phi<T, KY>, pgrid, pblock, c->stream, (const T *)c->buf.g[a], (T *)c->buf.g[b], nx,
-                           ny, nz, kzc, c->S);
+        T *ga = (T *)c->buf.g[a];
+        cudaError_t e = pass.collide((const T *)c->buf.f[a], ga, quads(ga, c->S), (T *)c->buf.f[b]);
+        if (e == cudaSuccess) e = pass.next_phi(ga, quads(ga, c->S), (T *)c->buf.g[b]);
         rc = e != cudaSuccess ? cuda_status(e) : check_launch();
         if (rc) return rc;
         c->buf.cur = b;
@@ -289,6 +336,74 @@ void g_rows_t(lb_ctx *c, int i0, int i1, double *out)
         g_rows<T, SH, 27>(c, i0, i1, out);
     else
         g_rows<T, SH, 7>(c, i0, i1, out);
+}
+
+// FP32-shifted steps of a general (19-value) state with tau_g = 1.  Within
+// one call g's 19 values are only wanted at its end: the first phi is the sum
+// of the stored g, the steps between are the reduced form's two passes on
+// scratch in the g level that the call does not end in, and the last step's
+// collision writes g* = geq in full.  n steps move 20 + 49 (n - 1) + 58 words
+// a site instead of 76 n (the bulk kernel) or 97 n (two passes), and the
+// stored state between calls stays the general one.
+template <int NP, int KY>
+static int run_geq(lb_ctx *c, int nsteps)
+{
+    T1Passes<float, true, NP, KY> pass;
+    int rc = pass.plan(c, 0);
+    if (rc) return rc;
+    int a = c->buf.cur;
+    const int last = (a + nsteps) & 1;
+    float *scratch = (float *)c->buf.g[1 - last];   // g(t) itself where nsteps is odd, until its phi is summed
+    float *phi = (float *)c->phi, *phi_next = scratch, *quad = quads(scratch, c->S);
+    cudaError_t e = launch_phi_pull(c, (const float *)c->buf.g[a], phi);
+    for (int t = 0; t + 1 < nsteps && e == cudaSuccess; t++, a = 1 - a) {
+        e = pass.collide((const float *)c->buf.f[a], phi, quad, (float *)c->buf.f[1 - a]);
+        if (e == cudaSuccess) e = pass.next_phi(phi, quad, phi_next);
+        std::swap(phi, phi_next);
+    }
+    if (e == cudaSuccess)
+        e = launch_collide_geq(c, (const float *)c->buf.f[a], phi, (float *)c->buf.f[last], (float *)c->buf.g[last]);
+    rc = e != cudaSuccess ? cuda_status(e) : check_launch();
+    if (rc) return rc;
+    c->buf.cur = last;
+    return LB_OK;
+}
+
+template <int KY>
+static int run_geq_np(lb_ctx *c, int nsteps)
+{
+    if (c->npts == 19) return run_geq<19, KY>(c, nsteps);
+    if (c->npts == 27) return run_geq<27, KY>(c, nsteps);
+    return run_geq<7, KY>(c, nsteps);
+}
+
+// When the library default takes these steps (microseconds a step over 50
+// steps, against two passes that leave g unread, 78 words a site):
+//   256^3 530 / 770, 200x152x136 140 / 200, 128^3 74 / 103, 80^3 21.1 / 26.8,
+//   72x64x64 14.3 / 14.3, 64^3 13.1 / 13.0, 32^3 7.7 / 4.6 -- below 2^18
+//   sites both passes wait on latency, and the phi pass's walk along z is the
+//   longer chain;
+//   rows of 16 sites 82 / 103, of 12 69 / 79, of 8 56 / 53 (2^20 sites or
+//   so) -- a warp's 30 output columns are mostly idle on short rows.
+// FP64 and double-float steps are bound by arithmetic, of which the reduced
+// form's phi pass has more; they take the two passes.
+constexpr long long kGeqMinSites = (1LL << 18) + 1;
+constexpr int kGeqMinRow = 12;
+// Two y rows a lane in the phi pass from 2^20 sites on (128^3 74.1 against
+// 75.5 us, 256^3 527 / 531, 300^3 838 / 874; 96^3 36.7 / 34.6: one row there,
+// for more warps), one where the lattice has fewer than four rows
+// (1024x1x1024 51 / 43).
+constexpr long long kGeqTwoRowSites = 1LL << 20;
+
+bool auto_uses_geq(const lb_ctx *c)
+{
+    return c->p.precision == LB_FP32_SHIFTED && g_is_equilibrium(c->p) && c->N >= kGeqMinSites &&
+           c->p.nx >= kGeqMinRow;
+}
+
+int launch_step_geq(lb_ctx *c, int nsteps)
+{
+    return c->N >= kGeqTwoRowSites && c->p.ny >= 4 ? run_geq_np<2>(c, nsteps) : run_geq_np<1>(c, nsteps);
 }
 
 int taug1_validate(const lb_params &p, int block_x, int block_y, int z_chunk)
