@@ -135,17 +135,24 @@ int cuda_status(cudaError_t e)
 
 int check_launch() { return cuda_status(cudaGetLastError()); }
 
-void adopt_into_batch(lb_ctx *c, unsigned int *shared_err)
+int state_written(lb_ctx *c)
+{
+    return c->moments ? cuda_status(cudaMemsetAsync(c->moments, 0, sizeof(int), c->stream)) : LB_OK;
+}
+
+void adopt_into_batch(lb_ctx *c, unsigned int *shared_err, int *moments)
 {
     cudaStreamSynchronize(c->stream);
     dev_free(c, c->err_flag, sizeof(unsigned int));
     c->err_flag = shared_err;
+    c->moments = moments;
     c->batch_owned = 1;
 }
 
 void release_from_batch(lb_ctx *c)
 {
     c->err_flag = nullptr;
+    c->moments = nullptr;
     c->batch_owned = 0;
 }
 

@@ -42,7 +42,11 @@ namespace {
 // CTA size limit and CTAs per SM the register budget must allow (measured:
 // 3 x 256 threads FP32 and 2 x 256 FP64 beat the unconstrained allocation
 // by 11 % and 9 %; the FP32 reduced form gains another 6 % at 4 x 256,
-// 64 registers, where the general form loses 3 % to spills)
+// 64 registers, where the general form loses 3 % to spills; general states
+// with every tau_g = 1 run the reduced form's passes and take its bound:
+// 259.7 -> 160 us a step for 64 lattices of sides 16..64 in FP32, 49 words a
+// site instead of 97, and 2340 -> 2223 us in FP64, where only the reading of
+// g and its 19 multiplications go)
 #ifndef LBK_BATCH_MAXT32
 #define LBK_BATCH_MAXT32 256
 #endif
@@ -69,13 +73,17 @@ struct LatDesc {
     const T *f[2];
     const T *g[2];
     T *phi;
+    int *moments;   // kUnreadG: phi and the quads of the last step are at hand (see there)
     Coll<T> p;
 };
 
+// z planes of a reduced-form phi tile, about (a lattice's planes are split
+// evenly; a run reads two planes more than it writes).  64 lattices of sides
+// 16..64, 256 threads: 158.6 us a step at 14, 159.8 at 8, 159.5 at 16, 165 at 24
 #ifndef LBK_BATCH_T1_KZC
-#define LBK_BATCH_T1_KZC 8
+#define LBK_BATCH_T1_KZC 14
 #endif
-constexpr int kBatchT1Kzc = LBK_BATCH_T1_KZC;   // z run of a reduced-form phi tile in the ensemble
+constexpr int kBatchT1Kzc = LBK_BATCH_T1_KZC;
 constexpr int kBatchPhiV = LBK_BATCH_PHI_V;   // phi-pass work items per trip (general form)
 
 struct GridBarrier {
@@ -132,9 +140,122 @@ __device__ bool grid_sync(GridBarrier *bar, unsigned int nblocks, long long time
     return !*s_fail;
 }
 
-template <typename T, bool SH, bool RED>
-__global__ void __launch_bounds__(sizeof(T) == 8 ? kBatchMaxThreads64 : kBatchMaxThreads,
-                                  sizeof(T) == 8 ? LBK_BATCH_MINB64 : (RED ? LBK_BATCH_MINB32_RED : LBK_BATCH_MINB32))
+// What a step of the ensemble does.
+enum BatchStep {
+    kTwoPass = 0,   // the default step: phi pass, collide/stream pass
+    kReduced = 1,   // the tau_g = 1 reduced form (lb_t1.cuh)
+    // General states, every tau_g = 1: the collide pass does not read g and,
+    // in FP32, the steps of a run are the reduced form's passes on scratch in
+    // the g level that the run does not end in; the last collision writes g in
+    // full as well.  The first phi of a run is the sum of the stored g after a
+    // new start (init, set_state), else the phi pass over the last step's phi
+    // (in the lattice's phi buffer) and quads (in the spare g level), which
+    // the last run left there: so k runs give the bits of one run of all their
+    // steps.  Which it is stands in device memory (LatDesc::moments, cleared on
+    // the stream by every call that writes a member's state), so that a
+    // captured run does not fix it.
+    kUnreadG = 2,
+};
+
+// CTAs per SM the register budget of a step allows
+template <typename T>
+constexpr int batch_min_ctas(int step)
+{
+    return sizeof(T) == 8 ? LBK_BATCH_MINB64 : step == kTwoPass ? LBK_BATCH_MINB32 : LBK_BATCH_MINB32_RED;
+}
+
+// The passes over a group's slice of the work lists, by CTA r of the group.
+template <typename T, bool SH>
+struct BatchPasses {
+    const LatDesc<T> *lats;
+    const int2 *work;
+    const int4 *work_t1;
+    Group G;
+    int r;
+
+    // phi of the stored g of level a (of the lattices that take(L) picks).
+    // kBatchPhiV work items per trip, their loads independent, so that the
+    // pass keeps as many loads in flight as its own kernel would at full
+    // occupancy (the collide pass sets the residency)
+    template <typename Take>
+    __device__ __forceinline__ void pull_phi(int a, Take &&take) const
+    {
+        const int wend = G.wo + G.wn;
+        for (int w0 = G.wo + r; w0 < wend; w0 += kBatchPhiV * G.m) {
+#pragma unroll
+            for (int u = 0; u < kBatchPhiV; u++) {
+                const int w = w0 + u * G.m;
+                if (w >= wend) break;
+                const int2 it = work[w];
+                const LatDesc<T> &L = lats[it.x];
+                const long long s = (long long)it.y * blockDim.x + threadIdx.x;
+                if (s < L.N && take(L)) {
+                    const Nbr n((int)s, L.nx, L.ny, L.nz);
+                    L.phi[s] = phi_site(L.g[a], n, L.S);
+                }
+            }
+        }
+    }
+    // the general collision from level a to level 1 - a
+    template <bool GEQ>
+    __device__ __forceinline__ void collide(int a) const
+    {
+        for (int w = G.wo + r; w < G.wo + G.wn; w += G.m) {
+            const int2 it = work[w];
+            const LatDesc<T> &L = lats[it.x];
+            const long long s = (long long)it.y * blockDim.x + threadIdx.x;
+            if (s < L.N) {
+                const Nbr n((int)s, L.nx, L.ny, L.nz);
+                collide_site<T, SH, 7, GEQ>(L.f[a], L.g[a], L.phi, const_cast<T *>(L.f[1 - a]),
+                                            const_cast<T *>(L.g[1 - a]), L.p, n, s, L.S);
+            }
+        }
+    }
+    // the reduced form's collision: f of level a to 1 - a, the quads into level
+    // q; full: g* into level 1 - a too, and phi into the lattice's phi buffer
+    template <typename Phi>
+    __device__ __forceinline__ void t1_collide(int a, int q, bool full, Phi &&phi) const
+    {
+        for (int w = G.wo + r; w < G.wo + G.wn; w += G.m) {
+            const int2 it = work[w];
+            const LatDesc<T> &L = lats[it.x];
+            const long long s = (long long)it.y * blockDim.x + threadIdx.x;
+            if (s < L.N) {
+                const T *ph = phi(L);
+                t1_collide_site<T, SH, 7>(L.f[a], ph, quads(const_cast<T *>(L.g[q]), L.S),
+                                          const_cast<T *>(L.f[1 - a]), L.p, L.nx, L.ny, L.nz, L.S, (int)s, nullptr,
+                                          full ? const_cast<T *>(L.g[1 - a]) : nullptr);
+                if (full && ph != L.phi) L.phi[s] = ph[s];
+            }
+        }
+    }
+    // the reduced form's phi pass with the quads of level q
+    template <typename Take, typename Phi, typename Out>
+    __device__ __forceinline__ void t1_phi(int q, Take &&take, Phi &&phi, Out &&out) const
+    {
+        constexpr int KY = PhiTile<T>::KY;
+        const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int w = G.to + r; w < G.to + G.tn; w += G.m) {
+            const int4 it = work_t1[w];   // (lattice, x block, warp group, z run)
+            const LatDesc<T> &L = lats[it.x];
+            if (!take(L)) continue;
+            t1_phi_tile<T, KY>(phi(L), quads(L.g[q], L.S), out(L), L.nx, L.ny, L.nz, L.kzc, it.y,
+                               (it.z * warps + warp) * KY, it.w, lane);
+        }
+    }
+    // the lattices of this CTA's first work items now have their moments
+    __device__ __forceinline__ void mark_moments() const
+    {
+        if (threadIdx.x != 0) return;
+        for (int w = G.wo + r; w < G.wo + G.wn; w += G.m) {
+            const int2 it = work[w];
+            if (it.y == 0) *lats[it.x].moments = 1;
+        }
+    }
+};
+
+template <typename T, bool SH, int STEP>
+__global__ void __launch_bounds__(sizeof(T) == 8 ? kBatchMaxThreads64 : kBatchMaxThreads, batch_min_ctas<T>(STEP))
     k_batch(const LatDesc<T> *__restrict__ lats, const int2 *__restrict__ work, const int4 *__restrict__ work_t1,
             const Group *__restrict__ groups, const int *__restrict__ cta_group, int nsteps, int parity0,
             GridBarrier *bars, unsigned int *err, long long timeout_ns, int skip_cta)
@@ -144,65 +265,46 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kBatchMaxThreads64 : kBatchMa
     if (gi < 0) return;   // a CTA the plan left without work
     const Group G = groups[gi];
     GridBarrier *bar = bars + gi;
-    const int r = blockIdx.x - G.cta0, wend = G.wo + G.wn;
+    const BatchPasses<T, SH> pass{lats, work, work_t1, G, (int)blockIdx.x - G.cta0};
     if (threadIdx.x == 0) s_fail = 0;
-    if constexpr (RED) {
-        constexpr int KY = PhiTile<T>::KY;
-        const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const int tend = G.to + G.tn;
+    const bool skip = (int)blockIdx.x == skip_cta;   // test hook: this CTA never arrives at its first barrier
+    auto sync = [&] { return !skip && grid_sync(bar, G.m, timeout_ns, err, &s_fail); };
+    using L = const LatDesc<T> &;
+    auto all = [](L) { return true; };
+    if constexpr (STEP == kReduced) {
         for (int t = 0; t < nsteps; t++) {
             const int a = (parity0 + t) & 1;
-            for (int w = G.wo + r; w < wend; w += G.m) {
-                const int2 it = work[w];
-                const LatDesc<T> &L = lats[it.x];
-                const long long s = (long long)it.y * blockDim.x + threadIdx.x;
-                if (s < L.N)
-                    t1_collide_site<T, SH, 7>(L.f[a], L.g[a], quads(const_cast<T *>(L.g[a]), L.S),
-                                              const_cast<T *>(L.f[1 - a]), L.p, L.nx, L.ny, L.nz, L.S, (int)s);
-            }
-            if ((int)blockIdx.x == skip_cta) return;   // test hook: this CTA never arrives
-            if (!grid_sync(bar, G.m, timeout_ns, err, &s_fail)) return;
-            for (int w = G.to + r; w < tend; w += G.m) {
-                const int4 it = work_t1[w];   // (lattice, x block, warp group, z run)
-                const LatDesc<T> &L = lats[it.x];
-                t1_phi_tile<T, KY>(L.g[a], quads(L.g[a], L.S), const_cast<T *>(L.g[1 - a]), L.nx, L.ny, L.nz, L.kzc,
-                                   it.y, (it.z * warps + warp) * KY, it.w, lane);
-            }
-            if (!grid_sync(bar, G.m, timeout_ns, err, &s_fail)) return;
+            pass.t1_collide(a, a, false, [&](L l) { return l.g[a]; });
+            if (!sync()) return;
+            pass.t1_phi(a, all, [&](L l) { return l.g[a]; }, [&](L l) { return const_cast<T *>(l.g[1 - a]); });
+            if (!sync()) return;
         }
+    } else if constexpr (STEP == kUnreadG && sizeof(T) == 4) {
+        const int a0 = parity0 & 1, spare = 1 - ((parity0 + nsteps) & 1);
+        auto kept = [](L l) { return *l.moments != 0; };
+        pass.pull_phi(a0, [&](L l) { return !kept(l); });
+        pass.t1_phi(1 - a0, kept, [](L l) { return l.phi; }, [&](L l) { return const_cast<T *>(l.g[spare]); });
+        if (!sync()) return;
+        for (int t = 0; t < nsteps; t++) {
+            // phi(t) stands in the phi buffer and in row 0 of the spare level
+            // by turns, from where the first pass put it
+            auto in_spare = [&](L l) { return ((t + kept(l)) & 1) != 0; };
+            auto phi = [&](L l) -> const T * { return in_spare(l) ? l.g[spare] : l.phi; };
+            auto next = [&](L l) { return in_spare(l) ? l.phi : const_cast<T *>(l.g[spare]); };
+            pass.t1_collide((parity0 + t) & 1, spare, t + 1 == nsteps, phi);
+            if (!sync()) return;
+            if (t + 1 == nsteps) break;
+            pass.t1_phi(spare, all, phi, next);
+            if (!sync()) return;
+        }
+        pass.mark_moments();
     } else {
         for (int t = 0; t < nsteps; t++) {
             const int a = (parity0 + t) & 1;
-            // kBatchPhiV work items per trip, their loads independent, so that
-            // the phi pass keeps as many loads in flight as its own kernel
-            // would at full occupancy (the collide pass sets the residency)
-            for (int w0 = G.wo + r; w0 < wend; w0 += kBatchPhiV * G.m) {
-#pragma unroll
-                for (int u = 0; u < kBatchPhiV; u++) {
-                    const int w = w0 + u * G.m;
-                    if (w >= wend) break;
-                    const int2 it = work[w];
-                    const LatDesc<T> &L = lats[it.x];
-                    const long long s = (long long)it.y * blockDim.x + threadIdx.x;
-                    if (s < L.N) {
-                        const Nbr n((int)s, L.nx, L.ny, L.nz);
-                        L.phi[s] = phi_site(L.g[a], n, L.S);
-                    }
-                }
-            }
-            if ((int)blockIdx.x == skip_cta) return;   // test hook: this CTA never arrives
-            if (!grid_sync(bar, G.m, timeout_ns, err, &s_fail)) return;
-            for (int w = G.wo + r; w < wend; w += G.m) {
-                const int2 it = work[w];
-                const LatDesc<T> &L = lats[it.x];
-                const long long s = (long long)it.y * blockDim.x + threadIdx.x;
-                if (s < L.N) {
-                    const Nbr n((int)s, L.nx, L.ny, L.nz);
-                    collide_site<T, SH>(L.f[a], L.g[a], L.phi, const_cast<T *>(L.f[1 - a]),
-                                        const_cast<T *>(L.g[1 - a]), L.p, n, s, L.S);
-                }
-            }
-            if (!grid_sync(bar, G.m, timeout_ns, err, &s_fail)) return;
+            pass.pull_phi(a, all);
+            if (!sync()) return;
+            pass.template collide<STEP == kUnreadG>(a);
+            if (!sync()) return;
         }
     }
 }
@@ -301,6 +403,8 @@ struct lb_batch {
     int ngroups = 0;
     int bins = 0;                              // lb_batch_set_plan: 0 = a group per lattice, k = k groups
     int reduced = 0;                           // all lattices in the tau_g = 1 reduced form
+    int unread_g = 0;                          // every tau_g = 1
+    int *d_moments = nullptr;                  // [n] LatDesc::moments
     lbk::GridBarrier *d_bar = nullptr;         // one per group
     int skip_cta = -1;                         // test hook: first CTA of the largest group
     unsigned int *d_err = nullptr;
@@ -321,6 +425,18 @@ void drop_graphs(lb_batch *b)
     b->graphs.clear();
 }
 
+// what a step of the ensemble does now, and its kernel
+int batch_step(const lb_batch *b) { return b->reduced ? lbk::kReduced : b->unread_g ? lbk::kUnreadG : lbk::kTwoPass; }
+
+template <typename T, bool SH>
+auto batch_kernel(const lb_batch *b)
+{
+    const int step = batch_step(b);
+    return step == lbk::kReduced   ? lbk::k_batch<T, SH, lbk::kReduced>
+           : step == lbk::kUnreadG ? lbk::k_batch<T, SH, lbk::kUnreadG>
+                                   : lbk::k_batch<T, SH, lbk::kTwoPass>;
+}
+
 template <typename T, bool SH>
 int batch_tables(lb_batch *b)
 {
@@ -329,8 +445,8 @@ int batch_tables(lb_batch *b)
     int rc = lbk::cuda_status(cudaGetDevice(&dev));
     if (!rc) rc = lbk::cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (!rc)
-        rc = lbk::cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, b->reduced ? lbk::k_batch<T, SH, true> : lbk::k_batch<T, SH, false>, b->threads, 0));
+        rc = lbk::cuda_status(
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<T, SH>(b), b->threads, 0));
     if (rc) return rc;
     if (per_sm < 1) return LB_ERR_INVALID;
     const int use = b->ctas_per_sm > 0 && b->ctas_per_sm < per_sm ? b->ctas_per_sm : per_sm;
@@ -353,10 +469,12 @@ int batch_tables(lb_batch *b)
             L[k].g[l] = (const T *)c->buf.g[l];
         }
         L[k].phi = (T *)c->phi;
+        L[k].moments = c->moments;
         L[k].p = lbk::make_coll<T>(c->p);
-        L[k].kzc = c->p.nz < lbk::kBatchT1Kzc ? c->p.nz : lbk::kBatchT1Kzc;
+        const int runs = std::max(1, (c->p.nz + lbk::kBatchT1Kzc / 2) / lbk::kBatchT1Kzc);
+        L[k].kzc = (c->p.nz + runs - 1) / runs;   // runs of about equal length
         nb[k] = (c->N + b->threads - 1) / b->threads;
-        if (b->reduced) {
+        if (b->reduced || (b->unread_g && sizeof(T) == 4)) {
             const int rows = (b->threads / 32) * lbk::PhiTile<T>::KY;   // y rows of one warp group
             const int gx = (c->p.nx + lbk::kPhiOut - 1) / lbk::kPhiOut, gy = (c->p.ny + rows - 1) / rows;
             const int gz = (c->p.nz + L[k].kzc - 1) / L[k].kzc;
@@ -454,7 +572,7 @@ int capture(lb_batch *b, int nsteps, int parity, cudaGraphExec_t *out)
     cfg.numAttrs = 1;
     const lbk::LatDesc<T> *lats = (const lbk::LatDesc<T> *)b->d_lats;
     const cudaError_t le =
-        cudaLaunchKernelEx(&cfg, b->reduced ? lbk::k_batch<T, SH, true> : lbk::k_batch<T, SH, false>, lats,
+        cudaLaunchKernelEx(&cfg, batch_kernel<T, SH>(b), lats,
                            (const int2 *)b->d_work, (const int4 *)b->d_work_t1, (const lbk::Group *)b->d_groups,
                            (const int *)b->d_cta_group, nsteps, parity, b->d_bar, b->d_err, b->timeout_ns,
                            b->debug_skip ? b->skip_cta : -1);
@@ -504,6 +622,7 @@ void lb_batch_destroy(lb_batch *b)
     cudaFree(b->d_cta_group);
     cudaFree(b->d_bar);
     cudaFree(b->d_err);
+    cudaFree(b->d_moments);
     if (b->ev_in) cudaEventDestroy(b->ev_in);
     if (b->ev_out) cudaEventDestroy(b->ev_out);
     if (b->stream) cudaStreamDestroy(b->stream);
@@ -535,8 +654,12 @@ int lb_batch_create(int n, const lb_params *p, void *cuda_stream, lb_batch **out
     if (!rc) rc = lbk::cuda_status(cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming));
     if (!rc) rc = lbk::cuda_status(cudaMalloc(&b->d_err, sizeof(unsigned int)));
     if (!rc) rc = lbk::cuda_status(cudaMemset(b->d_err, 0, sizeof(unsigned int)));
+    b->unread_g = 1;
+    for (int k = 0; k < n; k++) b->unread_g = b->unread_g && lbk::g_is_equilibrium(p[k]);
+    if (!rc) rc = lbk::cuda_status(cudaMalloc(&b->d_moments, n * sizeof(int)));
+    if (!rc) rc = lbk::cuda_status(cudaMemset(b->d_moments, 0, n * sizeof(int)));
     if (!rc)
-        for (lb_ctx *c : b->ctx) lbk::adopt_into_batch(c, b->d_err);
+        for (int k = 0; k < n; k++) lbk::adopt_into_batch(b->ctx[k], b->d_err, b->d_moments + k);
     if (!rc) rc = tables(b);
     if (rc) {
         lb_batch_destroy(b);
@@ -655,6 +778,7 @@ int lb_batch_set_form(lb_batch *b, int reduced)
     int rc = batch_sync(b);
     for (lb_ctx *c : b->ctx) {
         if (!rc) rc = lbk::taug1_convert(c, reduced);
+        if (!rc) rc = lbk::state_written(c);
         if (!rc) c->reduced = reduced;
     }
     if (!rc) rc = lbk::cuda_status(cudaStreamSynchronize(b->user_stream));

@@ -48,6 +48,7 @@ struct lb_ctx {
     double *adj = nullptr;        // [6N] adjoint scratch (lazy): phi_bar, d_bar (3), lap_bar, phi
     double *adj_part = nullptr;   // per-CTA partial dJ/dkappa
     int batch_owned = 0;  // member of an lb_batch: stepped and freed by it
+    int *moments = nullptr;   // member of an lb_batch: device flag, the last step's phi and quads are at hand
     int reduced = 0;      // tau_g = 1 form: g kept as phi and (gmh, u), see lb_taug1.cu
     int m_valid = 0;      // reduced form: the previous step's (gmh, u) are present
     int npts = 7;         // points of the phi stencil: 7, 19 or 27 (lb_set_stencil)
@@ -102,7 +103,10 @@ constexpr int kReduceBlocks = 304;   // 2 x 152 SMs, one wave; fixed so sums are
 constexpr int kReduceThreads = 256;
 
 // ensemble membership (lb_api.cu): the member shares the batch's error flag
-void adopt_into_batch(lb_ctx *c, unsigned int *shared_err);
+void adopt_into_batch(lb_ctx *c, unsigned int *shared_err, int *moments);
+// the stored state was written by other than a step: what an ensemble's last
+// run left beside a member's state no longer belongs to it (on the stream)
+int state_written(lb_ctx *c);
 void release_from_batch(lb_ctx *c);
 
 // status helpers (lb_api.cu)

@@ -253,7 +253,8 @@ int launch_init(lb_ctx *c, const double *phi0_d, const double *u0_d)
 {
     return by_precision(c, [&](auto P) {
         init_t<typename decltype(P)::T, decltype(P)::SH>(c, phi0_d, u0_d);
-        return check_launch();
+        const int rc = check_launch();
+        return rc ? rc : state_written(c);
     });
 }
 
@@ -295,7 +296,8 @@ static int set_rows(lb_ctx *c, int which, int i0, int i1, const double *in)
     return by_precision(c, [&](auto P) {
         using T = typename decltype(P)::T;
         k_set_state<T><<<grid, 256, 0, c->stream>>>((T *)a, in, i0, i1, shift, c->p.nx, c->p.ny, c->p.nz, c->S);
-        return check_launch();
+        const int rc = check_launch();
+        return rc ? rc : state_written(c);
     });
 }
 

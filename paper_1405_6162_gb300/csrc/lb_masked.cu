@@ -266,7 +266,8 @@ int launch_masked_rows(lb_ctx *c, long long total, const int *scratch, int which
         else
             k_masked_get<T><<<grid, kGatherThreads, 0, c->stream>>>((const T *)a, idx, tot, i0, i1, shift, io, nx,
                                                                     ny, nz, c->S);
-        return check_launch();
+        const int rc = check_launch();
+        return rc || !to_device_state ? rc : state_written(c);
     });
 }
 

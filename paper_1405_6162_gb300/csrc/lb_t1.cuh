@@ -218,11 +218,12 @@ __device__ __forceinline__ Eq<T> load_eq(const T *__restrict__ g, long long S, l
 
 // The collide pass at site s: pull f, the NP-point stencil of phi(t), the
 // general collision's f part (collide_mrt's with m); write f* and the quad
-// (gmh, u) of (s, t).
+// (gmh, u) of (s, t) and, with gb, the 19 values g* = geq as well.
 template <typename T, bool SH, int NP>
 __device__ __forceinline__ void t1_collide_site(const T *__restrict__ fa, const T *__restrict__ phi,
                                                 T *__restrict__ quad, T *__restrict__ fb, const Coll<T> &p, int nx,
-                                                int ny, int nz, long long S, int s, const Mrt<T> *m = nullptr)
+                                                int ny, int nz, long long S, int s, const Mrt<T> *m = nullptr,
+                                                T *__restrict__ gb = nullptr)
 {
     const Nbr n(s, nx, ny, nz);
     T f[Q];
@@ -240,6 +241,12 @@ __device__ __forceinline__ void t1_collide_site(const T *__restrict__ fa, const 
 #pragma unroll
     for (int i = 0; i < Q; i++) fb[(size_t)i * S + s] = f[i];
     Quad<T>::store(quad, s, gmh_of(ph, mu, p.gamma), ux, uy, uz);
+    if (gb) {
+        T g[Q];
+        collide_g<T, true>(p, g, ph, ux, uy, uz, mu);
+#pragma unroll
+        for (int i = 0; i < Q; i++) gb[(size_t)i * S + s] = g[i];
+    }
 }
 
 constexpr int kPhiOut = 30;    // output columns per warp

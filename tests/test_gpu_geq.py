@@ -123,3 +123,47 @@ def test_replayed_graph_steps_a_new_start():
             lat.step(4)
             assert all(torch.equal(a, b) for a, b in zip(lat.moments(device=True), g))
         stream.synchronize()
+
+
+def test_ensemble_runs_follow_the_members_state():
+    """An ensemble's run starts from the members' state, whichever call wrote
+    it last: after run(3), a member set to another state (whole or masked) or
+    started anew advances that state, and one left alone gives the bits of an
+    undivided run."""
+    from paper_1405_6162_gb300 import Batch
+    specs = [dict(P0, nx=20, ny=17, nz=16, tau=0.8), dict(P0, nx=33, ny=18, nz=21), dict(P0, nx=16, ny=16, nz=40),
+             dict(P0, nx=17, ny=31, nz=9, tau=0.6)]
+    dims = [(d["nx"], d["ny"], d["nz"]) for d in specs]
+    phi = [L.spinodal_phi0(*d, seed=860 + k, amp=0.3) for k, d in enumerate(dims)]
+    s1 = [to_abi(x) for x in nonequilibrium_state(dims[1], P0, seed=870)]
+    mask = (L.uniform(871, int(np.prod(dims[3])), 0, 1) < 0.4).astype(np.uint8)
+
+    def start(b):
+        for k in range(4):
+            b[k].init(phi[k])
+
+    with Batch(specs, precision="fp32_shifted") as b, Batch(specs, precision="fp32_shifted") as c:
+        start(b)
+        start(c)
+        b.run(3)
+        c.run(3)
+        b[1].set_state(*s1)
+        b[2].init(phi[2])
+        f3, g3 = b[3].get_state_masked(mask)
+        b[3].set_state_masked(mask, 1.01 * f3, 0.9 * g3)
+        whole3 = b[3].get_state()
+        b.run(2)
+        got = [b[k].get_state() for k in range(4)]
+        # the same from states that no run has touched
+        c[0].init(phi[0])
+        c[1].set_state(*s1)
+        c[2].init(phi[2])
+        c[3].set_state(*whole3)
+        c.run(2)
+        want = [c[k].get_state() for k in range(4)]
+        c[0].init(phi[0])
+        c.run(5)
+        want[0] = c[0].get_state()
+    for k in range(4):
+        for a, w in zip(got[k], want[k]):
+            assert np.array_equal(a, w), k
