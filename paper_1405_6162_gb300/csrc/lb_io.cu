@@ -6,6 +6,8 @@
 // per-site quantity here gathers A_i from x - c_i.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "d3q19.cuh"
 #include "df64.cuh"
 #include "lb_internal.cuh"
@@ -173,37 +175,135 @@ __device__ __forceinline__ double widen(double x) { return x; }
 // hi + lo of a double-float is exact in FP64 (|lo| <= ulp(hi) / 2)
 __device__ __forceinline__ double widen(df64 x) { return widen(x.hi) + widen(x.lo); }
 
+// s + e = a + b exactly (Knuth), s into a; e is returned
+__device__ __forceinline__ float two_sum_into(float &a, float b)
+{
+    float s, e;
+    dfops::two_sum(a, b, s, e);
+    a = s;
+    return e;
+}
+
+// The sum of a thread's values of one row.  double: a double.  float and
+// double-float: a float sum, the sum of its (exact) rounding errors with the
+// low parts, and that sum's rounding errors -- about 70 bits in all, more than
+// a double keeps.
+template <typename T>
+struct RowSum {
+    T s;
+    __device__ __forceinline__ void zero() { s = 0.0; }
+    __device__ __forceinline__ void add(T v) { s += v; }
+    __device__ __forceinline__ bool finite() const { return true; }   // inf and NaN are the double sum's own
+    __device__ __forceinline__ double total() const { return s; }
+};
+struct FloatRowSum {
+    float s, e, d;
+    __device__ __forceinline__ void zero() { s = e = d = 0.0f; }
+    __device__ __forceinline__ void add(float v) { d += two_sum_into(e, two_sum_into(s, v)); }
+    __device__ __forceinline__ void add(df64 v)
+    {
+        const float t = two_sum_into(s, v.hi);
+        const float t1 = two_sum_into(e, t), t2 = two_sum_into(e, v.lo);
+        d += t1 + t2;
+    }
+    __device__ __forceinline__ bool finite() const { return fabsf(s) <= 3.402823466e38f; }
+    __device__ __forceinline__ double total() const { return widen(s) + (widen(e) + widen(d)); }
+};
+template <>
+struct RowSum<float> : FloatRowSum {};
+template <>
+struct RowSum<df64> : FloatRowSum {};
+
+// V consecutive values of a row in one load
+template <typename T, int V>
+struct Packed {
+    T v[V];
+};
+template <>
+struct __align__(8) Packed<float, 2> {
+    float v[2];
+};
+
+// the values of V sites from s on added to the row sums (V = 2: s even, so
+// that the loads are aligned, rows starting at multiples of 64 elements)
+template <typename T, int G_ROWS, int GS, int V>
+__device__ __forceinline__ void add_sites(const T *__restrict__ fa, const T *__restrict__ ga, long long S, long long s,
+                                          RowSum<T> (&fs)[Q], RowSum<T> (&gs)[GS])
+{
+    using P = Packed<T, V>;
+    P f[Q], g[G_ROWS];
+#pragma unroll
+    for (int i = 0; i < Q; i++) f[i] = *reinterpret_cast<const P *>(fa + (size_t)i * S + s);
+#pragma unroll
+    for (int i = 0; i < G_ROWS; i++) g[i] = *reinterpret_cast<const P *>(ga + (size_t)i * S + s);
+#pragma unroll
+    for (int i = 0; i < Q; i++)
+#pragma unroll
+        for (int v = 0; v < V; v++) fs[i].add(f[i].v[v]);
+#pragma unroll
+    for (int i = 0; i < G_ROWS; i++)
+#pragma unroll
+        for (int v = 0; v < V; v++) gs[i % GS].add(g[i].v[v]);
+}
+
 // Per-block partial totals.  A thread sums each of the 19 f rows over its
-// sites in FP64 (sum_x A_i(x)), and the g rows (G rows: 19, or 1 in the
-// tau_g = 1 reduced form, whose row 0 holds phi) into four FP64 partial
-// sums, as only their total, sum phi, is wanted; R and j = sum_i c_i F_i are
-// formed from the 19 row totals once per thread.  That is 38 FP64 additions
-// a site (plus one per float of a double-float) against the 68 that forming
-// every site's moments takes.  The order of every addition is fixed by the
-// launch shape, so the totals are bitwise reproducible.
+// sites (sum_x A_i(x)), and the g rows (G rows: 19, or 1 in the tau_g = 1
+// reduced form, whose row 0 holds phi) into a few partial sums, as only their
+// total, sum phi, is wanted; R and j = sum_i c_i F_i are formed from the 19
+// row totals once per thread.  GB300 adds about 2 doubles a clock per SM, and
+// one FP64 addition per value bounded this kernel (256^3: 1.26 ms in FP32, two
+// additions a value and 2.47 ms in double-float), so float values are summed
+// on the FP32 units (RowSum) and reach FP64 once per thread: 0.44 and 0.77 ms,
+// the copy rate over the stored words being 0.38 and 0.75 ms.  FP64 storage
+// keeps its 38 additions a site (1.29 ms).  A thread whose float sums leave the
+// float range sums its sites again in FP64.  The order of every addition is
+// fixed by the launch shape, so the totals are bitwise reproducible.
 template <typename T, int G_ROWS>
 __global__ void __launch_bounds__(kReduceThreads, 2) k_reduce_partial(const T *__restrict__ fa,
                                                                       const T *__restrict__ ga, long long N,
                                                                       long long S, double *__restrict__ partial)
 {
-    double F[Q], G[4] = {0.0, 0.0, 0.0, 0.0};
+    constexpr int GS = G_ROWS < 4 ? G_ROWS : 4;   // partial sums of g
+    constexpr int V = std::is_same<T, float>::value ? 2 : 1;
+    const long long stride = (long long)gridDim.x * blockDim.x, first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    RowSum<T> fs[Q], gs[GS];
 #pragma unroll
-    for (int i = 0; i < Q; i++) F[i] = 0.0;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < N;
-         s += (long long)gridDim.x * blockDim.x) {
-        T f[Q], g[G_ROWS];
+    for (int i = 0; i < Q; i++) fs[i].zero();
 #pragma unroll
-        for (int i = 0; i < Q; i++) f[i] = fa[(size_t)i * S + s];
+    for (int i = 0; i < GS; i++) gs[i].zero();
+#pragma unroll 1
+    for (long long s = V * first; s + V <= N; s += V * stride) add_sites<T, G_ROWS, GS, V>(fa, ga, S, s, fs, gs);
+    if (V > 1 && first < N % V) add_sites<T, G_ROWS, GS, 1>(fa, ga, S, N - N % V + first, fs, gs);
+    bool ok = true;
 #pragma unroll
-        for (int i = 0; i < G_ROWS; i++) g[i] = ga[(size_t)i * S + s];
+    for (int i = 0; i < Q; i++) ok = ok && fs[i].finite();
 #pragma unroll
-        for (int i = 0; i < Q; i++) F[i] += widen(f[i]);
+    for (int i = 0; i < GS; i++) ok = ok && gs[i].finite();
+    double F[Q], G[GS];
 #pragma unroll
-        for (int i = 0; i < G_ROWS; i++) G[i & 3] += widen(g[i]);
+    for (int i = 0; i < Q; i++) F[i] = fs[i].total();
+#pragma unroll
+    for (int i = 0; i < GS; i++) G[i] = gs[i].total();
+    if (!ok) {
+#pragma unroll
+        for (int i = 0; i < Q; i++) F[i] = 0.0;
+#pragma unroll
+        for (int i = 0; i < GS; i++) G[i] = 0.0;
+        auto add_double = [&](long long s) {
+#pragma unroll
+            for (int i = 0; i < Q; i++) F[i] += widen(fa[(size_t)i * S + s]);
+#pragma unroll
+            for (int i = 0; i < G_ROWS; i++) G[i % GS] += widen(ga[(size_t)i * S + s]);
+        };
+#pragma unroll 1
+        for (long long s = V * first; s + V <= N; s += V * stride)
+#pragma unroll 1
+            for (int v = 0; v < V; v++) add_double(s + v);
+        if (V > 1 && first < N % V) add_double(N - N % V + first);
     }
     double acc[5];
     density_moments(F, acc[0], acc[1], acc[2], acc[3]);
-    acc[4] = (G[0] + G[1]) + (G[2] + G[3]);
+    acc[4] = GS == 4 ? (G[0] + G[GS > 1 ? 1 : 0]) + (G[GS > 2 ? 2 : 0] + G[GS - 1]) : G[0];
     block_sum<5>(acc, partial + 5 * blockIdx.x);
 }
 
