@@ -10,130 +10,126 @@
 //                 f_bar(x, t), the direct part of g_bar, and the adjoints of
 //                 phi, grad phi and lap phi at x; per-CTA partial dJ/dkappa
 //   k_adj_stencil phi_bar(x) = local part + transposed 7-point stencils;
-//                 g_bar_i(x, t) += phi_bar(x)
+//                 g_bar_i(x, t) += phi_bar(x); the sum of the partial dJ/dkappa
+// (launched with programmatic dependent launch, lb_pdl.cuh).
 // The equilibrium VJP sums each opposite pair (i+, i-) once: its even part
 // feeds rho and the stress, its odd part the momentum.
 #include <cuda_runtime.h>
 
 #include "d3q19.cuh"
 #include "lb_internal.cuh"
+#include "lb_pdl.cuh"
 #include "lb_site.cuh"
 
 namespace lbk {
 
 namespace {
 
+// Model parameters, and the relaxation rate folded into the factors of the
+// weight sums below (formed on the host): R = w/36, O = w/12 (3 w/36),
+// T = w/8 (9/2 w/36), W = w/24 (3/2 w/36), w the rate of f or of g.
 struct AdjP {
-    double omega, omega_g, rho0, gamma, A, B, kappa;
+    double rho0, gamma, A, B, B3, kappa, kappa2;   // B3 = 3 B, kappa2 = 2 kappa
+    double keep_f, keep_g;                         // 1 - w: the part of f, g that a step keeps
+    double fR, fO, fT, fW;
+    double gR, gO, gT, gW;
 };
 
-// c of the + member of pair k (k = 0..8: faces x, y, z; edges 7, 9, 11, 13, 15, 17)
-__device__ __forceinline__ int pc(int k, int a)
-{
-    const int ip = k < 3 ? 2 * k + 1 : 7 + 2 * (k - 3);
-    return a == 0 ? cx(ip) : (a == 1 ? cy(ip) : cz(ip));
-}
-__device__ __forceinline__ int pplus(int k) { return k < 3 ? 2 * k + 1 : 7 + 2 * (k - 3); }
-__device__ __forceinline__ double pw(int k) { return k < 3 ? 1.0 / 18.0 : 1.0 / 36.0; }
+// Sums of a distribution's adjoint F over the velocities, weighted in units
+// of 1/36 (36 w_i = 12, 2, 1): W = sum 36 w F, O = sum 36 w c F and
+// T = sum 36 w c c F.  Opposite pairs enter by their sum and difference and
+// every sum names the velocities that reach it: written as loops over c_i the
+// products with its zeros stay (0 * x is not 0 for every x), and they were
+// most of the FP64 instructions of this kernel.
+struct WeightSums {
+    double W, Ox, Oy, Oz, Txx, Tyy, Tzz, Txy, Txz, Tyz;
+};
 
-// Adjoint of (rho, j, phi, d, lap, kappa) -> (feq, geq) at one site, given
-// the weights Fe_i on feq_i and Ge_i on geq_i.  INIT: rho and j are inputs
-// (no adjoint flows into them).
-template <bool INIT>
-__device__ __forceinline__ void equilibrium_vjp(const AdjP &p, double rho, const double (&j)[3], double phi,
-                                                const double (&d)[3], double lap, const double (&Fe)[Q],
-                                                const double (&Ge)[Q], double &rho_b, double (&j_b)[3],
-                                                double &phi_b, double (&d_b)[3], double &lap_b, double &kap_b)
+__device__ __forceinline__ WeightSums weight_sums(const double (&F)[Q])
 {
-    const double u[3] = {j[0] / rho, j[1] / rho, j[2] / rho};
-    // pair sums: even parts (s) and odd parts (o)
-    double Wf = Fe[0] / 3.0, Wg = Ge[0] / 3.0;
-    double Tf[3][3] = {{0}}, Tg[3][3] = {{0}}, Of[3] = {0, 0, 0}, Og[3] = {0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-        const int ip = pplus(k);
-        const double w = pw(k);
-        const double sf = w * (Fe[ip] + Fe[ip + 1]), of = w * (Fe[ip] - Fe[ip + 1]);
-        const double sg = w * (Ge[ip] + Ge[ip + 1]), og = w * (Ge[ip] - Ge[ip + 1]);
-        Wf += sf;
-        Wg += sg;
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const int ca = pc(k, a);
-            Of[a] += of * ca;
-            Og[a] += og * ca;
-#pragma unroll
-            for (int b = 0; b < 3; b++) {
-                Tf[a][b] += sf * ca * pc(k, b);
-                Tg[a][b] += sg * ca * pc(k, b);
-            }
-        }
+    WeightSums m;
+    {
+        const double sx = F[1] + F[2], sy = F[3] + F[4], sz = F[5] + F[6];
+        const double xy = F[7] + F[8], xy_ = F[9] + F[10];   // along (1, 1, 0) and (1, -1, 0)
+        const double xz = F[11] + F[12], xz_ = F[13] + F[14];
+        const double yz = F[15] + F[16], yz_ = F[17] + F[18];
+        const double exy = xy + xy_, exz = xz + xz_, eyz = yz + yz_;
+        const double ex = exy + exz;
+        m.Txx = 2.0 * sx + ex;
+        m.Tyy = 2.0 * sy + (exy + eyz);
+        m.Tzz = 2.0 * sz + (exz + eyz);
+        m.Txy = xy - xy_;
+        m.Txz = xz - xz_;
+        m.Tyz = yz - yz_;
+        m.W = 12.0 * F[0] + (2.0 * ((sx + sy) + sz) + (ex + eyz));
     }
-    // feq_i = w_i [rho + 3 c.j + 9/2 c S c - 3/2 tr S]
-    double Sb[3][3], Gb[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            Sb[a][b] = 4.5 * Tf[a][b] - (a == b ? 1.5 * Wf : 0.0);
-            Gb[a][b] = 4.5 * Tg[a][b] - (a == b ? 1.5 * Wg : 0.0);
-        }
-    rho_b += Wf;
-    double u_b[3];
+    {
+        const double xy = F[7] - F[8], xy_ = F[9] - F[10];
+        const double xz = F[11] - F[12], xz_ = F[13] - F[14];
+        const double yz = F[15] - F[16], yz_ = F[17] - F[18];
+        m.Ox = 2.0 * (F[1] - F[2]) + ((xy + xy_) + (xz + xz_));
+        m.Oy = 2.0 * (F[3] - F[4]) + ((xy - xy_) + (yz + yz_));
+        m.Oz = 2.0 * (F[5] - F[6]) + ((xz - xz_) + (yz - yz_));
+    }
+    return m;
+}
+
+// Adjoint of (rho, j, phi, d, lap, kappa) -> (w feq, w geq) at one site from
+// the weight sums of the adjoints of f (mf) and g (mg), w in p's factors.
+// INIT: rho and j are inputs (no adjoint flows into them).
+template <bool INIT>
+__device__ __forceinline__ void equilibrium_vjp(const AdjP &p, double rinv, const double (&u)[3], double phi,
+                                                const double (&d)[3], double lap, const WeightSums &mf,
+                                                const WeightSums &mg, double &rho_b, double (&j_b)[3], double &phi_b,
+                                                double (&d_b)[3], double &lap_b, double &kap_b)
+{
+    const double third = 1.0 / 3.0;
+    // feq_i = w_i [rho + 3 c.j + 9/2 c S c - 3/2 tr S],  S = pb I + kappa d d + j j / rho
+    const double fw = p.fW * mf.W;
+    const double S[3][3] = {{p.fT * mf.Txx - fw, p.fT * mf.Txy, p.fT * mf.Txz},
+                            {p.fT * mf.Txy, p.fT * mf.Tyy - fw, p.fT * mf.Tyz},
+                            {p.fT * mf.Txz, p.fT * mf.Tyz, p.fT * mf.Tzz - fw}};
+    const double pb_b = S[0][0] + S[1][1] + S[2][2];
+    const double kpb = p.kappa * pb_b;
+    double dSd = 0.0, uSu = 0.0, Su[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        j_b[a] += 3.0 * Of[a];
-        u_b[a] = 3.0 * phi * Og[a];
+        const double Sd = S[a][0] * d[0] + S[a][1] * d[1] + S[a][2] * d[2];
+        dSd = a ? dSd + d[a] * Sd : d[a] * Sd;
+        d_b[a] = p.kappa2 * Sd - kpb * d[a];
+        if (!INIT) {
+            Su[a] = S[a][0] * u[0] + S[a][1] * u[1] + S[a][2] * u[2];
+            uSu = a ? uSu + u[a] * Su[a] : u[a] * Su[a];
+        }
     }
     // geq_i = w_i [phi + 3 phi c.u + 9/2 c G c - 3/2 tr G],  G = (Gamma mu - phi/3) I + phi u u
-    phi_b += Wg + 3.0 * (u[0] * Og[0] + u[1] * Og[1] + u[2] * Og[2]);
-    const double trG = Gb[0][0] + Gb[1][1] + Gb[2][2];
+    const double gw = p.gW * mg.W;
+    const double G[3][3] = {{p.gT * mg.Txx - gw, p.gT * mg.Txy, p.gT * mg.Txz},
+                            {p.gT * mg.Txy, p.gT * mg.Tyy - gw, p.gT * mg.Tyz},
+                            {p.gT * mg.Txz, p.gT * mg.Tyz, p.gT * mg.Tzz - gw}};
+    const double trG = G[0][0] + G[1][1] + G[2][2];
     const double mu_b = p.gamma * trG;
-    double uGu = 0.0;
+    const double o[3] = {p.gO * mg.Ox, p.gO * mg.Oy, p.gO * mg.Oz};
+    double uo = 0.0, uGu = 0.0, Gu[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        double Gu = 0.0;
-#pragma unroll
-        for (int b = 0; b < 3; b++) Gu += Gb[a][b] * u[b];
-        uGu += u[a] * Gu;
-        u_b[a] += 2.0 * phi * Gu;
+        Gu[a] = G[a][0] * u[0] + G[a][1] * u[1] + G[a][2] * u[2];
+        uo = a ? uo + u[a] * o[a] : u[a] * o[a];
+        uGu = a ? uGu + u[a] * Gu[a] : u[a] * Gu[a];
     }
-    phi_b += uGu - trG / 3.0;
-    // S = pb I + kappa d d + j j / rho
-    const double pb_b = Sb[0][0] + Sb[1][1] + Sb[2][2];
-    double dSd = 0.0, jSj = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        double Sd = 0.0, Sj = 0.0;
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            Sd += Sb[a][b] * d[b];
-            Sj += Sb[a][b] * j[b];
-        }
-        d_b[a] += 2.0 * p.kappa * Sd;
-        dSd += d[a] * Sd;
-        jSj += j[a] * Sj;
-        if (!INIT) j_b[a] += 2.0 * Sj / rho;
-    }
-    kap_b += dSd;
-    if (!INIT) rho_b -= jSj / (rho * rho);
-    // pb = A/2 phi^2 + 3B/4 phi^4 - kappa phi lap - kappa/2 |d|^2
+    // pb = A/2 phi^2 + 3B/4 phi^4 - kappa phi lap - kappa/2 |d|^2;  mu = A phi + B phi^3 - kappa lap
+    const double dmu = p.A + p.B3 * (phi * phi);
+    phi_b = (p.gR * mg.W + uo) + (uGu - third * trG) + pb_b * (phi * dmu - p.kappa * lap) + mu_b * dmu;
+    lap_b = -(kpb * phi + p.kappa * mu_b);
     const double dd = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    phi_b += pb_b * (p.A * phi + 3.0 * p.B * phi * phi * phi - p.kappa * lap);
-    lap_b -= p.kappa * phi * pb_b;
-#pragma unroll
-    for (int a = 0; a < 3; a++) d_b[a] -= p.kappa * d[a] * pb_b;
-    kap_b -= pb_b * (phi * lap + 0.5 * dd);
-    // mu = A phi + B phi^3 - kappa lap
-    phi_b += mu_b * (p.A + 3.0 * p.B * phi * phi);
-    lap_b -= p.kappa * mu_b;
-    kap_b -= lap * mu_b;
-    // u = j / rho
+    kap_b = dSd - pb_b * (phi * lap + 0.5 * dd) - lap * mu_b;
     if (!INIT) {
-        const double uj = u_b[0] * j[0] + u_b[1] * j[1] + u_b[2] * j[2];
+        // u = j / rho: with v = o + 2 G u, dJ/du = phi v (of g), dJ/dj = dJ/du / rho + 2 S u + direct
+        const double pr = phi * rinv;
+        const double fo[3] = {p.fO * mf.Ox, p.fO * mf.Oy, p.fO * mf.Oz};
 #pragma unroll
-        for (int a = 0; a < 3; a++) j_b[a] += u_b[a] / rho;
-        rho_b -= uj / (rho * rho);
+        for (int a = 0; a < 3; a++) j_b[a] = (fo[a] + 2.0 * Su[a]) + pr * (o[a] + 2.0 * Gu[a]);
+        rho_b = (p.fR * mf.W - uSu) - pr * (uo + 2.0 * uGu);
     }
 }
 
@@ -157,6 +153,7 @@ constexpr int kAdjThreads = 256;
 __global__ void __launch_bounds__(kAdjThreads) k_phi_local(const double *__restrict__ g, double *__restrict__ phi,
                                                            long long N)
 {
+    pdl_wait_then_release();
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
     double v[Q];
@@ -166,17 +163,28 @@ __global__ void __launch_bounds__(kAdjThreads) k_phi_local(const double *__restr
 }
 
 // Collision VJP per site.  INIT: the initial state (f_bar of the equilibria
-// in af_in/ag_in, no streaming, phi given by phi0, j = rho0 u0).
-template <bool INIT>
-__global__ void __launch_bounds__(kAdjThreads) k_adj_collide(const double *__restrict__ f, const double *__restrict__ g,
-                                                             const double *__restrict__ phi,
-                                                             const double *__restrict__ u0,
-                                                             const double *__restrict__ af_in,
-                                                             const double *__restrict__ ag_in,
-                                                             double *__restrict__ af_out, double *__restrict__ ag_out,
-                                                             double *__restrict__ aux, double *__restrict__ kpart,
-                                                             AdjP p, int nx, int ny, int nz)
+// in af_in/ag_in, no streaming, phi given by phi0, j = rho0 u0).  KEEP_F,
+// KEEP_G: tau, tau_g != 1, a step keeps a part of f, g; without it the values
+// of f_bar (g_bar) are not held for the output, and g_bar is phi_bar alone,
+// which k_adj_stencil writes.
+//
+// Bound by the FP64 pipe (2 lanes a clock per SM), so written for few FP64
+// instructions: weight_sums, one reciprocal of rho instead of eleven
+// divisions, rates folded into the factors.  64^3, tau = tau_g = 1: a reverse
+// step 0.40 -> 0.17 ms, the gradient through 200 steps 138.3 -> 92.6 ms.
+// Two CTAs an SM: the FP64 pipe is full with 16 warps.
+template <bool INIT, bool KEEP_F, bool KEEP_G>
+__global__ void __launch_bounds__(kAdjThreads, 2) k_adj_collide(const double *__restrict__ f,
+                                                                const double *__restrict__ phi,
+                                                                const double *__restrict__ u0,
+                                                                const double *__restrict__ af_in,
+                                                                const double *__restrict__ ag_in,
+                                                                double *__restrict__ af_out,
+                                                                double *__restrict__ ag_out, double *__restrict__ aux,
+                                                                double *__restrict__ kpart, AdjP p, int nx, int ny,
+                                                                int nz)
 {
+    pdl_wait_then_release();
     __shared__ double sh[kAdjThreads / 32];
     const long long N = (long long)nx * ny * nz;
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -184,39 +192,52 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_collide(const double *__res
     if (s < N) {
         const Nbr n((int)s, nx, ny, nz);
         const double ph = phi[s];
-        double dx, dy, dz, lap;
-        stencil(phi, n, ph, dx, dy, dz, lap);
-        double rho, j[3];
+        double d[3], lap;
+        stencil(phi, n, ph, d[0], d[1], d[2], lap);
+        double rinv = 0.0, u[3];
         if (INIT) {
-            rho = p.rho0;
-            j[0] = u0 ? p.rho0 * u0[s] : 0.0;
-            j[1] = u0 ? p.rho0 * u0[N + s] : 0.0;
-            j[2] = u0 ? p.rho0 * u0[2 * N + s] : 0.0;
+#pragma unroll
+            for (int a = 0; a < 3; a++) u[a] = u0 ? u0[a * N + s] : 0.0;
         } else {
-            double fv[Q];
+            double fv[Q], rho, j[3];
 #pragma unroll
             for (int i = 0; i < Q; i++) fv[i] = f[(size_t)i * N + s];
             density_moments(fv, rho, j[0], j[1], j[2]);
+            rinv = 1.0 / rho;
+#pragma unroll
+            for (int a = 0; a < 3; a++) u[a] = j[a] * rinv;
         }
         // adjoint after the streaming transpose: value of (x + c_i) at t+1
-        double Fe[Q], Ge[Q], fsb[Q], gsb[Q];
+        double fsb[Q], gsb[Q];
 #pragma unroll
-        for (int i = 0; i < Q; i++) {
-            const size_t o = (size_t)i * N + (INIT ? s : n.at(cx(i), cy(i), cz(i)));
-            fsb[i] = af_in[o];
-            gsb[i] = ag_in[o];
-            Fe[i] = (INIT ? 1.0 : p.omega) * fsb[i];
-            Ge[i] = (INIT ? 1.0 : p.omega_g) * gsb[i];
+        for (int i = 0; i < Q; i++) fsb[i] = af_in[(size_t)i * N + (INIT ? s : n.at(cx(i), cy(i), cz(i)))];
+        const WeightSums mf = weight_sums(fsb);
+#pragma unroll
+        for (int i = 0; i < Q; i++) gsb[i] = ag_in[(size_t)i * N + (INIT ? s : n.at(cx(i), cy(i), cz(i)))];
+        const WeightSums mg = weight_sums(gsb);
+        if (KEEP_G) {
+#pragma unroll
+            for (int i = 0; i < Q; i++) ag_out[(size_t)i * N + s] = p.keep_g * gsb[i];
         }
-        const double d[3] = {dx, dy, dz};
-        double rho_b = 0.0, j_b[3] = {0.0, 0.0, 0.0}, phi_b = 0.0, d_b[3] = {0.0, 0.0, 0.0}, lap_b = 0.0;
-        equilibrium_vjp<INIT>(p, rho, j, ph, d, lap, Fe, Ge, rho_b, j_b, phi_b, d_b, lap_b, kap_b);
+        double rho_b, j_b[3], phi_b, d_b[3], lap_b;
+        equilibrium_vjp<INIT>(p, rinv, u, ph, d, lap, mf, mg, rho_b, j_b, phi_b, d_b, lap_b, kap_b);
         if (!INIT) {
-#pragma unroll
-            for (int i = 0; i < Q; i++) {
-                af_out[(size_t)i * N + s] = (1.0 - p.omega) * fsb[i] + rho_b + (j_b[0] * cx(i) + j_b[1] * cy(i) + j_b[2] * cz(i));
-                ag_out[(size_t)i * N + s] = (1.0 - p.omega_g) * gsb[i];
-            }
+            // f_bar_i = keep f_bar_i(x + c_i) + rho_b + c_i.j_b
+            auto put = [&](int i, double v) { af_out[(size_t)i * N + s] = KEEP_F ? p.keep_f * fsb[i] + v : v; };
+            auto put_pair = [&](int i, double cj) {
+                put(i, rho_b + cj);
+                put(i + 1, rho_b - cj);
+            };
+            put(0, rho_b);
+            put_pair(1, j_b[0]);
+            put_pair(3, j_b[1]);
+            put_pair(5, j_b[2]);
+            put_pair(7, j_b[0] + j_b[1]);
+            put_pair(9, j_b[0] - j_b[1]);
+            put_pair(11, j_b[0] + j_b[2]);
+            put_pair(13, j_b[0] - j_b[2]);
+            put_pair(15, j_b[1] + j_b[2]);
+            put_pair(17, j_b[1] - j_b[2]);
         }
         aux[s] = phi_b;
         aux[N + s] = d_b[0];
@@ -228,12 +249,23 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_collide(const double *__res
     if (threadIdx.x == 0) kpart[blockIdx.x] = tot;
 }
 
-// phi_bar = local part + transposed stencils; g_bar_i += phi_bar (or, for the
-// initialisation, phi0_bar = phi_bar)
-template <bool INIT>
+// phi_bar = local part + transposed stencils; g_bar_i += phi_bar (KEEP_G) or,
+// where nothing of g is kept, g_bar_i = phi_bar; for the initialisation
+// phi0_bar = phi_bar.  The first CTA adds the per-CTA partials of dJ/dkappa
+// (fixed order) to *dkappa.
+template <bool INIT, bool KEEP_G>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_stencil(const double *__restrict__ aux, double *__restrict__ out,
-                                                             int nx, int ny, int nz)
+                                                             const double *__restrict__ kpart,
+                                                             double *__restrict__ dkappa, int nx, int ny, int nz)
 {
+    pdl_wait_then_release();
+    if (blockIdx.x == 0) {
+        __shared__ double sh[kAdjThreads / 32];
+        double v = 0.0;
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) v += kpart[b];
+        const double tot = block_sum_d(v, sh);
+        if (threadIdx.x == 0) *dkappa += tot;
+    }
     const long long N = (long long)nx * ny * nz;
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
@@ -247,7 +279,10 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_stencil(const double *__res
         out[s] = pb;
     } else {
 #pragma unroll
-        for (int i = 0; i < Q; i++) out[(size_t)i * N + s] += pb;
+        for (int i = 0; i < Q; i++) {
+            const size_t o = (size_t)i * N + s;
+            out[o] = KEEP_G ? out[o] + pb : pb;
+        }
     }
 }
 
@@ -267,27 +302,44 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_seed(const double *__restri
     }
 }
 
-// dkappa += sum of the per-CTA partials (one CTA, fixed order)
-__global__ void k_adj_kappa(const double *__restrict__ kpart, int nb, double *__restrict__ dkappa)
-{
-    __shared__ double sh[kAdjThreads / 32];
-    double v = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) v += kpart[b];
-    const double tot = block_sum_d(v, sh);
-    if (threadIdx.x == 0) *dkappa += tot;
-}
-
-AdjP adj_params(const lb_params &q)
+// rates w, w_g: 1 for the equilibria of the initialisation
+AdjP adj_params(const lb_params &q, double w, double wg)
 {
     AdjP p;
-    p.omega = 1.0 / q.tau;
-    p.omega_g = 1.0 / q.tau_g;
     p.rho0 = q.rho0;
     p.gamma = q.gamma;
     p.A = q.A;
     p.B = q.B;
+    p.B3 = 3.0 * q.B;
     p.kappa = q.kappa;
+    p.kappa2 = 2.0 * q.kappa;
+    p.keep_f = 1.0 - w;
+    p.keep_g = 1.0 - wg;
+    p.fR = w / 36.0;
+    p.fO = w / 12.0;
+    p.fT = w / 8.0;
+    p.fW = w / 24.0;
+    p.gR = wg / 36.0;
+    p.gO = wg / 12.0;
+    p.gT = wg / 8.0;
+    p.gW = wg / 24.0;
     return p;
+}
+
+// the collision's and the stencils' kernels of a reverse step
+template <bool KEEP_F, bool KEEP_G>
+cudaError_t reverse_step(lb_ctx *c, const double *f, const double *phi, const double *af_in, const double *ag_in,
+                         double *af_out, double *ag_out, double *dkappa, double *aux, double *kpart)
+{
+    const int nb = adjoint_blocks(c->N);
+    const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
+    const AdjP p = adj_params(c->p, 1.0 / c->p.tau, 1.0 / c->p.tau_g);
+    cudaError_t e = launch_pdl(k_adj_collide<false, KEEP_F, KEEP_G>, nb, kAdjThreads, c->stream, f, phi,
+                               (const double *)nullptr, af_in, ag_in, af_out, ag_out, aux, kpart, p, nx, ny, nz);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_adj_stencil<false, KEEP_G>, nb, kAdjThreads, c->stream, (const double *)aux, ag_out,
+                       (const double *)kpart, dkappa, nx, ny, nz);
+    return e;
 }
 
 }  // namespace
@@ -297,15 +349,14 @@ int adjoint_blocks(long long N) { return (int)((N + kAdjThreads - 1) / kAdjThrea
 int launch_adjoint_step(lb_ctx *c, const double *f, const double *g, const double *af_in, const double *ag_in,
                         double *af_out, double *ag_out, double *dkappa, double *aux, double *kpart)
 {
-    const int nb = adjoint_blocks(c->N);
-    const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     double *phi = aux + 5 * c->N;
-    k_phi_local<<<nb, kAdjThreads, 0, c->stream>>>(g, phi, c->N);
-    k_adj_collide<false><<<nb, kAdjThreads, 0, c->stream>>>(f, g, phi, nullptr, af_in, ag_in, af_out, ag_out, aux,
-                                                            kpart, adj_params(c->p), nx, ny, nz);
-    k_adj_stencil<false><<<nb, kAdjThreads, 0, c->stream>>>(aux, ag_out, nx, ny, nz);
-    k_adj_kappa<<<1, kAdjThreads, 0, c->stream>>>(kpart, nb, dkappa);
-    return check_launch();
+    cudaError_t e = launch_pdl(k_phi_local, adjoint_blocks(c->N), kAdjThreads, c->stream, g, phi, (long long)c->N);
+    if (e == cudaSuccess) {
+        const auto step = c->p.tau == 1.0 ? (c->p.tau_g == 1.0 ? reverse_step<false, false> : reverse_step<false, true>)
+                                          : (c->p.tau_g == 1.0 ? reverse_step<true, false> : reverse_step<true, true>);
+        e = step(c, f, phi, af_in, ag_in, af_out, ag_out, dkappa, aux, kpart);
+    }
+    return e != cudaSuccess ? cuda_status(e) : check_launch();
 }
 
 int launch_adjoint_seed(lb_ctx *c, const double *phi_bar, double *af, double *ag)
@@ -319,11 +370,13 @@ int launch_adjoint_init(lb_ctx *c, const double *phi0, const double *u0, const d
 {
     const int nb = adjoint_blocks(c->N);
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
-    k_adj_collide<true><<<nb, kAdjThreads, 0, c->stream>>>(nullptr, nullptr, phi0, u0, af0, ag0, nullptr, nullptr,
-                                                           aux, kpart, adj_params(c->p), nx, ny, nz);
-    k_adj_stencil<true><<<nb, kAdjThreads, 0, c->stream>>>(aux, phi0_bar, nx, ny, nz);
-    k_adj_kappa<<<1, kAdjThreads, 0, c->stream>>>(kpart, nb, dkappa);
-    return check_launch();
+    double *none = nullptr;
+    cudaError_t e = launch_pdl(k_adj_collide<true, false, false>, nb, kAdjThreads, c->stream, (const double *)none, phi0,
+                               u0, af0, ag0, none, none, aux, kpart, adj_params(c->p, 1.0, 1.0), nx, ny, nz);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_adj_stencil<true, false>, nb, kAdjThreads, c->stream, (const double *)aux, phi0_bar,
+                       (const double *)kpart, dkappa, nx, ny, nz);
+    return e != cudaSuccess ? cuda_status(e) : check_launch();
 }
 
 }  // namespace lbk

@@ -68,6 +68,32 @@ def test_init_reverse_matches_oracle():
     assert abs(dk.item() - dk_o) <= 1e-12 * abs(dk_o)
 
 
+# tau = 1 and tau_g = 1 leave parts of the reverse step out; ragged lattices,
+# periodic wraps onto the own site, the last CTA partly filled
+@pytest.mark.parametrize("dims", [(1, 1, 1), (5, 3, 1), (17, 8, 9)])
+@pytest.mark.parametrize("tau,tau_g", [(1.0, 1.0), (1.0, 0.9), (0.8, 1.0)])
+def test_reverse_step_at_unit_relaxation_times_matches_oracle(dims, tau, tau_g):
+    import torch
+    from paper_1405_6162_gb300 import Lattice
+    from paper_1405_6162_gb300 import _lib as LL
+    n = dims[0] * dims[1] * dims[2]
+    p = dict(P0, tau=tau, tau_g=tau_g, kappa=0.05)
+    f, g = nonequilibrium_state(dims, p, seed=230, amp=0.6)
+    af = L.uniform(231, 19 * n, -1, 1).reshape(19, n)
+    ag = L.uniform(232, 19 * n, -1, 1).reshape(19, n)
+    af_o, ag_o, dk_o = oracle.step_adjoint(dims, p, f, g, af, ag)
+    with Lattice.from_params(dims, p, precision="fp64") as lat:
+        tf, tg, taf, tag = (_cuda(to_abi(x)) for x in (f, g, af, ag))
+        oaf, oag = torch.full_like(taf, 7.0), torch.full_like(tag, 7.0)
+        dk = torch.full((1,), 3.0, dtype=torch.float64, device="cuda")   # added to
+        LL.check(LL.lib().lb_adjoint_step(lat.handle, tf.data_ptr(), tg.data_ptr(), taf.data_ptr(), tag.data_ptr(),
+                                          oaf.data_ptr(), oag.data_ptr(), dk.data_ptr()), "adjoint")
+        torch.cuda.synchronize()
+    assert rel(to_oracle(oaf.cpu().numpy().reshape(19, n)), af_o) <= 1e-12
+    assert rel(to_oracle(oag.cpu().numpy().reshape(19, n)), ag_o) <= 1e-12
+    assert abs(dk.item() - 3.0 - dk_o) <= 1e-12 * max(abs(dk_o), 3.0)
+
+
 @pytest.mark.parametrize("segment", [1, 5, 20])
 def test_trajectory_gradient_matches_oracle_16cubed(segment):
     """16^3, T = 20: the checkpointed GPU gradient equals the oracle's
