@@ -11,6 +11,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #ifndef LBK_ST_CS
 #define LBK_ST_CS 0   // 1: stores of post-collision values with the streaming (.cs) hint
 #endif
@@ -97,6 +99,8 @@ struct Coll {
     T rho0;                // shift of the FP32 form
     T gamma, A, B, kappa;
     T hA, qB;              // A/2, 3B/4 (the bulk pressure's coefficients)
+    T kappa4, kappa8;      // kappa/4, kappa/8 (gradients given twice, D2)
+    T gamma45;             // 9/2 gamma
     T cf, f0, f1, f2, f1h, f2h, f1t, f2t;   // 1-omega; omega*w_k; omega*w_k*9/2; omega*w_k*3
     T cg, g0, g1, g2, g1h, g2h, g1t, g2t;   // the same with omega_g
 };
@@ -193,7 +197,11 @@ __device__ __forceinline__ T sum19(const T (&g)[Q])
 // (also returns u and mu):
 // f*_i = (1 - omega) f_i + omega feq_i with omega feq_i expanded per weight
 // class (rest, face, edge) and per opposite pair, sharing every partial sum.
-template <typename T, bool SH>
+// FEQ (tau = 1, so 1 - omega = 0): f* is the equilibrium and f enters through
+// its moments alone.  D2: dx, dy, dz are twice the derivatives, the factor
+// 1/4 of their products in kappa (FP64 issues 2 lanes a clock per SM, and the
+// halvings are instructions like any other there).
+template <typename T, bool SH, bool FEQ = false, bool D2 = false>
 __device__ __forceinline__ void collide_f(const Coll<T>& p, T (&f)[Q], T phi, T dx, T dy, T dz, T lap,
                                           T& ux, T& uy, T& uz, T& mu)
 {
@@ -205,26 +213,43 @@ __device__ __forceinline__ void collide_f(const Coll<T>& p, T (&f)[Q], T phi, T 
     uy = jy * rinv;
     uz = jz * rinv;
     const T phi2 = phi * phi;
-    mu = phi * (p.A + p.B * phi2) - p.kappa * lap;
-    const T pb = phi2 * (p.hA + p.qB * phi2) - p.kappa * (phi * lap + half(dx * dx + dy * dy + dz * dz));
+    T pb;
+    if constexpr (D2) {
+        const T kl = p.kappa * lap;
+        mu = phi * (p.A + p.B * phi2) - kl;
+        pb = phi2 * (p.hA + p.qB * phi2) - (phi * kl + p.kappa8 * (dx * dx + dy * dy + dz * dz));
+    } else {
+        mu = phi * (p.A + p.B * phi2) - p.kappa * lap;
+        pb = phi2 * (p.hA + p.qB * phi2) - p.kappa * (phi * lap + half(dx * dx + dy * dy + dz * dz));
+    }
+    const T kd = D2 ? p.kappa4 : p.kappa;
     // S = P + rho u u
-    const T Sxx = pb + p.kappa * dx * dx + jx * ux;
-    const T Syy = pb + p.kappa * dy * dy + jy * uy;
-    const T Szz = pb + p.kappa * dz * dz + jz * uz;
-    const T Sxy = p.kappa * dx * dy + jx * uy;
-    const T Sxz = p.kappa * dx * dz + jx * uz;
-    const T Syz = p.kappa * dy * dz + jy * uz;
+    const T Sxx = pb + kd * dx * dx + jx * ux;
+    const T Syy = pb + kd * dy * dy + jy * uy;
+    const T Szz = pb + kd * dz * dz + jz * uz;
+    const T Sxy = kd * dx * dy + jx * uy;
+    const T Sxz = kd * dx * dz + jx * uz;
+    const T Syz = kd * dy * dz + jy * uz;
 
     // ---- f: omega feq_i = omega w_i (R - 9/2 t3) + 9/2 omega w_i c_i c_i : S + 3 omega w_i c_i . j,
     // t3 = tr S / 3, so 9/2 t3 = 3/2 tr S (3/2 exact in binary)
     const T cf = p.cf;
     const T b = R - T(1.5) * (Sxx + Syy + Szz);
-    f[0] = fmadd(cf, f[0], p.f0 * b);
+    if constexpr (FEQ)
+        f[0] = p.f0 * b;
+    else
+        f[0] = fmadd(cf, f[0], p.f0 * b);
+    auto relax = [&](T &fp, T &fm, T s, T a) {
+        if constexpr (FEQ)
+            equilibrium_pair(fp, fm, s, a);
+        else
+            relax_pair(cf, fp, fm, s, a);
+    };
     const T B1 = p.f1 * b, B2 = p.f2 * b;
 #define LBK_FACE(IP, IM, SAA, JA)                                  \
     {                                                              \
         const T s_ = fmadd(p.f1h, SAA, B1), a_ = p.f1t * JA;       \
-        relax_pair(cf, f[IP], f[IM], s_, a_);                      \
+        relax(f[IP], f[IM], s_, a_);                               \
     }
     LBK_FACE(1, 2, Sxx, jx)
     LBK_FACE(3, 4, Syy, jy)
@@ -236,8 +261,8 @@ __device__ __forceinline__ void collide_f(const Coll<T>& p, T (&f)[Q], T phi, T 
         const T e_ = fmadd(p.f2h, SAA + SBB, B2), o_ = p.f1h * SAB;  \
         const T sp = e_ + o_, sm = e_ - o_;                          \
         const T ap = p.f2t * (JA + JB), am = p.f2t * (JA - JB);      \
-        relax_pair(cf, f[IP], f[IM], sp, ap);                        \
-        relax_pair(cf, f[KP], f[KM], sm, am);                        \
+        relax(f[IP], f[IM], sp, ap);                                 \
+        relax(f[KP], f[KM], sm, am);                                 \
     }
     LBK_EDGES(7, 8, 9, 10, Sxx, Syy, Sxy, jx, jy)
     LBK_EDGES(11, 12, 13, 14, Sxx, Szz, Sxz, jx, jz)
@@ -264,6 +289,8 @@ __device__ __forceinline__ void collide_g(const Coll<T>& p, T (&g)[Q], T phi, T 
     T gm;
     if constexpr (GEQ && sizeof(T) == sizeof(float))
         gm = (T(4.5) * p.gamma) * mu - T(1.5) * phi;
+    else if constexpr (GEQ && std::is_same<T, double>::value)
+        gm = p.gamma45 * mu - T(1.5) * phi;   // one instruction less
     else
         gm = T(4.5) * (p.gamma * mu - phi * T(1.0 / 3.0));
     const T bg = phi - T(1.5) * (px * ux + py * uy + pz * uz);   // phi - 9/2 phi u^2 / 3
@@ -293,12 +320,25 @@ __device__ __forceinline__ void collide_g(const Coll<T>& p, T (&g)[Q], T phi, T 
         const T s_ = fmadd(p.g2h, pc_ * cu_, G2), a_ = p.g2t * pc_; \
         relax(g[IP], g[IM], s_, a_);                                \
     }
-    LBK_GEDGE(7, 8, px + py, ux + uy)
-    LBK_GEDGE(9, 10, px - py, ux - uy)
-    LBK_GEDGE(11, 12, px + pz, ux + uz)
-    LBK_GEDGE(13, 14, px - pz, ux - uz)
-    LBK_GEDGE(15, 16, py + pz, uy + uz)
-    LBK_GEDGE(17, 18, py - pz, uy - uz)
+    if constexpr (GEQ && std::is_same<T, double>::value) {
+        // FP64, bound by its instructions: phi (u_a +- u_b)^2 from its three
+        // products, 11 instructions for two pairs instead of 12
+        auto edges = [&](int ip, int kp, T paa, T pbb, T pab, T pa, T pb) {
+            const T e = fmadd(p.g2h, paa + pbb, G2), o = p.g1h * pab;   // 2 g2h = g1h
+            relax(g[ip], g[ip + 1], e + o, p.g2t * (pa + pb));
+            relax(g[kp], g[kp + 1], e - o, p.g2t * (pa - pb));
+        };
+        edges(7, 9, px * ux, py * uy, px * uy, px, py);
+        edges(11, 13, px * ux, pz * uz, px * uz, px, pz);
+        edges(15, 17, py * uy, pz * uz, py * uz, py, pz);
+    } else {
+        LBK_GEDGE(7, 8, px + py, ux + uy)
+        LBK_GEDGE(9, 10, px - py, ux - uy)
+        LBK_GEDGE(11, 12, px + pz, ux + uz)
+        LBK_GEDGE(13, 14, px - pz, ux - uz)
+        LBK_GEDGE(15, 16, py + pz, uy + uz)
+        LBK_GEDGE(17, 18, py - pz, uy - uz)
+    }
 #undef LBK_GEDGE
     if constexpr (sizeof(T) == 4) {
         // In float the folded weights do not sum to omega_g (1/3 + 6/18 +
@@ -314,12 +354,12 @@ __device__ __forceinline__ void collide_g(const Coll<T>& p, T (&g)[Q], T phi, T 
 }
 
 // In-place BGK collision of f (collide_f) and of g at one site.
-template <typename T, bool SH>
+template <typename T, bool SH, bool D2 = false>
 __device__ __forceinline__ void collide(const Coll<T>& p, T (&f)[Q], T (&g)[Q],
                                         T phi, T dx, T dy, T dz, T lap)
 {
     T ux, uy, uz, mu;
-    collide_f<T, SH>(p, f, phi, dx, dy, dz, lap, ux, uy, uz, mu);
+    collide_f<T, SH, false, D2>(p, f, phi, dx, dy, dz, lap, ux, uy, uz, mu);
     collide_g<T>(p, g, phi, ux, uy, uz, mu);
 }
 
@@ -344,13 +384,14 @@ struct Mrt {
 //   R' = w_gh R,  J' = w_gh rho u + (2 - w_gh)/2 F,
 //   S' = w_gh S + X - (1 - w_gh) N,
 // which is BGK when the three rates are equal and F = 0.
-template <typename T, bool SH>
+template <typename T, bool SH, bool D2 = false>
 __device__ __forceinline__ void collide_mrt_f(const Coll<T>& p, const Mrt<T>& m, T (&f)[Q], T phi, T dx, T dy,
                                               T dz, T lap, T& ux, T& uy, T& uz, T& mu)
 {
     T R, jx, jy, jz;
     density_moments(f, R, jx, jy, jz);
     const T third = T(1.0 / 3.0), h = T(4.5);
+    if constexpr (D2) dx = half(dx), dy = half(dy), dz = half(dz);
     const T rho = SH ? p.rho0 + R : R;
     const T rinv = T(1) / rho;
     const T Jx = jx + m.hFx, Jy = jy + m.hFy, Jz = jz + m.hFz;   // rho u
@@ -430,12 +471,12 @@ __device__ __forceinline__ void collide_mrt_f(const Coll<T>& p, const Mrt<T>& m,
 }
 
 // collide_mrt_f, then the collision of g with the force-corrected velocity
-template <typename T, bool SH>
+template <typename T, bool SH, bool D2 = false>
 __device__ __forceinline__ void collide_mrt(const Coll<T>& p, const Mrt<T>& m, T (&f)[Q], T (&g)[Q],
                                             T phi, T dx, T dy, T dz, T lap)
 {
     T ux, uy, uz, mu;
-    collide_mrt_f<T, SH>(p, m, f, phi, dx, dy, dz, lap, ux, uy, uz, mu);
+    collide_mrt_f<T, SH, D2>(p, m, f, phi, dx, dy, dz, lap, ux, uy, uz, mu);
     collide_g<T>(p, g, phi, ux, uy, uz, mu);
 }
 

@@ -11,6 +11,8 @@ namespace lbk {
 // (1 - omega_g = 0 in every arithmetic type), so the passes that would only
 // multiply g by that zero need not read it
 inline bool g_is_equilibrium(const lb_params &p) { return p.tau_g == 1.0; }
+// tau = 1: likewise the BGK collision of f
+inline bool f_is_equilibrium(const lb_params &p) { return p.tau == 1.0; }
 
 // Parameters of the step in the arithmetic type T (constants formed in
 // double, rounded once).
@@ -28,6 +30,9 @@ inline Coll<T> make_coll(const lb_params &p)
     c.kappa = T(p.kappa);
     c.hA = T(0.5 * p.A);
     c.qB = T(0.75 * p.B);
+    c.kappa4 = T(0.25 * p.kappa);
+    c.kappa8 = T(0.125 * p.kappa);
+    c.gamma45 = T(4.5 * p.gamma);
     c.cf = T(1.0 - om);
     c.f0 = T(om / 3.0);  c.f1 = T(om / 18.0);  c.f2 = T(om / 36.0);
     c.f1h = T(om / 4.0); c.f2h = T(om / 8.0);

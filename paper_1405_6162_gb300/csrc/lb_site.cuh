@@ -35,8 +35,9 @@ struct Nbr {
 // neighbourhoods, d_a phi = 3 sum_c W_c c_a phi(x + c) and
 // lap phi = 6 sum_c W_c (phi(x + c) - phi(x)), with W the D3Q19 weights
 // (1/18 faces, 1/36 edges) or the D3Q27 ones (2/27, 1/54, 1/216 corners).
-// Loads T, computes in R.
-template <int NP, typename R, typename T>
+// Loads T, computes in R.  D2: twice the gradient, as the 7-point differences
+// give it.
+template <int NP, typename R, bool D2 = false, typename T>
 __device__ __forceinline__ void stencil_np(const T *__restrict__ phi, const Nbr &n, R ph,
                                            R &dx, R &dy, R &dz, R &lap)
 {
@@ -45,9 +46,9 @@ __device__ __forceinline__ void stencil_np(const T *__restrict__ phi, const Nbr 
         const R xp = R(phi[n.at(1, 0, 0)]), xm = R(phi[n.at(-1, 0, 0)]);
         const R yp = R(phi[n.at(0, 1, 0)]), ym = R(phi[n.at(0, -1, 0)]);
         const R zp = R(phi[n.at(0, 0, 1)]), zm = R(phi[n.at(0, 0, -1)]);
-        dx = half(xp - xm);
-        dy = half(yp - ym);
-        dz = half(zp - zm);
+        dx = D2 ? xp - xm : half(xp - xm);
+        dy = D2 ? yp - ym : half(yp - ym);
+        dz = D2 ? zp - zm : half(zp - zm);
         lap = ((xp + xm) + (yp + ym)) + (zp + zm) - R(6) * ph;
     } else {
         // per weight class k (1 faces, 2 edges, 3 corners): sum of phi and the
@@ -83,6 +84,13 @@ __device__ __forceinline__ void stencil_np(const T *__restrict__ phi, const Nbr 
     }
 }
 
+// the FP64 step takes the 7-point gradient doubled (collide_f)
+template <typename T, int NP>
+constexpr bool doubled_gradient()
+{
+    return NP == 7 && std::is_same<T, double>::value;
+}
+
 // the 7-point stencil in the storage type
 template <typename T>
 __device__ __forceinline__ void stencil(const T *__restrict__ phi, const Nbr &n, T ph,
@@ -103,34 +111,37 @@ __device__ __forceinline__ T phi_site(const T *__restrict__ ga, const Nbr &n, lo
 
 // Pull f and g to site s, collide with the NP-point phi stencil, write the
 // post-collision values at s.  GEQ (tau_g = 1): g is not read, its result
-// depends on it through phi alone.  With m the collision of f is collide_mrt.
-template <typename T, bool SH, int NP = 7, bool GEQ = false>
+// depends on it through phi alone; FEQ (with GEQ): tau = 1.  With m the
+// collision of f is collide_mrt.
+template <typename T, bool SH, int NP = 7, bool GEQ = false, bool FEQ = false>
 __device__ __forceinline__ void collide_site(const T *__restrict__ fa, const T *__restrict__ ga,
                                              const T *__restrict__ phi, T *__restrict__ fb,
                                              T *__restrict__ gb, const Coll<T> &p, const Nbr &n, long long s,
                                              long long S, const Mrt<T> *m = nullptr)
 {
+    static_assert(GEQ || !FEQ, "tau = 1 is told apart where tau_g = 1");
+    constexpr bool D2 = doubled_gradient<T, NP>();
     T f[Q], g[Q];
     const T ph = phi[s];
     T dx, dy, dz, lap;
     // the 27-point stencil first, so that its temporaries are dead before the
     // 38 distribution values arrive (measured: +7 % for it in FP32, -2 % for
     // the 19-point one, which stays after the loads)
-    if constexpr (NP == 27) stencil_np<NP, T>(phi, n, ph, dx, dy, dz, lap);
+    if constexpr (NP == 27) stencil_np<NP, T, D2>(phi, n, ph, dx, dy, dz, lap);
 #pragma unroll
     for (int i = 0; i < Q; i++) {
         const size_t o = (size_t)i * S + n.src(i);
         f[i] = fa[o];
         if constexpr (!GEQ) g[i] = ga[o];
     }
-    if constexpr (NP != 27) stencil_np<NP, T>(phi, n, ph, dx, dy, dz, lap);
+    if constexpr (NP != 27) stencil_np<NP, T, D2>(phi, n, ph, dx, dy, dz, lap);
     if constexpr (GEQ) {
         // f's values are stored, and their registers free, before g's are formed
         T ux, uy, uz, mu;
         if (m)
-            collide_mrt_f<T, SH>(p, *m, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
+            collide_mrt_f<T, SH, D2>(p, *m, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
         else
-            collide_f<T, SH>(p, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
+            collide_f<T, SH, FEQ, D2>(p, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
 #pragma unroll
         for (int i = 0; i < Q; i++) fb[(size_t)i * S + s] = f[i];
         collide_g<T, true>(p, g, ph, ux, uy, uz, mu);
@@ -138,9 +149,9 @@ __device__ __forceinline__ void collide_site(const T *__restrict__ fa, const T *
         for (int i = 0; i < Q; i++) gb[(size_t)i * S + s] = g[i];
     } else {
         if (m)
-            collide_mrt<T, SH>(p, *m, f, g, ph, dx, dy, dz, lap);
+            collide_mrt<T, SH, D2>(p, *m, f, g, ph, dx, dy, dz, lap);
         else
-            collide<T, SH>(p, f, g, ph, dx, dy, dz, lap);
+            collide<T, SH, D2>(p, f, g, ph, dx, dy, dz, lap);
 #pragma unroll
         for (int i = 0; i < Q; i++) {
             fb[(size_t)i * S + s] = f[i];

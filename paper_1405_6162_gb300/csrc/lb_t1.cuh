@@ -231,13 +231,14 @@ __device__ __forceinline__ void t1_collide_site(const T *__restrict__ fa, const 
     for (int i = 0; i < Q; i++) f[i] = fa[(size_t)i * S + n.src(i)];
     const T ph = phi[s];
     T dx, dy, dz, lap;
-    stencil_np<NP, T>(phi, n, ph, dx, dy, dz, lap);
+    constexpr bool D2 = doubled_gradient<T, NP>();
+    stencil_np<NP, T, D2>(phi, n, ph, dx, dy, dz, lap);
     // the general collision's f part; g's result is its equilibrium, kept as moments
     T ux, uy, uz, mu;
     if (m)
-        collide_mrt_f<T, SH>(p, *m, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
+        collide_mrt_f<T, SH, D2>(p, *m, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
     else
-        collide_f<T, SH>(p, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
+        collide_f<T, SH, false, D2>(p, f, ph, dx, dy, dz, lap, ux, uy, uz, mu);
 #pragma unroll
     for (int i = 0; i < Q; i++) fb[(size_t)i * S + s] = f[i];
     Quad<T>::store(quad, s, gmh_of(ph, mu, p.gamma), ux, uy, uz);
