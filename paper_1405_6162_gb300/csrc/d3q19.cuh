@@ -105,72 +105,93 @@ struct Coll {
     T cg, g0, g1, g2, g1h, g2h, g1t, g2t;   // the same with omega_g
 };
 
-// Equilibria of f and g at one site.  R is rho (SH = false) or rho - rho0
-// (SH = true: the result is feq_i - w_i rho0).  j = sum f c = rho u.
-// sink(i, feq_i, geq_i) is called once per direction, i a literal after
-// inlining.
-template <typename T, bool SH, typename Sink>
-__device__ __forceinline__ void equilibria(const Coll<T>& p, T R, T jx, T jy, T jz,
-                                           T phi, T dx, T dy, T dz, T lap, Sink&& sink)
+// a + b as a term of further sums, and c x with c a power of two; for df64 a
+// sum that is not renormalised (df64.cuh)
+template <typename T>
+__device__ __forceinline__ T sum_term(T a, T b)
 {
-    const T third = T(1.0 / 3.0);
-    const T rho = SH ? p.rho0 + R : R;
-    const T rinv = T(1) / rho;
-    const T ux = jx * rinv, uy = jy * rinv, uz = jz * rinv;
+    return a + b;
+}
+template <typename T>
+__device__ __forceinline__ T scaled(float c, T x)
+{
+    return T(c) * x;
+}
+
+// Equilibria of f and g at one site at density rho0 and velocity u = (ux, uy,
+// uz).  SH: feq_i - w_i rho0 in place of feq_i.  FLOW = false: u = 0, nothing
+// of it is computed and opposite values are equal.  sink(i, feq_i, geq_i) is
+// called once per direction, i a literal after inlining, with values that for
+// df64 still are to be renormalised.
+template <typename T, bool SH, bool FLOW, typename Sink>
+__device__ __forceinline__ void equilibria(const Coll<T>& p, T ux, T uy, T uz, T phi, T dx, T dy, T dz, T lap,
+                                           Sink&& sink)
+{
+    const T zero = T(0);
     const T phi2 = phi * phi;
-    const T mu = phi * (p.A + p.B * phi2) - p.kappa * lap;
-    const T pb = phi2 * (T(0.5) * p.A + T(0.75) * p.B * phi2)
-               - p.kappa * (phi * lap + T(0.5) * (dx * dx + dy * dy + dz * dz));
-    // S = P + rho u u
-    const T Sxx = pb + p.kappa * dx * dx + jx * ux;
-    const T Syy = pb + p.kappa * dy * dy + jy * uy;
-    const T Szz = pb + p.kappa * dz * dz + jz * uz;
-    const T Sxy = p.kappa * dx * dy + jx * uy;
-    const T Sxz = p.kappa * dx * dz + jx * uz;
-    const T Syz = p.kappa * dy * dz + jy * uz;
-    const T t3 = (Sxx + Syy + Szz) * third;
-    // g: G = (Gamma mu - phi/3) I + phi u u;  G:Q_i = phi (c.u)^2 - phi u^2/3 + (Gamma mu - phi/3)(c^2 - 1)
-    const T pu2 = phi * (ux * ux + uy * uy + uz * uz) * third;
-    const T gm = p.gamma * mu - phi * third;
-
-    const T w0 = T(1.0 / 3.0), w1 = T(1.0 / 18.0), w2 = T(1.0 / 36.0);
-    const T h = T(4.5), three = T(3);
-
-    sink(0, w0 * (R - h * t3), w0 * (phi - h * (pu2 + gm)));
-
-    // faces: S:Q = S_aa - t3
-    {
-        T fs = w1 * (R + h * (Sxx - t3)), fa = w1 * three * jx;
-        T gs = w1 * (phi + h * (phi * ux * ux - pu2)), ga = w1 * three * phi * ux;
-        sink(1, fs + fa, gs + ga); sink(2, fs - fa, gs - ga);
+    const T kl = p.kappa * lap;
+    const T mu = phi * (p.A + p.B * phi2) - kl;
+    const T kx = p.kappa * dx, ky = p.kappa * dy, kz = p.kappa * dz;
+    const T xx = kx * dx, yy = ky * dy, zz = kz * dz;
+    const T pb = phi2 * (p.hA + p.qB * phi2) - (phi * kl + half(xx + yy + zz));
+    // S = P + rho u u, by the direct sums
+    T Sxx = pb + xx, Syy = pb + yy, Szz = pb + zz;
+    T Sxy = kx * dy, Sxz = kx * dz, Syz = ky * dz;
+    // 3 w2 j and 3 w2 phi u (w2 = 1/36), and the products phi u u
+    T jx = zero, jy = zero, jz = zero, px = zero, py = zero, pz = zero;
+    T pxx = zero, pyy = zero, pzz = zero, pxy = zero, pxz = zero, pyz = zero;
+    T bg = phi;
+    if constexpr (FLOW) {
+        const T Jx = p.rho0 * ux, Jy = p.rho0 * uy, Jz = p.rho0 * uz;
+        Sxx = fmadd(Jx, ux, Sxx), Syy = fmadd(Jy, uy, Syy), Szz = fmadd(Jz, uz, Szz);
+        Sxy = fmadd(Jx, uy, Sxy), Sxz = fmadd(Jx, uz, Sxz), Syz = fmadd(Jy, uz, Syz);
+        const T t2 = T(1.0 / 12.0), pt = phi * t2;
+        jx = t2 * Jx, jy = t2 * Jy, jz = t2 * Jz;
+        px = pt * ux, py = pt * uy, pz = pt * uz;
+        const T qx = phi * ux, qy = phi * uy, qz = phi * uz;
+        pxx = qx * ux, pyy = qy * uy, pzz = qz * uz;
+        pxy = qx * uy, pxz = qx * uz, pyz = qy * uz;
+        bg = phi - T(1.5) * (pxx + pyy + pzz);
     }
-    {
-        T fs = w1 * (R + h * (Syy - t3)), fa = w1 * three * jy;
-        T gs = w1 * (phi + h * (phi * uy * uy - pu2)), ga = w1 * three * phi * uy;
-        sink(3, fs + fa, gs + ga); sink(4, fs - fa, gs - ga);
-    }
-    {
-        T fs = w1 * (R + h * (Szz - t3)), fa = w1 * three * jz;
-        T gs = w1 * (phi + h * (phi * uz * uz - pu2)), ga = w1 * three * phi * uz;
-        sink(5, fs + fa, gs + ga); sink(6, fs - fa, gs - ga);
-    }
-    // edges: S:Q = S_aa + S_bb +/- 2 S_ab - t3
-#define LBK_EDGE(IP, IM, SAA, SBB, SAB, JA, JB, UA, UB, SGN)                          \
-    {                                                                                 \
-        const T cu = UA + SGN * UB;                                                   \
-        T fs = w2 * (R + h * (SAA + SBB + SGN * T(2) * SAB - t3));                    \
-        T fa = w2 * three * (JA + SGN * JB);                                          \
-        T gs = w2 * (phi + h * (phi * cu * cu - pu2 + gm));                           \
-        T ga = w2 * three * phi * cu;                                                 \
-        sink(IP, fs + fa, gs + ga); sink(IM, fs - fa, gs - ga);                       \
-    }
-    LBK_EDGE(7, 8, Sxx, Syy, Sxy, jx, jy, ux, uy, T(1))
-    LBK_EDGE(9, 10, Sxx, Syy, Sxy, jx, jy, ux, uy, T(-1))
-    LBK_EDGE(11, 12, Sxx, Szz, Sxz, jx, jz, ux, uz, T(1))
-    LBK_EDGE(13, 14, Sxx, Szz, Sxz, jx, jz, ux, uz, T(-1))
-    LBK_EDGE(15, 16, Syy, Szz, Syz, jy, jz, uy, uz, T(1))
-    LBK_EDGE(17, 18, Syy, Szz, Syz, jy, jz, uy, uz, T(-1))
-#undef LBK_EDGE
+    // feq_i = w_i [R + 3 c.j + 9/2 c S c - 3/2 tr S];
+    // geq_i = w_i [phi + 3 phi c.u + 9/2 (phi (c.u)^2 + (Gamma mu - phi/3)(c^2 - 1)) - 3/2 phi u^2]
+    // by weight class and opposite pair, the partial sums shared (collide_f,
+    // collide_g); 9/2 w is 1/4 for the faces and 1/8 for the edges
+    const T w0 = T(1.0 / 3.0), w2 = T(1.0 / 36.0);
+    const T b = (SH ? zero : p.rho0) - T(1.5) * (Sxx + Syy + Szz);
+    const T gm = p.gamma45 * mu - T(1.5) * phi;
+    sink(0, w0 * b, w0 * (bg - gm));
+    auto pair = [&](int ip, T fs, T fa, T gs, T ga) {
+        if constexpr (FLOW) {
+            sink(ip, sum_term(fs, fa), sum_term(gs, ga));
+            sink(ip + 1, sum_term(fs, -fa), sum_term(gs, -ga));
+        } else {
+            sink(ip, fs, gs);
+            sink(ip + 1, fs, gs);
+        }
+    };
+    const T F2 = w2 * b, F1 = twice(F2), G1 = twice(w2 * bg), G2 = w2 * (bg + gm);
+    auto face = [&](int ip, T saa, T ja, T paa, T pa) {
+        pair(ip, sum_term(scaled(0.25f, saa), F1), twice(ja), FLOW ? sum_term(scaled(0.25f, paa), G1) : G1, twice(pa));
+    };
+    face(1, Sxx, jx, pxx, px);
+    face(3, Syy, jy, pyy, py);
+    face(5, Szz, jz, pzz, pz);
+    // edge pairs (a + b, -a - b) from ip and (a - b, -a + b) from ip + 2
+    auto edges = [&](int ip, T saa, T sbb, T sab, T ja, T jb, T paa, T pbb, T pab, T pa, T pbc) {
+        const T fe = sum_term(scaled(0.125f, sum_term(saa, sbb)), F2), fo = scaled(0.25f, sab);
+        if constexpr (FLOW) {
+            const T ge = sum_term(scaled(0.125f, sum_term(paa, pbb)), G2), go = scaled(0.25f, pab);
+            pair(ip, sum_term(fe, fo), sum_term(ja, jb), sum_term(ge, go), sum_term(pa, pbc));
+            pair(ip + 2, sum_term(fe, -fo), sum_term(ja, -jb), sum_term(ge, -go), sum_term(pa, -pbc));
+        } else {
+            pair(ip, sum_term(fe, fo), zero, G2, zero);
+            pair(ip + 2, sum_term(fe, -fo), zero, G2, zero);
+        }
+    };
+    edges(7, Sxx, Syy, Sxy, jx, jy, pxx, pyy, pxy, px, py);
+    edges(11, Sxx, Szz, Sxz, jx, jz, pxx, pzz, pxz, px, pz);
+    edges(15, Syy, Szz, Syz, jy, jz, pyy, pzz, pyz, py, pz);
 }
 
 // Density moments of a (possibly shifted) distribution: R = sum f, j = sum f c.

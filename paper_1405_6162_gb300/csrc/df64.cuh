@@ -182,6 +182,27 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b)
     return r;
 }
 
+// a + b without the renormalisation: the high parts' sum, and its error with
+// the low parts.  Further sums of such values err no more (the parts' errors
+// are relative to the terms, not to the sum); renormalised() before a product
+// or storage.
+__device__ __forceinline__ df64 sum_term(df64 a, df64 b)
+{
+    df64 r;
+    float e;
+    dfops::two_sum(a.hi, b.hi, r.hi, e);
+    r.lo = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
+    return r;
+}
+__device__ __forceinline__ df64 renormalised(df64 a)
+{
+    df64 r;
+    dfops::two_sum(a.hi, a.lo, r.hi, r.lo);
+    return r;
+}
+// c x, c a power of two (exact, barring underflow)
+__device__ __forceinline__ df64 scaled(float c, df64 x) { return df64(c * x.hi, c * x.lo); }
+
 // x / 2: both parts halved, exactly (barring underflow)
 __device__ __forceinline__ df64 half(df64 a) { return df64(0.5f * a.hi, 0.5f * a.lo); }
 
@@ -281,5 +302,48 @@ __device__ __forceinline__ void equilibrium_pair(df64 &fp, df64 &fm, df64 s, df6
 __device__ __forceinline__ df64 &operator+=(df64 &a, df64 b) { return a = a + b; }
 __device__ __forceinline__ df64 &operator-=(df64 &a, df64 b) { return a = a - b; }
 __device__ __forceinline__ df64 &operator*=(df64 &a, df64 b) { return a = a * b; }
+
+// A stored value widened to FP64 exactly.  float: from the IEEE 754
+// binary32 and binary64 layouts -- sign and fraction kept (the fraction
+// moved up 29 bits), the exponent rebiased by 1023 - 127 = 896; a subnormal
+// is first scaled by 2^64 (exact in FP32, and normal) and rebiased by 64
+// less; zero keeps its sign, infinity stays infinite and NaN becomes a quiet
+// NaN.  Integer and FP32 operations only: on GB300 the conversion
+// instruction runs on the FP64 pipe (about 2 lanes a clock per SM), where it
+// costs as much as an addition.
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+    const bool sub = a < 0x00800000u;   // zero or subnormal
+    const unsigned v = sub ? (__float_as_uint(x * 0x1p64f) & 0x7fffffffu) : a;
+    unsigned hi = (v >> 3) + (sub ? 0x34000000u : 0x38000000u);
+    hi = v ? hi : 0u;
+    if (a >= 0x7f800000u) hi = (a >> 3) | 0x7ff00000u | (a > 0x7f800000u ? 0x00080000u : 0u);
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(v << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+// hi + lo of a double-float is exact in FP64 (|lo| <= ulp(hi) / 2)
+__device__ __forceinline__ double widen(df64 x) { return widen(x.hi) + widen(x.lo); }
+
+// A double as a double-float, to 2^-47, on the integer and FP32 units (the
+// conversions of df64(double) are four instructions of the FP64 pipe): the
+// top 24 bits and the next 23 are cut out of the IEEE 754 layout, the cut-off
+// part as an integer below 2^23 in the fraction of 2^23.  Values that are
+// zero, or too small or large for the parts to be normal floats, are
+// converted (zero by its sign bit).
+__device__ __forceinline__ df64 split_double(double d)
+{
+    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+    const unsigned e = (h >> 20) & 0x7ffu, sign = h & 0x80000000u;
+    if (e - 960u < 190u) {   // 2^-63 <= |d| < 2^127
+        const float hi = __uint_as_float(sign | (((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29));
+        const float cut = __fsub_rn(__uint_as_float(0x4b000000u | ((l >> 6) & 0x7fffffu)), 8388608.0f);
+        df64 r;
+        dfops::fast_two_sum(hi, __fmul_rn(__uint_as_float(sign | ((e - 942u) << 23)), cut), r.hi, r.lo);
+        return r;
+    }
+    if (((h << 1) | l) == 0) return df64(__uint_as_float(sign), 0.0f);
+    return df64(d);
+}
 
 }  // namespace lbk

@@ -19,47 +19,66 @@ namespace lbk {
 // ------------------------------------------------------------------ init
 
 // A_i(x - c_i) = feq_i(x), so that the first pull yields the equilibrium of
-// phi0 (its stencils taken in double) and u0.  Double storage evaluates the
-// equilibria in double.  Float and double-float storage evaluate them in
-// double-float arithmetic on the FP32 units (df64.cuh, ~48 bits; the double
-// pipe runs at 1/64 of the float rate): double-float storage keeps the
-// value, float storage its high part -- the float nearest to it, the same
-// float as rounding a double result except at a near tie.
-__device__ __forceinline__ void init_store(float *a, size_t o, df64 v) { a[o] = v.hi; }
-__device__ __forceinline__ void init_store(df64 *a, size_t o, df64 v) { a[o] = v; }
+// phi0 and u0.  Double storage evaluates stencils and equilibria in double.
+// Float and double-float storage evaluate the equilibria in double-float
+// arithmetic on the FP32 units (df64.cuh, ~48 bits; the double pipe runs at
+// 1/64 of the float rate): double-float storage, its stencils in double, keeps
+// the value, float storage its high part -- the float nearest to it, the same
+// float as rounding a double result except at a near tie.  Float storage
+// splits the inputs on the integer units and takes the stencils in
+// double-float too: with them in double, 50 instructions a site of the FP64
+// pipe (120 more at 27 points) bounded this kernel.  Without u0 half the sums
+// are not formed (opposite values are equal).
+// 256^3 float: 1659 -> 639 us without u0 (380 is the copy rate over its
+// bytes), 1959 -> 1247 us with it, bound by the FP32 units; 27 points
+// 129x97x65 197 -> 119 us.
+__device__ __forceinline__ void init_store(float *a, size_t o, df64 v) { a[o] = __fadd_rn(v.hi, v.lo); }
+__device__ __forceinline__ void init_store(df64 *a, size_t o, df64 v) { a[o] = renormalised(v); }
+__device__ __forceinline__ void init_store(double *a, size_t o, double v) { a[o] = v; }
 
-template <typename T, bool SH, int NP>
+// inputs and stencils of storage T: split on the integer units for float
+// storage, else doubles
+template <typename T>
+struct InitArith {
+    using type = double;
+    static __device__ __forceinline__ double in(double v) { return v; }
+};
+template <>
+struct InitArith<float> {
+    using type = df64;
+    static __device__ __forceinline__ df64 in(double v) { return split_double(v); }
+};
+template <>
+__device__ __forceinline__ df64 stencil_value<df64, double>(double v)
+{
+    return split_double(v);
+}
+
+// p in the arithmetic type E of the equilibria; FLOW: u0 is given
+template <typename T, typename E, bool SH, int NP, bool FLOW>
 __global__ void __launch_bounds__(256) k_init(const double *__restrict__ phi0,
                                               const double *__restrict__ u0,
                                               T *__restrict__ fa, T *__restrict__ ga,
-                                              Coll<double> p, Coll<df64> pd, int nx, int ny, int nz, long long S)
+                                              Coll<E> p, int nx, int ny, int nz, long long S)
 {
     const long long N = (long long)nx * ny * nz;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
     const Nbr n(s, nx, ny, nz);
-    const double ph = phi0[s];
-    double dx, dy, dz, lap;
-    stencil_np<NP, double>(phi0, n, ph, dx, dy, dz, lap);
-    const double jx = u0 ? p.rho0 * u0[s] : 0.0;
-    const double jy = u0 ? p.rho0 * u0[N + s] : 0.0;
-    const double jz = u0 ? p.rho0 * u0[2 * N + s] : 0.0;
-    const double R = SH ? 0.0 : p.rho0;
-    if constexpr (sizeof(T) == 8 && !is_df64<T>::value) {
-        equilibria<double, SH>(p, R, jx, jy, jz, ph, dx, dy, dz, lap, [&](int i, double fe, double ge) {
-            const size_t o = (size_t)i * S + n.src(i);
-            fa[o] = fe;
-            ga[o] = ge;
-        });
-    } else {
-        const df64 zero(0.0f, 0.0f);
-        equilibria<df64, SH>(pd, df64(R), u0 ? df64(jx) : zero, u0 ? df64(jy) : zero, u0 ? df64(jz) : zero,
-                             df64(ph), df64(dx), df64(dy), df64(dz), df64(lap), [&](int i, df64 fe, df64 ge) {
-                                 const size_t o = (size_t)i * S + n.src(i);
-                                 init_store(fa, o, fe);
-                                 init_store(ga, o, ge);
-                             });
-    }
+    using In = InitArith<T>;
+    using R = typename In::type;
+    const R ph = In::in(phi0[s]);
+    R dx, dy, dz, lap;
+    stencil_np<NP, R>(phi0, n, ph, dx, dy, dz, lap);
+    E u[3] = {E(0), E(0), E(0)};
+    if (FLOW)
+#pragma unroll
+        for (int a = 0; a < 3; a++) u[a] = E(In::in(u0[a * N + s]));
+    equilibria<E, SH, FLOW>(p, u[0], u[1], u[2], E(ph), E(dx), E(dy), E(dz), E(lap), [&](int i, E fe, E ge) {
+        const size_t o = (size_t)i * S + n.src(i);
+        init_store(fa, o, fe);
+        init_store(ga, o, ge);
+    });
 }
 
 // ------------------------------------------------------------------ moments / state
@@ -152,28 +171,6 @@ __device__ __forceinline__ void block_sum(double (&acc)[K], double *out)
         }
     }
 }
-
-// A stored value widened to FP64 exactly.  float: from the IEEE 754
-// binary32 and binary64 layouts -- sign and fraction kept (the fraction
-// moved up 29 bits), the exponent rebiased by 1023 - 127 = 896; a subnormal
-// is first scaled by 2^64 (exact in FP32, and normal) and rebiased by 64
-// less; zero keeps its sign, infinity stays infinite and NaN becomes a quiet
-// NaN.  Integer and FP32 operations only: on GB300 the conversion
-// instruction runs on the FP64 pipe (about 2 lanes a clock per SM), where it
-// would double this kernel's FP64 work.
-__device__ __forceinline__ double widen(float x)
-{
-    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
-    const bool sub = a < 0x00800000u;   // zero or subnormal
-    const unsigned v = sub ? (__float_as_uint(x * 0x1p64f) & 0x7fffffffu) : a;
-    unsigned hi = (v >> 3) + (sub ? 0x34000000u : 0x38000000u);
-    hi = v ? hi : 0u;
-    if (a >= 0x7f800000u) hi = (a >> 3) | 0x7ff00000u | (a > 0x7f800000u ? 0x00080000u : 0u);
-    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(v << 29));
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-// hi + lo of a double-float is exact in FP64 (|lo| <= ulp(hi) / 2)
-__device__ __forceinline__ double widen(df64 x) { return widen(x.hi) + widen(x.lo); }
 
 // s + e = a + b exactly (Knuth), s into a; e is returned
 __device__ __forceinline__ float two_sum_into(float &a, float b)
@@ -332,10 +329,10 @@ template <typename T, bool SH, int NP>
 static void init_np(lb_ctx *c, const double *phi0_d, const double *u0_d)
 {
     const int cur = c->buf.cur;
-    k_init<T, SH, NP><<<grid_for(c->N, 256), 256, 0, c->stream>>>(phi0_d, u0_d, (T *)c->buf.f[cur],
-                                                                  (T *)c->buf.g[cur], make_coll<double>(c->p),
-                                                                  make_coll<df64>(c->p), c->p.nx, c->p.ny,
-                                                                  c->p.nz, c->S);
+    using E = typename std::conditional<std::is_same<T, double>::value, double, df64>::type;
+    const auto kernel = u0_d ? k_init<T, E, SH, NP, true> : k_init<T, E, SH, NP, false>;
+    kernel<<<grid_for(c->N, 256), 256, 0, c->stream>>>(phi0_d, u0_d, (T *)c->buf.f[cur], (T *)c->buf.g[cur],
+                                                       make_coll<E>(c->p), c->p.nx, c->p.ny, c->p.nz, c->S);
 }
 
 template <typename T, bool SH>
