@@ -784,7 +784,7 @@ def run_ours(args):
         ach = adds * n / t / 1e12 if adds else None
         tr = _profile_value("reduce_128cubed", f"dram_bytes_per_site_{prec}")
         return {"ms_per_call": t * 1e3, "sites_per_s": n / t,
-                "roofline": {"bound": "alu (FP64 pipe)", "kernel": "k_reduce_partial", "achieved": ach,
+                "roofline": {"bound": "alu (FP64 pipe)", "kernel": "k_reduce", "achieved": ach,
                              "peak": pk / 2 if pk else None, "unit": "T FP64 instructions/s",
                              "frac": ach / (pk / 2) if (ach and pk) else None, "fp64_adds_per_site": adds,
                              "peak_kind": "measured in this run: FMA instructions/s of lb_probe_fp64_fma",

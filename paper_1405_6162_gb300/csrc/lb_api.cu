@@ -57,7 +57,7 @@ void free_all(lb_ctx *c)
     dev_free(c, c->phi, (size_t)c->N * c->esize);
     dev_free(c, c->io, io_bytes(c));
     dev_free(c, c->partial, (size_t)lbk::kReduceBlocks * 5 * sizeof(double));
-    dev_free(c, c->dev_out, 8 * sizeof(double));
+    dev_free(c, c->dev_out, sizeof(lbk::ReduceOut));
     dev_free(c, c->lag_counters, (size_t)(c->p.nz + 1) * sizeof(unsigned long long));
     if (!c->batch_owned) dev_free(c, c->err_flag, sizeof(unsigned int));
     dev_free(c, c->mask_buf, (size_t)c->N);
@@ -215,7 +215,7 @@ int lb_create(const lb_params *p, void *cuda_stream, lb_ctx **out)
     }
     c->phi = dev_alloc(c, (size_t)c->N * c->esize);
     c->partial = (double *)dev_alloc(c, (size_t)lbk::kReduceBlocks * 5 * sizeof(double));
-    c->dev_out = (double *)dev_alloc(c, 8 * sizeof(double));
+    c->dev_out = (lbk::ReduceOut *)dev_alloc(c, sizeof(lbk::ReduceOut));
     c->lag_counters = (unsigned long long *)dev_alloc(c, (size_t)(p->nz + 1) * sizeof(unsigned long long));
     c->err_flag = (unsigned int *)dev_alloc(c, sizeof(unsigned int));
     bool ok = c->phi && c->partial && c->dev_out && c->lag_counters && c->err_flag;
@@ -228,6 +228,7 @@ int lb_create(const lb_params *p, void *cuda_stream, lb_ctx **out)
     rc = lbk::cuda_status(cudaMemsetAsync(c->lag_counters, 0, (size_t)(p->nz + 1) * sizeof(unsigned long long),
                                           c->stream));
     if (!rc) rc = lbk::cuda_status(cudaMemsetAsync(c->err_flag, 0, sizeof(unsigned int), c->stream));
+    if (!rc) rc = lbk::cuda_status(cudaMemsetAsync(c->dev_out, 0, sizeof(lbk::ReduceOut), c->stream));
     for (int k = 0; k < 2 && !rc; k++) {
         rc = lbk::cuda_status(cudaMemsetAsync(c->buf.f[k], 0, dist_bytes(c), c->stream));
         if (!rc) rc = lbk::cuda_status(cudaMemsetAsync(c->buf.g[k], 0, dist_bytes(c), c->stream));
@@ -475,10 +476,16 @@ int lb_moments(lb_ctx *c, double *rho, double *u, double *phi, int ptr_kind)
 int lb_reduce(lb_ctx *c, double out[5])
 {
     if (!c || !out) return LB_ERR_INVALID;
-    int rc = lbk::launch_reduce(c, c->dev_out);
-    if (!rc) rc = copy(c, out, c->dev_out, 5 * sizeof(double), cudaMemcpyDeviceToHost);
-    if (!rc) rc = sync(c);
+    lbk::ReduceOut res;
+    int rc = lbk::launch_reduce(c);
+    if (!rc) rc = copy(c, &res, c->dev_out, sizeof(res), cudaMemcpyDeviceToHost);
+    if (!rc) rc = lbk::cuda_status(cudaStreamSynchronize(c->stream));
     if (rc) return rc;
+    for (int k = 0; k < 5; k++) out[k] = res.totals[k];
+    if (res.wait_failed) {
+        rc = sync(c);   // reports and clears it
+        if (rc) return rc;
+    }
     for (int k = 0; k < 5; k++)
         if (!std::isfinite(out[k])) return LB_ERR_NONFINITE;
     return LB_OK;

@@ -26,6 +26,13 @@ struct Buffers {
     int cur = 0;                      // index of the buffer holding the state
 };
 
+// result of lb_reduce in device memory
+struct ReduceOut {
+    double totals[5];           // sum rho, sum rho u, sum phi
+    unsigned int wait_failed;   // *err_flag when the totals were formed
+    unsigned int ticket;        // CTAs of the reduction that are done; 0 between calls
+};
+
 }  // namespace lbk
 
 struct lb_ctx {
@@ -39,7 +46,7 @@ struct lb_ctx {
     void *phi = nullptr;   // [N] storage type: order parameter of the two-pass kernel
     double *io = nullptr;  // [4N] FP64 staging for host transfers (lazy)
     double *partial = nullptr;  // reduction partials [kReduceBlocks][5]
-    double *dev_out = nullptr;  // [8] reduction result
+    lbk::ReduceOut *dev_out = nullptr;   // reduction result
     // lagged kernel: [0] = CTA ticket counter, [1 + z] = phi-done counter of plane z
     unsigned long long *lag_counters = nullptr;
     unsigned int *err_flag = nullptr;         // set by a device-side wait that timed out
@@ -130,7 +137,7 @@ int launch_get_state(lb_ctx *c, double *f, double *g);
 int launch_set_state(lb_ctx *c, const double *f, const double *g);
 // rows [i0, i1) of f (which = 0) or g (which = 1): dir 0 = out of the state, 1 = into it
 int launch_rows(lb_ctx *c, int which, int i0, int i1, double *buf, int dir);
-int launch_reduce(lb_ctx *c, double *dev_out5);   // reduced form: phi from component 0
+int launch_reduce(lb_ctx *c);   // into c->dev_out; reduced form: phi from component 0
 
 // fused kernel (lb_fused.cu)
 int launch_step_fused(lb_ctx *c, int nsteps);
