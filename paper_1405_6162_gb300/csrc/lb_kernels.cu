@@ -111,6 +111,30 @@ k_collide_pull_mrt(const T *__restrict__ fa, const T *__restrict__ ga, const T *
 
 static inline unsigned grid_for(long long N, int tpb) { return (unsigned)((N + tpb - 1) / tpb); }
 
+// Threads per CTA of both passes where the caller leaves them open; small
+// lattices want small CTAs, which spread over the SMs.  Microseconds a step:
+//   FP64 (bound by its instructions): 32 below 2^18 sites -- 16^3 19.8 at 256
+//   threads, 10.8 at 32; 70x37x11 21.9 / 16.3 (tau, tau_g != 1 30.8 / 18.5);
+//   32^3 23.2 / 17.8; 48^3 56.7 / 50.7; 56x52x60 84.9 / 74.0.  Above, 128 or
+//   192, whichever leaves the busiest of the 152 SMs fewer sites: 64^3 114.5
+//   at 256, 113.6 at 128, 109.8 at 192; 80^3 221.3, 213.6, 214.1; 100^3 407.1,
+//   405.5, 409.2.
+//   FP32: 128 below 2^20 sites -- 16^3 4.28 / 3.64, 64^3 13.05 / 12.33 (tau_g
+//   != 1 14.1 / 13.4), 80^3 26.6 / 25.7, 100^3 51.2 / 50.6 -- and 256 above,
+//   where 128 lose up to 2 % (160^3 234.6 / 239.5).
+//   Double-float: 64 below 2^18 sites (16^3 to 56x52x60 3 to 8 % with tau_g
+//   != 1, 1 % without), 256 above (128x128x64 152.3 / 155.4).
+template <typename T>
+static int default_threads(long long N)
+{
+    const bool small = N < (1LL << 18);
+    if (is_df64<T>::value) return small ? 64 : 256;
+    if (sizeof(T) == 4) return N < (1LL << 20) ? 128 : 256;
+    if (small) return 32;
+    auto busiest = [&](int tpb) { return ((N + tpb - 1) / tpb + 151) / 152 * tpb; };
+    return busiest(192) < busiest(128) ? 192 : 128;
+}
+
 // the phi pass with V sites per thread
 template <typename T>
 static cudaError_t launch_phi(lb_ctx *c, const T *ga, T *phi, int tpb, int vvl)
@@ -145,8 +169,8 @@ template <typename T, bool SH, int NP>
 static int two_pass(lb_ctx *c, int nsteps)
 {
     // launch shape: threads per CTA of both passes, sites per thread of the
-    // phi pass (lb_set_kernel's block_x, block_y; 0 = 256 and 1)
-    const int tpb = c->block_x ? c->block_x : 256;
+    // phi pass (lb_set_kernel's block_x, block_y; 0 = default_threads and 1)
+    const int tpb = c->block_x ? c->block_x : default_threads<T>(c->N);
     const int vvl = c->block_y ? c->block_y : 1;
     for (int t = 0; t < nsteps; t++) {
         const int a = c->buf.cur, b = 1 - a;
@@ -168,23 +192,24 @@ int launch_two_pass_fp64_raw(const lb_params &prm, const double *fa, const doubl
 {
     const auto p = make_coll<double>(prm);
     const long long N = (long long)prm.nx * prm.ny * prm.nz;
-    const unsigned grid = grid_for(N, 256);
-    k_phi_pull<double, 1><<<grid, 256, 0, stream>>>(ga, phi, prm.nx, prm.ny, prm.nz, S);
+    const int tpb = default_threads<double>(N);
+    const unsigned grid = grid_for(N, tpb);
+    k_phi_pull<double, 1><<<grid, tpb, 0, stream>>>(ga, phi, prm.nx, prm.ny, prm.nz, S);
     const auto collide = !g_is_equilibrium(prm)  ? k_collide_pull<double, false, 7, false, false>
                          : f_is_equilibrium(prm) ? k_collide_pull<double, false, 7, true, true>
                                                  : k_collide_pull<double, false, 7, true, false>;
-    collide<<<grid, 256, 0, stream>>>(fa, ga, phi, fb, gb, p, prm.nx, prm.ny, prm.nz, S);
+    collide<<<grid, tpb, 0, stream>>>(fa, ga, phi, fb, gb, p, prm.nx, prm.ny, prm.nz, S);
     return check_launch();
 }
 
 cudaError_t launch_phi_pull(lb_ctx *c, const float *ga, float *phi)
 {
-    return launch_phi<float>(c, ga, phi, c->block_x ? c->block_x : 256, c->block_y ? c->block_y : 1);
+    return launch_phi<float>(c, ga, phi, c->block_x ? c->block_x : default_threads<float>(c->N), c->block_y ? c->block_y : 1);
 }
 
 cudaError_t launch_collide_geq(lb_ctx *c, const float *fa, const float *phi, float *fb, float *gb)
 {
-    const int tpb = c->block_x ? c->block_x : 256;
+    const int tpb = c->block_x ? c->block_x : default_threads<float>(c->N);
     const float *no_g = nullptr;
     if (c->npts == 19) return launch_collide<float, true, 19, true>(c, fa, no_g, phi, fb, gb, tpb);
     if (c->npts == 27) return launch_collide<float, true, 27, true>(c, fa, no_g, phi, fb, gb, tpb);
