@@ -116,6 +116,40 @@ def test_trajectory_gradient_matches_oracle_16cubed(segment):
     assert abs(kappa.grad.item() - gk_o) <= 1e-10 * abs(gk_o)
 
 
+def test_states_are_kept_as_memory_allows(monkeypatch):
+    """Every state where the free memory holds 8 times as much, else one every
+    ~sqrt(T) steps, none where no backward can follow: the same phi_T and
+    gradient bit for bit."""
+    import torch
+    from paper_1405_6162_gb300 import adjoint
+    dims, T = (9, 8, 7), 11
+    n = 504
+    phi0 = _cuda(L.spinodal_phi0(*dims, seed=240, amp=0.3))
+    allocated = []
+    states = adjoint._States
+    monkeypatch.setattr(adjoint, "_States", lambda n, count: allocated.append(count) or states(n, count))
+
+    def gradient(free):
+        monkeypatch.setattr(adjoint, "_free_bytes", lambda: free)
+        allocated.clear()
+        x = phi0.clone().requires_grad_(True)
+        y = adjoint.trajectory(x, P0["kappa"], dims, P0, T)
+        y.square().sum().backward()
+        return y.detach(), x.grad, list(allocated)
+
+    need = T * 38 * n * 8
+    y1, g1, kept = gradient(8 * need)
+    assert kept == [T, 0]
+    y2, g2, kept = gradient(8 * need - 8)
+    assert kept == [4, 2]          # round(sqrt(11)) = 3 steps apart, 2 between
+    assert torch.equal(y1, y2) and torch.equal(g1, g2)
+    with torch.no_grad():
+        y3 = adjoint.trajectory(phi0.clone().requires_grad_(True), P0["kappa"], dims, P0, T)
+    y4 = adjoint.trajectory(phi0, P0["kappa"], dims, P0, T)
+    assert torch.equal(y3, y1) and torch.equal(y4, y1) and not y3.requires_grad and not y4.requires_grad
+    assert allocated == [4, 2]
+
+
 def test_gradient_agrees_with_finite_differences_64cubed_T200():
     """The 64^3, T = 200 workload: loss sum (phi_T - phi_target)^2 with a
     seeded tanh droplet of radius 16; gradient wrt kappa and along random
