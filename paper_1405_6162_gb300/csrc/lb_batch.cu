@@ -16,8 +16,8 @@
 // per-site arithmetic is the default step's (lb_site.cuh), or, for an
 // ensemble whose lattices all have tau_g = 1 and that was switched to the
 // reduced form, the reduced form's two passes (lb_t1.cuh): the collide pass
-// over the same (lattice, block) items, then the phi pass over (lattice, x
-// block, warp group, z run) tiles.  The launch (with a reset of the barrier
+// over the same (lattice, block) items, then the phi pass over (lattice,
+// block of positions, z run) tiles, one a warp.  The launch (with a reset of the barrier
 // state) is captured once per (steps, parity) into a CUDA graph and
 // replayed.  The block size and CTAs per SM -- the paper's TPB and its
 // per-thread work (targetDP Sec. III.C) -- are the knobs the autotuner sets.
@@ -77,13 +77,6 @@ struct LatDesc {
     Coll<T> p;
 };
 
-// z planes of a reduced-form phi tile, about (a lattice's planes are split
-// evenly; a run reads two planes more than it writes).  64 lattices of sides
-// 16..64, 256 threads: 158.6 us a step at 14, 159.8 at 8, 159.5 at 16, 165 at 24
-#ifndef LBK_BATCH_T1_KZC
-#define LBK_BATCH_T1_KZC 14
-#endif
-constexpr int kBatchT1Kzc = LBK_BATCH_T1_KZC;
 constexpr int kBatchPhiV = LBK_BATCH_PHI_V;   // phi-pass work items per trip (general form)
 
 struct GridBarrier {
@@ -235,12 +228,11 @@ struct BatchPasses {
     {
         constexpr int KY = PhiTile<T>::KY;
         const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int w = G.to + r; w < G.to + G.tn; w += G.m) {
-            const int4 it = work_t1[w];   // (lattice, x block, warp group, z run)
+        for (int w = G.to + r * warps + warp; w < G.to + G.tn; w += G.m * warps) {
+            const int4 it = work_t1[w];   // (lattice, block of positions, z run, -)
             const LatDesc<T> &L = lats[it.x];
             if (!take(L)) continue;
-            t1_phi_tile<T, KY>(phi(L), quads(L.g[q], L.S), out(L), L.nx, L.ny, L.nz, L.kzc, it.y,
-                               (it.z * warps + warp) * KY, it.w, lane);
+            t1_phi_tile<T, KY>(phi(L), quads(L.g[q], L.S), out(L), L.nx, L.ny, L.nz, L.kzc, it.y, 1, 0, it.z, lane);
         }
     }
     // the lattices of this CTA's first work items now have their moments
@@ -455,7 +447,6 @@ int batch_tables(lb_batch *b)
     // per lattice: descriptor, collide items, reduced-form phi tiles
     const int n = b->n;
     std::vector<lbk::LatDesc<T>> L(n);
-    std::vector<std::vector<int4>> tiles(n);
     std::vector<long long> nb(n);
     for (int k = 0; k < n; k++) {
         lb_ctx *c = b->ctx[k];
@@ -471,17 +462,7 @@ int batch_tables(lb_batch *b)
         L[k].phi = (T *)c->phi;
         L[k].moments = c->moments;
         L[k].p = lbk::make_coll<T>(c->p);
-        const int runs = std::max(1, (c->p.nz + lbk::kBatchT1Kzc / 2) / lbk::kBatchT1Kzc);
-        L[k].kzc = (c->p.nz + runs - 1) / runs;   // runs of about equal length
         nb[k] = (c->N + b->threads - 1) / b->threads;
-        if (b->reduced || (b->unread_g && sizeof(T) == 4)) {
-            const int rows = (b->threads / 32) * lbk::PhiTile<T>::KY;   // y rows of one warp group
-            const int gx = (c->p.nx + lbk::kPhiOut - 1) / lbk::kPhiOut, gy = (c->p.ny + rows - 1) / rows;
-            const int gz = (c->p.nz + L[k].kzc - 1) / L[k].kzc;
-            for (int z = 0; z < gz; z++)
-                for (int y = 0; y < gy; y++)
-                    for (int x = 0; x < gx; x++) tiles[k].push_back(make_int4(k, x, y, z));
-        }
     }
 
     // CTA groups, and the work lists ordered group by group
@@ -490,6 +471,8 @@ int batch_tables(lb_batch *b)
     rc = lbk::plan_groups(n, nb.data(), b->grid, b->bins, lat_group.data(), cta0.data(), m.data(), &ng);
     if (rc) return rc;
     std::vector<lbk::Group> groups(ng);
+    std::vector<long long> load(ng, 0);   // collide items of the group
+    for (int k = 0; k < n; k++) load[lat_group[k]] += nb[k];
     std::vector<int> cta_group(b->grid, -1);
     std::vector<int2> work;
     std::vector<int4> work_t1;
@@ -502,7 +485,19 @@ int batch_tables(lb_batch *b)
         for (int k = 0; k < n; k++) {
             if (lat_group[k] != g) continue;
             for (long long j = 0; j < nb[k]; j++) work.push_back(make_int2(k, (int)j));
-            work_t1.insert(work_t1.end(), tiles[k].begin(), tiles[k].end());
+            if (!b->reduced && !(b->unread_g && sizeof(T) == 4)) continue;
+            // the lattice's tiles, their run length for its share of the group's
+            // warps.  Tiles go to single warps: a group has some tens of CTAs at
+            // most, and whole-CTA tiles of one run length for all left it 1.9
+            // times the work of an even split on average, 2.9 in the worst group.
+            // 64 lattices of sides 16..64, 100 steps with starts and read-out:
+            // 20.8 -> 18.7 ms.
+            const lb_params &p = b->ctx[k]->p;
+            const int blocks = lbk::phi_blocks(p.nx, p.ny, lbk::PhiTile<T>::KY, 1);
+            const long long warps = std::max(1LL, G.m * (b->threads / 32) * nb[k] / load[g]);
+            L[k].kzc = lbk::phi_run_length(blocks, p.nz, warps);
+            for (int z = 0; z * L[k].kzc < p.nz; z++)
+                for (int x = 0; x < blocks; x++) work_t1.push_back(make_int4(k, x, z, 0));
         }
         G.wn = (int)work.size() - G.wo;
         G.tn = (int)work_t1.size() - G.to;

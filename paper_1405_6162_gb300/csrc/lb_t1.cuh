@@ -4,6 +4,8 @@
 // lb_taug1.cu.
 #pragma once
 
+#include <algorithm>
+
 #include "d3q19.cuh"
 #include "df64.cuh"
 #include "lb_site.cuh"
@@ -250,7 +252,43 @@ __device__ __forceinline__ void t1_collide_site(const T *__restrict__ fa, const 
     }
 }
 
-constexpr int kPhiOut = 30;    // output columns per warp
+constexpr int kPhiOut = 30;    // output positions per warp (t1_phi_tile)
+
+// Positions of a phi pass whose warps are stacked `stack` high in y: rows of
+// KY * stack lattice rows, each row its nx columns and a halo column at
+// either end; and the warps (stacks of warps) that cover them.
+// (Unsigned: rows of one site have three positions each.)
+__host__ __device__ inline unsigned phi_positions(int nx, int ny, int ky, int stack)
+{
+    return (unsigned)((ny - 1) / (ky * stack) + 1) * (unsigned)(nx + 2);
+}
+__host__ __device__ inline int phi_blocks(int nx, int ny, int ky, int stack)
+{
+    return (int)((phi_positions(nx, ny, ky, stack) - 1) / kPhiOut + 1);
+}
+
+// z planes of a phi pass's tiles: `blocks` tiles cover a plane, `slots` tiles
+// run at a time.  The planes are split into runs of about equal length, at
+// most 64, such that the planes walked one after the other are the fewest: a
+// run reads two planes more than it writes, and its first loads wait, counted
+// as a third.  FP32, us a step, against runs sized for about three waves of
+// CTAs: 256^3 530 -> 513, 128^3 74.5 -> 68.2, 200x152x136 140.0 -> 131.2,
+// 129x97x65 32.6 -> 31.0, 80^3 21.4 -> 19.4; no run length of 12, 16, 24, 32
+// or 64 was faster on any of nine sizes.
+inline int phi_run_length(long long blocks, int nz, long long slots)
+{
+    int best = 0;
+    long long best_cost = 0;
+    for (int k = 1; k <= 64 && (k <= nz || !best); k++) {
+        const int runs = (nz - 1) / k + 1, kzc = (nz - 1) / runs + 1;
+        const long long cost = (blocks * runs - 1) / slots + 1;
+        if (!best || cost * (kzc + 3) < best_cost) {
+            best_cost = cost * (kzc + 3);
+            best = kzc;
+        }
+    }
+    return std::max(best, (nz - 1) / 65535 + 1);   // the grid's limit on runs
+}
 
 #ifndef LBK_T1_KY32
 #define LBK_T1_KY32 1
@@ -282,28 +320,42 @@ __device__ __forceinline__ void t1_load_site(const T *__restrict__ phi, const T 
     d[0] = phi[o], d[1] = v[0], d[2] = v[1], d[3] = v[2], d[4] = v[3];
 }
 
-// The phi pass for the tile of one warp: x columns bx*30 - 1 .. bx*30 + 30
-// (lane = column - bx*30 + 1), y rows y0 .. y0 + KY - 1, output planes
-// bz*kzc .. bz*kzc + kzc - 1.  No block-level synchronisation.  Source plane
+// The phi pass for the tile of one warp.  The rows of the lattice (groups of
+// KY * stack rows, of which this warp takes the wy-th KY) follow one another
+// as a stream of positions, each row its columns 0 .. nx - 1 between a halo
+// position for column -1 and one for column nx; the tile is positions
+// bxy*30 - 1 .. bxy*30 + 30 of the stream (lane = position - bxy*30 + 1) and
+// the output planes bz*kzc .. bz*kzc + kzc - 1.  Of a warp the inner 30 lanes
+// write, those on halo positions excepted, and a lane's neighbours are its
+// columns x - 1 and x + 1 also where a row ends.  So nx / (nx + 2) of the
+// writing lanes have work on rows of any length, where a warp per 30 columns
+// left 14 % of them idle at nx = 129, 29 % at 64 and 45 % at 33.
+// No block-level synchronisation.  Source plane
 // j of the run (z0 + j - 1, j = 0 .. nzc + 1) is summed row by row; once a
 // row's moments are expanded its registers take the same row of plane
 // j + 1, so a plane of arithmetic covers each load's latency and one plane
 // of raw moments is held.  Site offsets fit an int (N < 2^31).
 template <typename T, int KY>
 __device__ __forceinline__ void t1_phi_tile(const T *__restrict__ phi, const T *__restrict__ q0,
-                                            T *__restrict__ phi_out, int nx, int ny, int nz, int kzc, int bx, int y0,
-                                            int bz, int lane)
+                                            T *__restrict__ phi_out, int nx, int ny, int nz, int kzc, int bxy,
+                                            int stack, int wy, int bz, int lane)
 {
-    if (y0 >= ny) return;   // uniform over the warp
     const int z0 = bz * kzc;
     const int nzc = min(kzc, nz - z0);   // output planes z0 .. z0 + nzc - 1
-    const int xu = bx * kPhiOut + lane - 1;   // unwrapped column, -1 .. nx + 30
-    const int x = wrap_up(xu + nx, nx);
-    const bool out_x = lane >= 1 && lane <= kPhiOut && xu < nx;
+    const unsigned positions = phi_positions(nx, ny, KY, stack);
+    const unsigned after = (unsigned)bxy * kPhiOut + lane;   // position + 1; 0 and those past the end feed no output
+    const unsigned in = min(after ? after - 1 : 0, positions - 1);
+    const int row = (int)(in / (nx + 2));
+    const int xu = (int)(in - (unsigned)row * (nx + 2)) - 1;   // column, -1 and nx the halo
+    const int x = xu < 0 ? nx - 1 : xu == nx ? 0 : xu;
+    const int y0 = (row * stack + wy) * KY;   // past the lattice in the last group: wrapped, not written
+    // rows this lane writes
+    const bool writes = lane >= 1 && lane <= kPhiOut && after <= positions && xu >= 0 && xu < nx;
+    const int nrows = writes ? min(KY, ny - y0) : 0;
     const int plane = nx * ny;
     int yoff[KY + 2];
 #pragma unroll
-    for (int k = 0; k < KY + 2; k++) yoff[k] = x + wrap_up(y0 - 1 + k + ny, ny) * nx;
+    for (int k = 0; k < KY + 2; k++) yoff[k] = x + wrap_up(y0 - 1 + k + ny, ny) * nx;   // ny times a few at most
     // partial sums of output plane oz live in slot oz mod 3
     T acc[3][KY], acc_r[3][KY], acc_l[3][KY];
 #pragma unroll
@@ -388,7 +440,7 @@ __device__ __forceinline__ void t1_phi_tile(const T *__restrict__ phi, const T *
             for (int a = 0; a < KY; a++) {
                 const T from_left = shfl_up1(acc_r[qd][a]);
                 const T from_right = shfl_down1(acc_l[qd][a]);
-                if (out_x && oz >= 0 && y0 + a < ny)
+                if (a < nrows && oz >= 0)
                     phi_out[yoff[a + 1] + (z0 + oz) * plane] =
                         fmadd(T(1.0 / 36.0), add_px(acc[qd][a], add_px(from_left, from_right)), own[a]);
                 acc[qd][a] = acc_r[qd][a] = acc_l[qd][a] = T(0);

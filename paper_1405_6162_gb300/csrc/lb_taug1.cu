@@ -18,8 +18,9 @@
 //                 other level's component 0          (5 r, 1 w words)
 // -- 49 words per site instead of the 97 of the general two-pass step.
 // k_t1_phi streams along z so that each source site's moments are loaded and
-// expanded about once: a warp covers 32 consecutive x columns of which the
-// 30 inner ones are outputs (the outer two only feed their neighbours); each
+// expanded about once: a warp covers 32 consecutive positions of the rows
+// (with halo positions between them, t1_phi_tile) of which the 30 inner ones
+// are outputs (the outer two only feed their neighbours); each
 // lane walks a run of z planes for KY rows of its column, holding the
 // partial sums of the three output planes a source plane reaches.  Sources
 // in the lane's own column (c_x = 0) add to its own outputs; those with
@@ -34,6 +35,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <type_traits>
 #include <utility>
 
 #include "d3q19.cuh"
@@ -82,8 +84,8 @@ __global__ void __launch_bounds__(32 * kPhiMaxWarps) k_t1_phi(const T *__restric
                                                                int nx, int ny, int nz, int kzc)
 {
     pdl_wait_then_release();
-    t1_phi_tile<T, KY>(phi, quad, phi_out, nx, ny, nz, kzc, blockIdx.x,
-                       (blockIdx.y * blockDim.y + threadIdx.y) * KY, blockIdx.z, threadIdx.x);
+    t1_phi_tile<T, KY>(phi, quad, phi_out, nx, ny, nz, kzc, blockIdx.x, blockDim.y, threadIdx.y, blockIdx.y,
+                       threadIdx.x);
 }
 
 // g state of the reduced form as post-streaming FP64 rows [i0, i1):
@@ -195,8 +197,8 @@ int blocks_per_sm(K kernel, int threads, int smem, std::atomic<int> &cache, int 
     return LB_OK;
 }
 
-// z run of the phi pass: the launch's choice, else 8..64 planes, as long as
-// about three waves of resident blocks remain
+// z run of the phi pass: the launch's choice, else by the resident blocks
+// (phi_run_length)
 int phi_z_run(lb_ctx *c, long long columns, int bps, int *kzc)
 {
     int z = c->z_chunk;
@@ -205,9 +207,7 @@ int phi_z_run(lb_ctx *c, long long columns, int bps, int *kzc)
         int rc = cuda_status(cudaGetDevice(&dev));
         if (!rc) rc = cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         if (rc) return rc;
-        const long long want = 3LL * sms * bps;
-        const long long zz = (long long)c->p.nz * columns / (want > 0 ? want : 1);
-        z = zz < 8 ? 8 : (zz > 64 ? 64 : (int)zz);
+        z = phi_run_length(columns, c->p.nz, (long long)sms * bps);
     }
     *kzc = z > c->p.nz ? c->p.nz : z;
     return LB_OK;
@@ -226,12 +226,12 @@ struct T1Passes {
         c = ctx;
         const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
         const int warps = block_warps ? block_warps : kPhiWarps;
-        const unsigned gx = (nx + kPhiOut - 1) / kPhiOut, gy = (ny + KY * warps - 1) / (KY * warps);
+        const int gxy = phi_blocks(nx, ny, KY, warps);
         static std::atomic<int> cache[kPhiMaxWarps + 1];
         int bps = 0;
         int rc = blocks_per_sm(k_t1_phi<T, KY>, 32 * warps, 0, cache[warps], &bps);
-        if (!rc) rc = phi_z_run(c, (long long)gx * gy, bps, &kzc);
-        pgrid = dim3(gx, gy, (nz + kzc - 1) / (kzc ? kzc : 1));
+        if (!rc) rc = phi_z_run(c, gxy, bps, &kzc);
+        pgrid = dim3(gxy, (nz + kzc - 1) / (kzc ? kzc : 1));
         pblock = dim3(32, warps);
         return rc;
     }
@@ -274,10 +274,17 @@ int run_t1(lb_ctx *c, int nsteps)
     return LB_OK;
 }
 
+// y rows a lane of the phi pass in FP32: two from 2^20 sites on (us a step:
+// 128^3 68.2 against 70.1, 256^3 513 / 529, 200x152x136 131.2 / 137.1; below,
+// one: 129x97x65 31.5 / 31.0, 96^3 33.4 / 33.5), one where the lattice has
+// fewer than four rows (1024x1x1024 51 / 43).
+int phi_rows(const lb_ctx *c) { return c->N >= (1LL << 20) && c->p.ny >= 4 ? 2 : 1; }
+
 template <typename T, bool SH, int NP>
 int run_t1_ky(lb_ctx *c, int nsteps)
 {
-    switch (c->block_x ? c->block_x : PhiTile<T>::KY) {
+    const int rows = std::is_same<T, float>::value ? phi_rows(c) : PhiTile<T>::KY;
+    switch (c->block_x ? c->block_x : rows) {
     case 1: return run_t1<T, SH, NP, 1>(c, nsteps);
     case 2: return run_t1<T, SH, NP, 2>(c, nsteps);
     case 4:
@@ -389,11 +396,6 @@ static int run_geq_np(lb_ctx *c, int nsteps)
 // form's phi pass has more; they take the two passes.
 constexpr long long kGeqMinSites = (1LL << 18) + 1;
 constexpr int kGeqMinRow = 12;
-// Two y rows a lane in the phi pass from 2^20 sites on (128^3 74.1 against
-// 75.5 us, 256^3 527 / 531, 300^3 838 / 874; 96^3 36.7 / 34.6: one row there,
-// for more warps), one where the lattice has fewer than four rows
-// (1024x1x1024 51 / 43).
-constexpr long long kGeqTwoRowSites = 1LL << 20;
 
 bool auto_uses_geq(const lb_ctx *c)
 {
@@ -403,7 +405,7 @@ bool auto_uses_geq(const lb_ctx *c)
 
 int launch_step_geq(lb_ctx *c, int nsteps)
 {
-    return c->N >= kGeqTwoRowSites && c->p.ny >= 4 ? run_geq_np<2>(c, nsteps) : run_geq_np<1>(c, nsteps);
+    return phi_rows(c) == 2 ? run_geq_np<2>(c, nsteps) : run_geq_np<1>(c, nsteps);
 }
 
 int taug1_validate(const lb_params &p, int block_x, int block_y, int z_chunk)

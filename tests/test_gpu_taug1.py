@@ -99,6 +99,25 @@ def test_rejected_unless_tau_g_is_one():
             lat.set_kernel("taug1")
 
 
+# the phi pass takes the rows as a stream with halo positions between them,
+# 30 outputs a warp: rows around one, two and no warps' length, lattices of
+# fewer rows than a CTA holds, the last warp partly filled
+@pytest.mark.parametrize("rows,warps", [(1, 4), (2, 8), (4, 1)])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (2, 3, 2), (3, 37, 2), (28, 5, 3), (29, 4, 4), (30, 9, 2), (31, 2, 3),
+                                  (62, 7, 5), (131, 3, 4)])
+def test_reduced_form_row_lengths(dims, rows, warps):
+    from paper_1405_6162_gb300 import Lattice
+    phi0 = L.spinodal_phi0(*dims, seed=325, amp=0.3)
+    u0 = 0.02 * L.uniform(326, 3 * phi0.size, -1, 1).reshape(3, -1)
+    fo, go = oracle.step(dims, P0, *oracle.init(dims, P0, phi0, u0), 3)
+    with Lattice.from_params(dims, P0, precision="fp64") as lat:
+        lat.set_kernel("taug1", rows, warps, 2)
+        lat.init(phi0, u0)
+        lat.step(3)
+        f, g = lat.get_state()
+    assert rel(to_oracle(f), fo) <= TOL_FP64 and rel(to_oracle(g), go) <= TOL_FP64
+
+
 TOL_FP32_PER_STEP = {"rho": 2.5e-8, "u": 2.5e-8, "phi": 1e-7}
 
 
