@@ -545,10 +545,10 @@ int lb_set_state(lb_ctx *c, const double *f, const double *g, int ptr_kind)
     return rc;
 }
 
-// Device mask and the compaction offsets of the selected sites; *total
-// receives their number (synchronises the stream).
+// Device mask, the compaction offsets and (index) the list of the selected
+// sites; *total receives their number (synchronises the stream).
 static int masked_prepare(lb_ctx *c, const unsigned char *mask, int ptr_kind, const unsigned char **mask_d,
-                          long long *total)
+                          long long *total, bool index)
 {
     // the compaction buffers (and, for a host mask, its device copy) are
     // allocated on first use; a failure keeps nothing allocated by this call
@@ -574,11 +574,12 @@ static int masked_prepare(lb_ctx *c, const unsigned char *mask, int ptr_kind, co
     } else {
         *mask_d = mask;
     }
-    if (!rc) rc = lbk::launch_mask_scan(c, *mask_d, c->mask_scratch);
-    int tot = 0;
-    if (!rc) rc = copy(c, &tot, c->mask_scratch + lbk::masked_total_offset(c->N), sizeof(int), cudaMemcpyDeviceToHost);
-    if (!rc) rc = sync(c);
-    *total = tot;
+    if (!rc) rc = lbk::launch_mask_scan(c, *mask_d, c->mask_scratch, index);
+    int res[2] = {0, 0};   // the total, the flag of bounded waits
+    if (!rc) rc = copy(c, res, c->mask_scratch + lbk::masked_total_offset(c->N), sizeof(res), cudaMemcpyDeviceToHost);
+    if (!rc) rc = lbk::cuda_status(cudaStreamSynchronize(c->stream));
+    if (!rc && res[1]) rc = sync(c);   // reports and clears it
+    *total = res[0];
     return rc;
 }
 
@@ -588,7 +589,7 @@ int lb_moments_masked(lb_ctx *c, const unsigned char *mask, double *rho, double 
     if (!c || !mask || (ptr_kind != LB_HOST && ptr_kind != LB_DEVICE)) return LB_ERR_INVALID;
     const unsigned char *mask_d = nullptr;
     long long total = 0;
-    int rc = masked_prepare(c, mask, ptr_kind, &mask_d, &total);
+    int rc = masked_prepare(c, mask, ptr_kind, &mask_d, &total, rho || u || phi);
     if (rc) return rc;
     if (count) *count = total;
     if (total == 0 || (!rho && !u && !phi)) return LB_OK;
@@ -618,7 +619,7 @@ static int masked_state(lb_ctx *c, const unsigned char *mask, double *f, double 
     if (!c || !mask || (ptr_kind != LB_HOST && ptr_kind != LB_DEVICE) || c->reduced) return LB_ERR_INVALID;
     const unsigned char *mask_d = nullptr;
     long long total = 0;
-    int rc = masked_prepare(c, mask, ptr_kind, &mask_d, &total);
+    int rc = masked_prepare(c, mask, ptr_kind, &mask_d, &total, true);
     if (rc) return rc;
     if (count) *count = total;
     if (total == 0) return LB_OK;

@@ -82,8 +82,10 @@ __device__ __forceinline__ int warp_incl(int x)
     return x;
 }
 
-// offsets[i] = counts[0] + ... + counts[i - 1] for i < nb, offsets[nb] = total
+// offsets[i] = counts[0] + ... + counts[i - 1] for i < nb, offsets[nb] = total,
+// offsets[nb + 1] = the flag of bounded waits, read back with it
 __global__ void __launch_bounds__(kMaskThreads) k_mask_scan(const int *__restrict__ counts, int nb,
+                                                            const unsigned int *__restrict__ err,
                                                             int *__restrict__ offsets)
 {
     __shared__ int warp_tot[32];
@@ -108,7 +110,10 @@ __global__ void __launch_bounds__(kMaskThreads) k_mask_scan(const int *__restric
         if (threadIdx.x == 0) carry_s = carry + warp_tot[kMaskWarps - 1];
         __syncthreads();
     }
-    if (threadIdx.x == 0) offsets[nb] = carry_s;
+    if (threadIdx.x == 0) {
+        offsets[nb] = carry_s;
+        offsets[nb + 1] = *err != 0;
+    }
 }
 
 // idx[k] = site of the k-th selected site (site order): each thread's 16
@@ -202,20 +207,21 @@ inline unsigned gather_blocks(long long total) { return (unsigned)((total + kGat
 
 }  // namespace
 
-// scratch: counts [nb], offsets [nb + 1], site indices [N]
-size_t masked_scratch_ints(long long N) { return 2 * (size_t)mask_blocks(N) + 1 + (size_t)N; }
+// scratch: counts [nb], offsets [nb + 1], flag of bounded waits, site indices [N]
+size_t masked_scratch_ints(long long N) { return 2 * (size_t)mask_blocks(N) + 2 + (size_t)N; }
 
-// counts, offsets and site indices of the selected sites
-int launch_mask_scan(lb_ctx *c, const unsigned char *mask_d, int *scratch)
+// counts and offsets of the selected sites, and (index) their site indices
+int launch_mask_scan(lb_ctx *c, const unsigned char *mask_d, int *scratch, bool index)
 {
     const int nb = mask_blocks(c->N);
-    int *counts = scratch, *offsets = scratch + nb, *idx = scratch + 2 * nb + 1;
+    int *counts = scratch, *offsets = scratch + nb, *idx = scratch + 2 * nb + 2;
     const bool vec = ((unsigned long long)mask_d & 15) == 0;
     if (vec)
         k_mask_count<true><<<nb, kTileThreads, 0, c->stream>>>(mask_d, c->N, counts);
     else
         k_mask_count<false><<<nb, kTileThreads, 0, c->stream>>>(mask_d, c->N, counts);
-    k_mask_scan<<<1, kMaskThreads, 0, c->stream>>>(counts, nb, offsets);
+    k_mask_scan<<<1, kMaskThreads, 0, c->stream>>>(counts, nb, c->err_flag, offsets);
+    if (!index) return check_launch();
     if (vec)
         k_mask_index<true><<<nb, kTileThreads, 0, c->stream>>>(mask_d, c->N, offsets, idx);
     else
@@ -223,12 +229,12 @@ int launch_mask_scan(lb_ctx *c, const unsigned char *mask_d, int *scratch)
     return check_launch();
 }
 
-int masked_total_offset(long long N) { return 2 * mask_blocks(N); }   // index of offsets[nb] in the scratch
+int masked_total_offset(long long N) { return 2 * mask_blocks(N); }   // index of offsets[nb], the flag after it, in the scratch
 
 int launch_masked_moments(lb_ctx *c, long long total, const int *scratch, double *rho, double *u, double *phi)
 {
     if (total <= 0) return LB_OK;
-    const int *idx = scratch + 2 * mask_blocks(c->N) + 1;
+    const int *idx = scratch + 2 * mask_blocks(c->N) + 2;
     const int cur = c->buf.cur;
     const double hF[3] = {0.5 * c->force[0], 0.5 * c->force[1], 0.5 * c->force[2]};
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
@@ -251,7 +257,7 @@ int launch_masked_rows(lb_ctx *c, long long total, const int *scratch, int which
                        int to_device_state)
 {
     if (total <= 0) return LB_OK;
-    const int *idx = scratch + 2 * mask_blocks(c->N) + 1;
+    const int *idx = scratch + 2 * mask_blocks(c->N) + 2;
     const int cur = c->buf.cur;
     const double shift = (which == 0 && c->p.precision == LB_FP32_SHIFTED) ? c->p.rho0 : 0.0;
     void *a = which == 0 ? c->buf.f[cur] : c->buf.g[cur];
