@@ -6,6 +6,7 @@
 // per-site quantity here gathers A_i from x - c_i.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "d3q19.cuh"
@@ -243,6 +244,10 @@ __device__ __forceinline__ void add_sites(const T *__restrict__ fa, const T *__r
         for (int v = 0; v < V; v++) gs[i % GS].add(g[i].v[v]);
 }
 
+// sites of a thread's load
+template <typename T>
+constexpr int kReduceSites = std::is_same<T, float>::value ? 2 : 1;
+
 // Per-block partial totals.  A thread sums each of the 19 f rows over its
 // sites (sum_x A_i(x)), and the g rows (G rows: 19, or 1 in the tau_g = 1
 // reduced form, whose row 0 holds phi) into a few partial sums, as only their
@@ -266,7 +271,7 @@ __global__ void __launch_bounds__(kReduceThreads, 2) k_reduce(const T *__restric
                                                               double offset0, const unsigned int *err, ReduceOut *out)
 {
     constexpr int GS = G_ROWS < 4 ? G_ROWS : 4;   // partial sums of g
-    constexpr int V = std::is_same<T, float>::value ? 2 : 1;
+    constexpr int V = kReduceSites<T>;
     const long long stride = (long long)gridDim.x * blockDim.x, first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     RowSum<T> fs[Q], gs[GS];
 #pragma unroll
@@ -435,7 +440,13 @@ int launch_reduce(lb_ctx *c)
         using T = typename decltype(P)::T;
         const T *fa = (const T *)c->buf.f[cur], *ga = (const T *)c->buf.g[cur];
         const auto kernel = c->reduced ? k_reduce<T, 1> : k_reduce<T, Q>;
-        kernel<<<kReduceBlocks, kReduceThreads, 0, c->stream>>>(fa, ga, c->N, c->S, c->partial, off, c->err_flag,
+        // no CTA without a site: forming and adding a thread's totals is some
+        // 70 FP64 additions, which on small lattices are most of the work
+        // (70x37x11 FP64, a step and its totals: 3 us less of 60
+        // with its 112 CTAs than with 304)
+        const long long per = kReduceThreads * kReduceSites<T>;
+        const int grid = (int)std::min<long long>(kReduceBlocks, (c->N + per - 1) / per);
+        kernel<<<grid, kReduceThreads, 0, c->stream>>>(fa, ga, c->N, c->S, c->partial, off, c->err_flag,
                                                                 c->dev_out);
         return check_launch();
     });
