@@ -38,6 +38,9 @@ BYTES_PER_SITE = {"fp32_shifted": 4 * 19 * 4, "fp64": 4 * 19 * 8}   # read+write
 # tau_g = 1 reduced form: collide reads f (19) + phi, writes f (19) + (gmh, u) (4);
 # the phi pass reads phi + (gmh, u) and writes phi -- 49 words per site
 BYTES_PER_SITE_TAUG1 = {"fp32_shifted": 49 * 4, "fp64": 49 * 8}
+# the library default with tau_g = 1: in FP32 the steps of one call keep g as
+# its moments (49 words); FP64 stores all of it
+BYTES_PER_SITE_DEFAULT = {"fp32_shifted": 49 * 4, "fp64": 4 * 19 * 8}
 METRIC = "MLUPS and % of HBM roofline (fused step), FP32-shifted vs FP64 at stated error"
 ORACLE_SAMPLE = (64, 64, 64)
 ORACLE_STEPS = 30
@@ -335,7 +338,7 @@ def _ensemble(torch, with_oracle=True):
         info = b.info()
         out = {"lattices": len(specs), "sites": b.sites, "steps": 500, "seconds": t,
                "MLUPS": b.sites * 500 / t / 1e6, "precision": "fp32_shifted",
-               "hbm_frac": b.sites * 500 * BYTES_PER_SITE["fp32_shifted"] / t / 1e9 / _peaks()[0],
+               "hbm_frac": b.sites * 500 * BYTES_PER_SITE_DEFAULT["fp32_shifted"] / t / 1e9 / _peaks()[0],
                "launch": {"threads": info[3], "ctas": info[2], "work_items": info[1], "plan": b.plan,
                           "groups": b.groups()},
                "graph_replays": 1}
@@ -749,7 +752,7 @@ def run_ours(args):
 
     def stencil_for(npts, prec):
         r = stencils[(npts, prec)]
-        achieved = BYTES_PER_SITE[prec] * n / r["t_step"] / 1e9
+        achieved = BYTES_PER_SITE_DEFAULT[prec] * n / r["t_step"] / 1e9
         out = {"value": ws * n * r["steps"] / r["wall"] / 1e6, "unit": "MLUPS", "steps": r["steps"],
                "ms_per_step": r["wall"] / r["steps"] * 1e3, "clocks": r["clocks"],
                "hbm_frac": achieved / peak, "achieved_gbs": achieved}
@@ -763,7 +766,7 @@ def run_ours(args):
 
     def mrt_for(prec):
         r = mrt[prec]
-        achieved = BYTES_PER_SITE[prec] * n / r["t_step"] / 1e9
+        achieved = BYTES_PER_SITE_DEFAULT[prec] * n / r["t_step"] / 1e9
         out = {"value": ws * n * r["steps"] / r["wall"] / 1e6, "unit": "MLUPS", "steps": r["steps"],
                "ms_per_step": r["wall"] / r["steps"] * 1e3, "clocks": r["clocks"],
                "hbm_frac": achieved / peak, "achieved_gbs": achieved}
@@ -776,10 +779,10 @@ def run_ours(args):
         return out
 
     def reduce_for(prec):
-        # lb_reduce is bound by the FP64 pipe: FP64 additions per site from
-        # ncu counters against the measured FP64 FMA-instruction rate (the
-        # probe's TFLOP/s over 2); the HBM fraction of its 38 stored words
-        # a site is given beside it
+        # lb_reduce: FP32 storage is summed on the FP32 units and bound by the
+        # 38 stored words a site; FP64 storage by the FP64 pipe: additions per
+        # site from ncu counters against the measured FP64 FMA-instruction
+        # rate (the probe's TFLOP/s over 2)
         t = results[prec]["t_reduce"]
         adds = _profile_value("reduce_128cubed", f"fp64_adds_per_site_{prec}")
         pk = fp64_peak["tflops"]
@@ -787,14 +790,15 @@ def run_ours(args):
         ach = adds * n / t / 1e12 if adds else None
         tr = _profile_value("reduce_128cubed", f"dram_bytes_per_site_{prec}")
         return {"ms_per_call": t * 1e3, "sites_per_s": n / t,
-                "roofline": {"bound": "alu (FP64 pipe)", "kernel": "k_reduce", "achieved": ach,
+                "roofline": {"bound": "hbm" if prec == "fp32_shifted" else "alu (FP64 pipe)", "kernel": "k_reduce",
+                             "achieved": ach,
                              "peak": pk / 2 if pk else None, "unit": "T FP64 instructions/s",
                              "frac": ach / (pk / 2) if (ach and pk) else None, "fp64_adds_per_site": adds,
                              "peak_kind": "measured in this run: FMA instructions/s of lb_probe_fp64_fma",
                              "achieved_gbs": gbs, "hbm_frac": gbs / peak,
                              "traffic": tr * n if tr else None,
-                             "timing": "median of 10 calls, CUDA events around each (both kernels, the "
-                                       "40-byte read-back and the return)"}}
+                             "timing": "median of 10 calls, CUDA events around each (the kernel, the "
+                                       "48-byte read-back and the return)"}}
 
     def df_line():
         r = df
@@ -838,7 +842,7 @@ def run_ours(args):
                     **df_line()},
         "lattice_128": {"what": "the 128^3 spinodal lattice (seed 1), default step", **l128},
         "mrt": {"what": f"multiple-relaxation-time collision of f (lb_set_collision), tau = 1, "
-                        f"tau_bulk = {MRT_RATES[0]}, tau_ghost = {MRT_RATES[1]}, on the default two-pass step",
+                        f"tau_bulk = {MRT_RATES[0]}, tau_ghost = {MRT_RATES[1]}, on the library default step; hbm_frac over 49 words a site in FP32 (tau_g = 1), 76 in FP64",
                 "fp32_shifted": mrt_for("fp32_shifted"), "fp64": mrt_for("fp64")},
         "reductions": {"what": "lb_reduce: FP64 totals of rho, rho u and phi over the 256^3 lattice of each "
                                "precision after the timed steps",
@@ -847,8 +851,8 @@ def run_ours(args):
                                    "random site mask on the 256^3 FP32 lattice, device outputs, one call "
                                    "includes the read-back of the count",
                            **masked},
-        "stencils": {"what": "isotropic 19- / 27-point phi stencils (lb_set_stencil) on the default "
-                             "two-pass step; hbm_frac over the same 76-word algorithmic bytes",
+        "stencils": {"what": "isotropic 19- / 27-point phi stencils (lb_set_stencil) on the library default "
+                             "step; hbm_frac over 49 words a site in FP32 (tau_g = 1), 76 in FP64",
                      **{f"{npts}pt": {prec: stencil_for(npts, prec) for prec in ("fp32_shifted", "fp64")}
                         for npts in (19, 27)}},
         "autotune": {"what": "kernel and launch shape of the headline (fp32_shifted) and of the fp64 line, "
