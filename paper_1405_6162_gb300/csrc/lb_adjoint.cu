@@ -147,7 +147,7 @@ __device__ __forceinline__ double block_sum_d(double v, double *sh)
     return r;
 }
 
-constexpr int kAdjThreads = 256;
+constexpr int kAdjThreads = 256;   // at most; k_phi_local and k_adj_collide run fp64_threads(N), like the FP64 step
 
 // phi(x) = sum_i g_i(x) of a post-streaming state
 __global__ void __launch_bounds__(kAdjThreads) k_phi_local(const double *__restrict__ g, double *__restrict__ phi,
@@ -171,8 +171,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_phi_local(const double *__restr
 // Bound by the FP64 pipe (2 lanes a clock per SM), so written for few FP64
 // instructions: weight_sums, one reciprocal of rho instead of eleven
 // divisions, rates folded into the factors.  64^3, tau = tau_g = 1: a reverse
-// step 0.40 -> 0.17 ms, the gradient through 200 steps 138.3 -> 92.6 ms.
-// Two CTAs an SM: the FP64 pipe is full with 16 warps.
+// step 0.40 -> 0.17 ms (168 us at 192 threads, 175 at 256), the gradient
+// through 200 steps 138.3 -> 92.6 ms.
+// Two CTAs of 256 an SM: the FP64 pipe is full with 16 warps.
 template <bool INIT, bool KEEP_F, bool KEEP_G>
 __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_collide(const double *__restrict__ f,
                                                                 const double *__restrict__ phi,
@@ -255,14 +256,14 @@ __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_collide(const double *__
 // (fixed order) to *dkappa.
 template <bool INIT, bool KEEP_G>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_stencil(const double *__restrict__ aux, double *__restrict__ out,
-                                                             const double *__restrict__ kpart,
+                                                             const double *__restrict__ kpart, int nparts,
                                                              double *__restrict__ dkappa, int nx, int ny, int nz)
 {
     pdl_wait_then_release();
     if (blockIdx.x == 0) {
         __shared__ double sh[kAdjThreads / 32];
         double v = 0.0;
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) v += kpart[b];
+        for (int b = threadIdx.x; b < nparts; b += blockDim.x) v += kpart[b];
         const double tot = block_sum_d(v, sh);
         if (threadIdx.x == 0) *dkappa += tot;
     }
@@ -326,6 +327,8 @@ AdjP adj_params(const lb_params &q, double w, double wg)
     return p;
 }
 
+int full_blocks(long long N) { return (int)((N + kAdjThreads - 1) / kAdjThreads); }
+
 // the collision's and the stencils' kernels of a reverse step
 template <bool KEEP_F, bool KEEP_G>
 cudaError_t reverse_step(lb_ctx *c, const double *f, const double *phi, const double *af_in, const double *ag_in,
@@ -334,23 +337,29 @@ cudaError_t reverse_step(lb_ctx *c, const double *f, const double *phi, const do
     const int nb = adjoint_blocks(c->N);
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     const AdjP p = adj_params(c->p, 1.0 / c->p.tau, 1.0 / c->p.tau_g);
-    cudaError_t e = launch_pdl(k_adj_collide<false, KEEP_F, KEEP_G>, nb, kAdjThreads, c->stream, f, phi,
+    cudaError_t e = launch_pdl(k_adj_collide<false, KEEP_F, KEEP_G>, nb, fp64_threads(c->N), c->stream, f, phi,
                                (const double *)nullptr, af_in, ag_in, af_out, ag_out, aux, kpart, p, nx, ny, nz);
     if (e == cudaSuccess)
-        e = launch_pdl(k_adj_stencil<false, KEEP_G>, nb, kAdjThreads, c->stream, (const double *)aux, ag_out,
-                       (const double *)kpart, dkappa, nx, ny, nz);
+        e = launch_pdl(k_adj_stencil<false, KEEP_G>, full_blocks(c->N), kAdjThreads, c->stream, (const double *)aux,
+                       ag_out, (const double *)kpart, nb, dkappa, nx, ny, nz);
     return e;
 }
 
 }  // namespace
 
-int adjoint_blocks(long long N) { return (int)((N + kAdjThreads - 1) / kAdjThreads); }
+// CTAs of k_adj_collide, each with a partial dJ/dkappa
+int adjoint_blocks(long long N)
+{
+    const int tpb = fp64_threads(N);
+    return (int)((N + tpb - 1) / tpb);
+}
 
 int launch_adjoint_step(lb_ctx *c, const double *f, const double *g, const double *af_in, const double *ag_in,
                         double *af_out, double *ag_out, double *dkappa, double *aux, double *kpart)
 {
     double *phi = aux + 5 * c->N;
-    cudaError_t e = launch_pdl(k_phi_local, adjoint_blocks(c->N), kAdjThreads, c->stream, g, phi, (long long)c->N);
+    cudaError_t e =
+        launch_pdl(k_phi_local, adjoint_blocks(c->N), fp64_threads(c->N), c->stream, g, phi, (long long)c->N);
     if (e == cudaSuccess) {
         const auto step = c->p.tau == 1.0 ? (c->p.tau_g == 1.0 ? reverse_step<false, false> : reverse_step<false, true>)
                                           : (c->p.tau_g == 1.0 ? reverse_step<true, false> : reverse_step<true, true>);
@@ -361,7 +370,7 @@ int launch_adjoint_step(lb_ctx *c, const double *f, const double *g, const doubl
 
 int launch_adjoint_seed(lb_ctx *c, const double *phi_bar, double *af, double *ag)
 {
-    k_adj_seed<<<adjoint_blocks(c->N), kAdjThreads, 0, c->stream>>>(phi_bar, af, ag, c->N);
+    k_adj_seed<<<full_blocks(c->N), kAdjThreads, 0, c->stream>>>(phi_bar, af, ag, c->N);
     return check_launch();
 }
 
@@ -371,11 +380,12 @@ int launch_adjoint_init(lb_ctx *c, const double *phi0, const double *u0, const d
     const int nb = adjoint_blocks(c->N);
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     double *none = nullptr;
-    cudaError_t e = launch_pdl(k_adj_collide<true, false, false>, nb, kAdjThreads, c->stream, (const double *)none, phi0,
-                               u0, af0, ag0, none, none, aux, kpart, adj_params(c->p, 1.0, 1.0), nx, ny, nz);
+    cudaError_t e = launch_pdl(k_adj_collide<true, false, false>, nb, fp64_threads(c->N), c->stream,
+                               (const double *)none, phi0, u0, af0, ag0, none, none, aux, kpart,
+                               adj_params(c->p, 1.0, 1.0), nx, ny, nz);
     if (e == cudaSuccess)
-        e = launch_pdl(k_adj_stencil<true, false>, nb, kAdjThreads, c->stream, (const double *)aux, phi0_bar,
-                       (const double *)kpart, dkappa, nx, ny, nz);
+        e = launch_pdl(k_adj_stencil<true, false>, full_blocks(c->N), kAdjThreads, c->stream, (const double *)aux,
+                       phi0_bar, (const double *)kpart, nb, dkappa, nx, ny, nz);
     return e != cudaSuccess ? cuda_status(e) : check_launch();
 }
 

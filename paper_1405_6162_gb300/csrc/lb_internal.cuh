@@ -147,6 +147,9 @@ int fused_validate(int precision, int block_x, int block_y, int z_chunk);
 int launch_step_staged(lb_ctx *c, int nsteps);
 int staged_validate(int precision, int block_x, int block_y, int z_chunk);
 
+// threads per CTA of FP64-bound kernels over N sites (lb_kernels.cu)
+int fp64_threads(long long N);
+
 // adjoint (lb_adjoint.cu)
 int adjoint_blocks(long long N);
 int launch_adjoint_step(lb_ctx *c, const double *f, const double *g, const double *af_in, const double *ag_in,

@@ -135,6 +135,8 @@ static int default_threads(long long N)
     return busiest(192) < busiest(128) ? 192 : 128;
 }
 
+int fp64_threads(long long N) { return default_threads<double>(N); }
+
 // the phi pass with V sites per thread
 template <typename T>
 static cudaError_t launch_phi(lb_ctx *c, const T *ga, T *phi, int tpb, int vvl)
