@@ -147,7 +147,10 @@ __device__ __forceinline__ double block_sum_d(double v, double *sh)
     return r;
 }
 
-constexpr int kAdjThreads = 256;   // at most; k_phi_local and k_adj_collide run fp64_threads(N), like the FP64 step
+// At most: k_phi_local and k_adj_collide run fp64_threads(N), like the FP64
+// step.  A reverse step at 256 threads and so: 12^3 28.4 -> 16.6 us, 32^3 31.6
+// -> 27.2, 48x40x44 77.3 -> 66.7, 64^3 174.4 -> 168.4, 80^3 332 -> 322.
+constexpr int kAdjThreads = 256;
 
 // phi(x) = sum_i g_i(x) of a post-streaming state
 __global__ void __launch_bounds__(kAdjThreads) k_phi_local(const double *__restrict__ g, double *__restrict__ phi,
