@@ -66,9 +66,20 @@ def _keep(n, nsteps, segment):
     return int(segment), _States(n, -(-nsteps // int(segment)))
 
 
+def _steps(nsteps, segment):
+    """Steps to take.  A negative count without a segment, and a segment that
+    takes no step of some, are refused before anything is allocated."""
+    if not segment and nsteps < 0:
+        raise ValueError(f"nsteps = {nsteps} is negative")
+    if segment and int(segment) < 1 and nsteps > 0:
+        raise L.LBError(L.LB_ERR_INVALID, f"trajectory in segments of {segment} steps")
+    return max(nsteps, 0)
+
+
 class LBTrajectory(torch.autograd.Function):
     @staticmethod
     def forward(ctx, phi0, kappa, dims, params, nsteps, segment, keep=True):
+        nsteps = _steps(nsteps, segment)
         p = dict(params)
         p["kappa"] = float(kappa)
         lat, lib = Lattice.from_params(dims, p, precision="fp64"), L.lib()
