@@ -80,9 +80,9 @@ enum { LB_HOST = 0, LB_DEVICE = 1 };
 enum {
     LB_KERNEL_AUTO = 0,     /* library default, the fastest measured on GB300.
                                FP32-shifted with tau_g = 1, more than 2^18
-                               sites and rows of 12 or more: within one
-                               lb_step call g is kept as its equilibrium's
-                               moments, and written in full by the last step.
+                               sites and rows of 12 or more: between steps
+                               g is kept as its equilibrium's moments; the
+                               last step of a call writes it in full as well.
                                Else LB_KERNEL_BULK (3 slots, clusters of 2,
                                16 planes) for FP32-shifted 7-point BGK steps
                                with tau_g != 1 on rows of 256 sites with ny
@@ -177,6 +177,7 @@ int lb_init(lb_ctx *c, const double *phi0, const double *u0, int ptr_kind);
  *               + 9/2 ((Gamma mu - phi/3) I + phi u u):(c_i c_i - I/3)];
  *   f*_i = f_i - (f_i - feq_i)/tau;  g*_i = g_i - (g_i - geq_i)/tau_g;
  *   f_i(x + c_i, t+1) = f*_i(x, t), likewise g (periodic wrap).
+ * The bits of a run do not depend on how its steps are divided into calls.
  * Errors: LB_ERR_INVALID (c NULL, nsteps < 0), LB_ERR_CUDA.
  * Paper: the binary-collision benchmark, Sec. IV; TARGET_LAUNCH, Sec. III.C. */
 int lb_step(lb_ctx *c, int nsteps);

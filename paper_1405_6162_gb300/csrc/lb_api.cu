@@ -218,6 +218,7 @@ int lb_create(const lb_params *p, void *cuda_stream, lb_ctx **out)
     c->dev_out = (lbk::ReduceOut *)dev_alloc(c, sizeof(lbk::ReduceOut));
     c->lag_counters = (unsigned long long *)dev_alloc(c, (size_t)(p->nz + 1) * sizeof(unsigned long long));
     c->err_flag = (unsigned int *)dev_alloc(c, sizeof(unsigned int));
+    if (c->dev_out && lbk::auto_uses_geq(c)) c->moments = &c->dev_out->moments;
     bool ok = c->phi && c->partial && c->dev_out && c->lag_counters && c->err_flag;
     for (int k = 0; k < 2; k++) ok = ok && c->buf.f[k] && c->buf.g[k];
     if (!ok) {
@@ -352,6 +353,8 @@ int lb_step(lb_ctx *c, int nsteps)
     if (c->kernel == LB_KERNEL_AUTO && lbk::auto_uses_geq(c)) return lbk::launch_step_geq(c, nsteps);
     if (c->kernel == LB_KERNEL_AUTO && lbk::auto_uses_bulk(c)) return lbk::launch_step_bulk_auto(c, nsteps);
     if (c->kernel == LB_KERNEL_TWO_PASS || c->kernel == LB_KERNEL_AUTO) return lbk::launch_step_two_pass(c, nsteps);
+    const int rc = lbk::state_written(c);   // (the two passes' first kernel does it for them)
+    if (rc) return rc;
     if (c->kernel == LB_KERNEL_STAGED) return lbk::launch_step_staged(c, nsteps);
     if (c->kernel == LB_KERNEL_SLAB) return lbk::launch_step_slab(c, nsteps);
     if (c->kernel == LB_KERNEL_LAG) return lbk::launch_step_lag(c, nsteps);

@@ -785,7 +785,6 @@ int lb_batch_set_form(lb_batch *b, int reduced)
     int rc = batch_sync(b);
     for (lb_ctx *c : b->ctx) {
         if (!rc) rc = lbk::taug1_convert(c, reduced);
-        if (!rc) rc = lbk::state_written(c);
         if (!rc) c->reduced = reduced;
     }
     if (!rc) rc = lbk::cuda_status(cudaStreamSynchronize(b->user_stream));

@@ -31,6 +31,7 @@ struct ReduceOut {
     double totals[5];           // sum rho, sum rho u, sum phi
     unsigned int wait_failed;   // *err_flag when the totals were formed
     unsigned int ticket;        // CTAs of the reduction that are done; 0 between calls
+    int moments;                // lb_ctx::moments of a lattice of its own
 };
 
 }  // namespace lbk
@@ -55,7 +56,9 @@ struct lb_ctx {
     double *adj = nullptr;        // [6N] adjoint scratch (lazy): phi_bar, d_bar (3), lap_bar, phi
     double *adj_part = nullptr;   // per-CTA partial dJ/dkappa
     int batch_owned = 0;  // member of an lb_batch: stepped and freed by it
-    int *moments = nullptr;   // member of an lb_batch: device flag, the last step's phi and quads are at hand
+    // device flag, the last step's phi and quads are at hand (LB_KERNEL_AUTO
+    // steps that keep g as moments, lb_taug1.cu; members of an lb_batch)
+    int *moments = nullptr;
     int reduced = 0;      // tau_g = 1 form: g kept as phi and (gmh, u), see lb_taug1.cu
     int m_valid = 0;      // reduced form: the previous step's (gmh, u) are present
     int npts = 7;         // points of the phi stencil: 7, 19 or 27 (lb_set_stencil)
@@ -111,8 +114,8 @@ constexpr int kReduceThreads = 256;
 
 // ensemble membership (lb_api.cu): the member shares the batch's error flag
 void adopt_into_batch(lb_ctx *c, unsigned int *shared_err, int *moments);
-// the stored state was written by other than a step: what an ensemble's last
-// run left beside a member's state no longer belongs to it (on the stream)
+// the stored state was written by other than a step that keeps g as moments:
+// what the last such step left beside it no longer belongs to it (on the stream)
 int state_written(lb_ctx *c);
 void release_from_batch(lb_ctx *c);
 
@@ -128,10 +131,6 @@ int two_pass_validate(int block_x, int block_y, int z_chunk);   // threads per C
 // of N doubles supplied by the caller)
 int launch_two_pass_fp64_raw(const lb_params &p, const double *fa, const double *ga, double *phi, double *fb,
                              double *gb, long long S, cudaStream_t stream);
-// the FP32-shifted passes of a step with tau_g = 1: phi of the stored g, and
-// the collide/stream pass that does not read g
-cudaError_t launch_phi_pull(lb_ctx *c, const float *ga, float *phi);
-cudaError_t launch_collide_geq(lb_ctx *c, const float *fa, const float *phi, float *fb, float *gb);
 int launch_moments(lb_ctx *c, double *rho, double *u, double *phi);
 int launch_get_state(lb_ctx *c, double *f, double *g);
 int launch_set_state(lb_ctx *c, const double *f, const double *g);

@@ -23,12 +23,14 @@ namespace lbk {
 
 // phi = sum_i g_i(x - c_i) of V sites per thread (the paper's virtual vector
 // length): the thread's sites are blockDim.x apart, their 19 V loads are
-// issued before any sum
+// issued before any sum.  A step that changes g by these passes takes back the
+// moments flag (lb_ctx::moments, if any): a launch less than a memset
 template <typename T, int V>
 __global__ void __launch_bounds__(256) k_phi_pull(const T *__restrict__ ga, T *__restrict__ phi,
-                                                  int nx, int ny, int nz, long long S)
+                                                  int *__restrict__ moments, int nx, int ny, int nz, long long S)
 {
     pdl_wait_then_release();
+    if (moments && blockIdx.x == 0 && threadIdx.x == 0) *moments = 0;
     const int N = nx * ny * nz;
     const int s0 = blockIdx.x * blockDim.x * V + threadIdx.x;
     T g[V][Q];
@@ -143,9 +145,8 @@ static cudaError_t launch_phi(lb_ctx *c, const T *ga, T *phi, int tpb, int vvl)
 {
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     const unsigned grid = grid_for(c->N, tpb * vvl);
-    if (vvl == 4) return launch_pdl(k_phi_pull<T, 4>, grid, tpb, c->stream, ga, phi, nx, ny, nz, c->S);
-    if (vvl == 2) return launch_pdl(k_phi_pull<T, 2>, grid, tpb, c->stream, ga, phi, nx, ny, nz, c->S);
-    return launch_pdl(k_phi_pull<T, 1>, grid, tpb, c->stream, ga, phi, nx, ny, nz, c->S);
+    const auto kernel = vvl == 4 ? k_phi_pull<T, 4> : vvl == 2 ? k_phi_pull<T, 2> : k_phi_pull<T, 1>;
+    return launch_pdl(kernel, grid, tpb, c->stream, ga, phi, c->moments, nx, ny, nz, c->S);
 }
 
 // the collide/stream pass from level fa, ga (and phi of the state) to fb, gb
@@ -205,26 +206,12 @@ int launch_two_pass_fp64_raw(const lb_params &prm, const double *fa, const doubl
     const long long N = (long long)prm.nx * prm.ny * prm.nz;
     const int tpb = default_threads<double>(N);
     const unsigned grid = grid_for(N, tpb);
-    k_phi_pull<double, 1><<<grid, tpb, 0, stream>>>(ga, phi, prm.nx, prm.ny, prm.nz, S);
+    k_phi_pull<double, 1><<<grid, tpb, 0, stream>>>(ga, phi, nullptr, prm.nx, prm.ny, prm.nz, S);
     const auto collide = !g_is_equilibrium(prm)  ? k_collide_pull<double, false, 7, false, false>
                          : f_is_equilibrium(prm) ? k_collide_pull<double, false, 7, true, true>
                                                  : k_collide_pull<double, false, 7, true, false>;
     collide<<<grid, tpb, 0, stream>>>(fa, ga, phi, fb, gb, p, prm.nx, prm.ny, prm.nz, S);
     return check_launch();
-}
-
-cudaError_t launch_phi_pull(lb_ctx *c, const float *ga, float *phi)
-{
-    return launch_phi<float>(c, ga, phi, c->block_x ? c->block_x : default_threads<float>(c->N), c->block_y ? c->block_y : 1);
-}
-
-cudaError_t launch_collide_geq(lb_ctx *c, const float *fa, const float *phi, float *fb, float *gb)
-{
-    const int tpb = c->block_x ? c->block_x : default_threads<float>(c->N);
-    const float *no_g = nullptr;
-    if (c->npts == 19) return launch_collide<float, true, 19, true>(c, fa, no_g, phi, fb, gb, tpb);
-    if (c->npts == 27) return launch_collide<float, true, 27, true>(c, fa, no_g, phi, fb, gb, tpb);
-    return launch_collide<float, true, 7, true>(c, fa, no_g, phi, fb, gb, tpb);
 }
 
 template <typename T, bool SH>

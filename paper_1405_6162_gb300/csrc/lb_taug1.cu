@@ -62,17 +62,26 @@ k_t1_collide(const T *__restrict__ fa, const T *__restrict__ phi, T *__restrict_
     t1_collide_site<T, SH, NP>(fa, phi, quad, fb, p, nx, ny, nz, S, s);
 }
 
-// the same with the multiple-relaxation-time collision or a body force
-template <typename T, bool SH, int NP>
-__global__ void __launch_bounds__(kT1Threads, sizeof(T) == 8 ? 2 : 3)
-k_t1_collide_mrt(const T *__restrict__ fa, const T *__restrict__ phi, T *__restrict__ quad, T *__restrict__ fb,
-                 Coll<T> p, Mrt<T> m, int nx, int ny, int nz, long long S)
+// The same on a general state (run_geq).  With gb, a call's last step: g* = geq
+// in full as well, phi in the phi buffer (keep, if it is not there) and the
+// flag that quads and phi are at hand.  One kernel for a call's last step and
+// the others, since two kernels' products and sums need not be contracted
+// alike and a run's bits would depend on where its calls end.  MRT: the
+// multiple relaxation times or a body force.
+template <int NP, bool MRT>
+__global__ void __launch_bounds__(kT1Threads, 3)
+k_geq_collide(const float *__restrict__ fa, const float *__restrict__ phi, float *__restrict__ quad,
+              float *__restrict__ fb, float *__restrict__ gb, float *__restrict__ keep, int *__restrict__ moments,
+              Coll<float> p, Mrt<float> m, int nx, int ny, int nz, long long S)
 {
     pdl_wait_then_release();
     const long long N = (long long)nx * ny * nz;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
-    t1_collide_site<T, SH, NP>(fa, phi, quad, fb, p, nx, ny, nz, S, s, &m);
+    t1_collide_site<float, true, NP>(fa, phi, quad, fb, p, nx, ny, nz, S, s, MRT ? &m : nullptr, gb);
+    if (!gb) return;
+    if (keep) keep[s] = phi[s];
+    if (s == 0) *moments = 1;
 }
 
 constexpr int kPhiWarps = 4;      // default warps per block, stacked in y
@@ -86,6 +95,31 @@ __global__ void __launch_bounds__(32 * kPhiMaxWarps) k_t1_phi(const T *__restric
     pdl_wait_then_release();
     t1_phi_tile<T, KY>(phi, quad, phi_out, nx, ny, nz, kzc, blockIdx.x, blockDim.y, threadIdx.y, blockIdx.y,
                        threadIdx.x);
+}
+
+// The phi pass on a general state (run_geq); one kernel for all of a run's, as
+// k_geq_collide.  With ga, a call's first: phi and the quads may not be at hand
+// (*moments), and phi is the sum of the stored g then.  phi_out may be row 0
+// of ga, which only its own site reads (so neither is declared __restrict__).
+// The bounds are the registers that k_t1_phi takes by itself, 64 and 80: with
+// the sum beside it ptxas takes 54 for one row (80^3 20.0 instead of 19.6 us a
+// step), and one CTA in place of 6 costs two rows 4 % (256^3 536 / 516).
+template <int KY>
+__global__ void __launch_bounds__(32 * kPhiWarps, KY == 1 ? 8 : 6)
+k_geq_phi(const float *ga, const int *moments, const float *phi, const float *quad, float *phi_out, int nx, int ny,
+          int nz, int kzc, long long S)
+{
+    pdl_wait_then_release();
+    if (ga && !*moments) {
+        const int N = nx * ny * nz, threads = 32 * blockDim.y;
+        const long long stride = (long long)gridDim.x * gridDim.y * threads;
+        for (long long s = (long long)(blockIdx.y * gridDim.x + blockIdx.x) * threads + threadIdx.y * 32 + threadIdx.x;
+             s < N; s += stride)
+            phi_out[s] = phi_site(ga, Nbr((int)s, nx, ny, nz), S);
+        return;
+    }
+    t1_phi_tile<float, KY>(phi, quad, phi_out, nx, ny, nz, kzc, blockIdx.x, blockDim.y, threadIdx.y, blockIdx.y,
+                           threadIdx.x);
 }
 
 // g state of the reduced form as post-streaming FP64 rows [i0, i1):
@@ -213,59 +247,44 @@ int phi_z_run(lb_ctx *c, long long columns, int bps, int *kzc)
     return LB_OK;
 }
 
-// The two passes of the reduced form for context c: the launch shapes of its
-// phi pass (warps per CTA, z run) worked out once.
-template <typename T, bool SH, int NP, int KY>
-struct T1Passes {
-    lb_ctx *c;
-    dim3 pgrid, pblock;
+// launch shape of a phi pass: KY rows a lane, block_warps warps a CTA (0: the default)
+template <int KY>
+struct PhiLaunch {
+    dim3 grid, block;
     int kzc = 0;
 
-    int plan(lb_ctx *ctx, int block_warps)
+    template <typename K>
+    int plan(lb_ctx *c, K kernel, int block_warps, std::atomic<int> (&cache)[kPhiMaxWarps + 1])
     {
-        c = ctx;
         const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
         const int warps = block_warps ? block_warps : kPhiWarps;
         const int gxy = phi_blocks(nx, ny, KY, warps);
-        static std::atomic<int> cache[kPhiMaxWarps + 1];
         int bps = 0;
-        int rc = blocks_per_sm(k_t1_phi<T, KY>, 32 * warps, 0, cache[warps], &bps);
+        int rc = blocks_per_sm(kernel, 32 * warps, 0, cache[warps], &bps);
         if (!rc) rc = phi_z_run(c, gxy, bps, &kzc);
-        pgrid = dim3(gxy, (nz + kzc - 1) / (kzc ? kzc : 1));
-        pblock = dim3(32, warps);
+        grid = dim3(gxy, (nz + kzc - 1) / (kzc ? kzc : 1));
+        block = dim3(32, warps);
         return rc;
-    }
-    // f of the step into fb, the quads of (mu, u); phi is phi(t)
-    cudaError_t collide(const T *fa, const T *phi, T *quad, T *fb) const
-    {
-        const unsigned grid = grid_of(c->N);
-        const auto p = make_coll<T>(c->p);
-        const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
-        if (uses_mrt(c))
-            return launch_pdl(k_t1_collide_mrt<T, SH, NP>, grid, kT1Threads, c->stream, fa, phi, quad, fb, p,
-                              make_mrt<T>(c), nx, ny, nz, c->S);
-        return launch_pdl(k_t1_collide<T, SH, NP>, grid, kT1Threads, c->stream, fa, phi, quad, fb, p, nx, ny, nz,
-                          c->S);
-    }
-    // phi(t + 1) from phi(t) and the quads
-    cudaError_t next_phi(const T *phi, const T *quad, T *phi_out) const
-    {
-        return launch_pdl(k_t1_phi<T, KY>, pgrid, pblock, c->stream, phi, quad, phi_out, c->p.nx, c->p.ny, c->p.nz,
-                          kzc);
     }
 };
 
 template <typename T, bool SH, int NP, int KY>
 int run_t1(lb_ctx *c, int nsteps)
 {
-    T1Passes<T, SH, NP, KY> pass;
-    int rc = pass.plan(c, c->block_y);
+    static std::atomic<int> cache[kPhiMaxWarps + 1];
+    PhiLaunch<KY> phi;
+    int rc = phi.plan(c, k_t1_phi<T, KY>, c->block_y, cache);
     if (rc) return rc;
+    const auto p = make_coll<T>(c->p);
+    const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     for (int t = 0; t < nsteps; t++) {
         const int a = c->buf.cur, b = 1 - a;
-        T *ga = (T *)c->buf.g[a];
-        cudaError_t e = pass.collide((const T *)c->buf.f[a], ga, quads(ga, c->S), (T *)c->buf.f[b]);
-        if (e == cudaSuccess) e = pass.next_phi(ga, quads(ga, c->S), (T *)c->buf.g[b]);
+        T *ga = (T *)c->buf.g[a], *quad = quads(ga, c->S);   // phi in row 0
+        cudaError_t e = launch_pdl(k_t1_collide<T, SH, NP>, grid_of(c->N), kT1Threads, c->stream,
+                                   (const T *)c->buf.f[a], (const T *)ga, quad, (T *)c->buf.f[b], p, nx, ny, nz, c->S);
+        if (e == cudaSuccess)
+            e = launch_pdl(k_t1_phi<T, KY>, phi.grid, phi.block, c->stream, (const T *)ga, (const T *)quad,
+                           (T *)c->buf.g[b], nx, ny, nz, phi.kzc);
         rc = e != cudaSuccess ? cuda_status(e) : check_launch();
         if (rc) return rc;
         c->buf.cur = b;
@@ -346,30 +365,50 @@ void g_rows_t(lb_ctx *c, int i0, int i1, double *out)
 }
 
 // FP32-shifted steps of a general (19-value) state with tau_g = 1.  Within
-// one call g's 19 values are only wanted at its end: the first phi is the sum
-// of the stored g, the steps between are the reduced form's two passes on
-// scratch in the g level that the call does not end in, and the last step's
-// collision writes g* = geq in full.  n steps move 20 + 49 (n - 1) + 58 words
-// a site instead of 76 n (the bulk kernel) or 97 n (two passes), and the
-// stored state between calls stays the general one.
+// one call g's 19 values are only wanted at its end: the steps are the reduced
+// form's two passes on scratch in the g level that the call does not end in,
+// and the last step's collision writes g* = geq in full too.  The stored state
+// between calls stays the general one.
+// The first phi is the sum of the stored g after a new start (init,
+// set_state, steps of another kernel), else the phi pass over the last step's
+// phi (kept in the phi buffer) and quads (in the spare g level), so that the
+// bits of a run do not depend on how it is cut into calls.  Which it is stands
+// in device memory (lb_ctx::moments, cleared on the stream by every call that
+// writes the state), so that captured steps do not fix it.  n steps move
+// 6 + 49 (n - 1) + 64 words a site (20 + 49 (n - 1) + 64 after a new start)
+// instead of 76 n (the bulk kernel) or 97 n (two passes).
 template <int NP, int KY>
 static int run_geq(lb_ctx *c, int nsteps)
 {
-    T1Passes<float, true, NP, KY> pass;
-    int rc = pass.plan(c, 0);
+    static std::atomic<int> cache[kPhiMaxWarps + 1];
+    PhiLaunch<KY> pass;
+    int rc = pass.plan(c, k_geq_phi<KY>, 0, cache);
     if (rc) return rc;
+    const auto collide = uses_mrt(c) ? k_geq_collide<NP, true> : k_geq_collide<NP, false>;
+    const auto p = make_coll<float>(c->p);
+    const auto m = make_mrt<float>(c);
+    const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     int a = c->buf.cur;
     const int last = (a + nsteps) & 1;
+    float *kept = (float *)c->phi;
     float *scratch = (float *)c->buf.g[1 - last];   // g(t) itself where nsteps is odd, until its phi is summed
-    float *phi = (float *)c->phi, *phi_next = scratch, *quad = quads(scratch, c->S);
-    cudaError_t e = launch_phi_pull(c, (const float *)c->buf.g[a], phi);
-    for (int t = 0; t + 1 < nsteps && e == cudaSuccess; t++, a = 1 - a) {
-        e = pass.collide((const float *)c->buf.f[a], phi, quad, (float *)c->buf.f[1 - a]);
-        if (e == cudaSuccess) e = pass.next_phi(phi, quad, phi_next);
-        std::swap(phi, phi_next);
+    float *quad = quads(scratch, c->S);
+    // phi(t) stands in row 0 of scratch and in the phi buffer by turns
+    float *phi = scratch, *next = kept;
+    auto phi_pass = [&](const float *ga, const float *from, const float *q, float *to) {
+        return launch_pdl(k_geq_phi<KY>, pass.grid, pass.block, c->stream, ga, (const int *)c->moments, from, q, to,
+                          nx, ny, nz, pass.kzc, c->S);
+    };
+    cudaError_t e = phi_pass((const float *)c->buf.g[a], kept, quads((float *)c->buf.g[1 - a], c->S), phi);
+    for (int t = 0; t < nsteps && e == cudaSuccess; t++, a = 1 - a) {
+        const bool ends = t + 1 == nsteps;
+        e = launch_pdl(collide, grid_of(c->N), kT1Threads, c->stream, (const float *)c->buf.f[a], (const float *)phi,
+                       quad, (float *)c->buf.f[1 - a], ends ? (float *)c->buf.g[last] : nullptr,
+                       phi == kept ? nullptr : kept, c->moments, p, m, nx, ny, nz, c->S);
+        if (ends || e != cudaSuccess) break;
+        e = phi_pass(nullptr, phi, quad, next);
+        std::swap(phi, next);
     }
-    if (e == cudaSuccess)
-        e = launch_collide_geq(c, (const float *)c->buf.f[a], phi, (float *)c->buf.f[last], (float *)c->buf.g[last]);
     rc = e != cudaSuccess ? cuda_status(e) : check_launch();
     if (rc) return rc;
     c->buf.cur = last;
@@ -442,7 +481,8 @@ int taug1_convert(lb_ctx *c, int to_reduced)
             // moments are read from the other level)
             to_full_t<T, decltype(P)::SH>(c);
         }
-        return check_launch();
+        const int rc = check_launch();
+        return rc ? rc : state_written(c);
     });
 }
 
