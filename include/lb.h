@@ -410,7 +410,8 @@ int lb_batch_run(lb_batch *b, int nsteps);
 int lb_batch_sync(lb_batch *b);
 
 /* Launch shape: threads per CTA (= sites per work item; multiple of 32, at
- * most 256; by default 256, 128 with every tau_g = 1) and CTAs per SM
+ * most 256; by default 256, with every tau_g = 1 128 in FP64 and in FP32 from
+ * 1.5 x 2^20 sites on) and CTAs per SM
  * (0 = as many as fit; the grid is
  * always co-resident).  Paper: TPB and VVL tuning, Sec. III.C and IV. */
 int lb_batch_set_launch(lb_batch *b, int threads, int ctas_per_sm);

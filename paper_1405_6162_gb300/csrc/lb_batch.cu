@@ -44,10 +44,10 @@ namespace {
 // 3 x 256 threads FP32 and 2 x 256 FP64 beat the unconstrained allocation
 // by 11 % and 9 %; the FP32 reduced form gains another 6 % at 4 x 256,
 // 64 registers, where the general form loses 3 % to spills; general states
-// with every tau_g = 1 run the reduced form's passes and take its bound:
-// 259.7 -> 160 us a step for 64 lattices of sides 16..64 in FP32, 49 words a
-// site instead of 97, and 2340 -> 2223 us in FP64, where only the reading of
-// g and its 19 multiplications go)
+// that run the reduced form's passes take its bound, the two passes that leave
+// g unread do not: 32^3 10.5 us a step at 4 x 256, 9.2 at 3 x 256.  In FP64
+// only the reading of g and its 19 multiplications go, 64 lattices of sides
+// 16..64 2340 -> 2223 us)
 #ifndef LBK_BATCH_MAXT32
 #define LBK_BATCH_MAXT32 256
 #endif
@@ -74,7 +74,7 @@ struct LatDesc {
     const T *f[2];
     const T *g[2];
     T *phi;
-    int *moments;   // kUnreadG: phi and the quads of the last step are at hand (see there)
+    int *moments;   // kMoments: phi and the quads of the last step are at hand (see there)
     Coll<T> p;
 };
 
@@ -138,24 +138,59 @@ __device__ bool grid_sync(GridBarrier *bar, unsigned int nblocks, long long time
 enum BatchStep {
     kTwoPass = 0,   // the default step: phi pass, collide/stream pass
     kReduced = 1,   // the tau_g = 1 reduced form (lb_t1.cuh)
-    // General states, every tau_g = 1: the collide pass does not read g and,
-    // in FP32, the steps of a run are the reduced form's passes on scratch in
-    // the g level that the run does not end in; the last collision writes g in
-    // full as well.  The first phi of a run is the sum of the stored g after a
+    // general states, every tau_g = 1: the two passes, g not read by the second
+    kUnreadG = 2,
+    // The same in FP32 on many sites: the steps of a run are the
+    // reduced form's passes on scratch in the g level that the run does not end
+    // in; the last collision writes g in full as well.  The first phi of a run
+    // is the sum of the stored g after a
     // new start (init, set_state), else the phi pass over the last step's phi
     // (in the lattice's phi buffer) and quads (in the spare g level), which
     // the last run left there: so k runs give the bits of one run of all their
     // steps.  Which it is stands in device memory (LatDesc::moments, cleared on
     // the stream by every call that writes a member's state), so that a
     // captured run does not fix it.
-    kUnreadG = 2,
+    kMoments = 3,
 };
+
+// The step of an ensemble's general states, and the default threads per CTA.
+// Every tau_g = 1, FP32, us a step at 256 threads, moments against two passes
+// that leave g unread (and two that read it, the step until either was there):
+//   few sites wait on latency, and the phi pass's walk along z is the longer
+//   chain: 32^3 12.9 / 9.2 (10.2), 16 lattices of sides 8..24 13.2 / 10.0 (11.1),
+//   139 k sites in 32 lattices 12.8 / 12.6 (14.0), 196 k in 48 15.0 / 13.6 (16.1);
+//   about even from 2^18 on: 229 k in 4 lattices 15.9 / 14.9 (16.8), 235 k in 16
+//   15.7 / 16.9 (19.2), 64^3 17.7 / 18.5 (21.7), 351 k in 2 18.5 / 20.8 (23.9);
+//   many are bound by the words moved: 506 k 24.8 / 30.2 (35.8), 4.5 M in 64
+//   lattices of sides 16..64 171 / 239 (287).
+// CTAs of 128 threads share many lattices out more evenly, and are more to wait
+// for at a group's barrier, FP32 us a step at 256 / 128 threads: 139 k sites
+// 12.8 / 17.1, 267 k 16.9 / 21.6, 506 k 24.8 / 28.2, 1.06 M 43.8 / 44.2, 1.6 M
+// 68.3 / 65.4, 1.7 M 68.2 / 68.8, 1.9 M 75.1 / 73.5, 2.3 M 89.4 / 86.5, 4.5 M
+// 171.2 / 165.3.  FP64, bound by its instructions: 261 k 134.8 / 129.2, 1.06 M
+// 529.9 / 487.9, 32^3 38.6 / 39.1; with g read 42.4 / 41.8 and it keeps 256.
+constexpr long long kMomentsMinSites = 7LL << 15, kSmallCtaSites = 3LL << 19;
+
+struct BatchDefaults {
+    int step, threads;
+};
+inline BatchDefaults batch_defaults(int n, const lb_params *p)
+{
+    long long sites = 0;
+    for (int k = 0; k < n; k++) {
+        if (!g_is_equilibrium(p[k])) return {kTwoPass, 256};
+        sites += (long long)p[k].nx * p[k].ny * p[k].nz;
+    }
+    if (p[0].precision == LB_FP64) return {kUnreadG, 128};
+    return {sites > kMomentsMinSites ? kMoments : kUnreadG, sites >= kSmallCtaSites ? 128 : 256};
+}
 
 // CTAs per SM the register budget of a step allows
 template <typename T>
 constexpr int batch_min_ctas(int step)
 {
-    return sizeof(T) == 8 ? LBK_BATCH_MINB64 : step == kTwoPass ? LBK_BATCH_MINB32 : LBK_BATCH_MINB32_RED;
+    return sizeof(T) == 8 ? LBK_BATCH_MINB64
+           : step == kTwoPass || step == kUnreadG ? LBK_BATCH_MINB32 : LBK_BATCH_MINB32_RED;
 }
 
 // The passes over a group's slice of the work lists, by CTA r of the group.
@@ -272,7 +307,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kBatchMaxThreads64 : kBatchMa
             pass.t1_phi(a, all, [&](L l) { return l.g[a]; }, [&](L l) { return const_cast<T *>(l.g[1 - a]); });
             if (!sync()) return;
         }
-    } else if constexpr (STEP == kUnreadG && sizeof(T) == 4) {
+    } else if constexpr (STEP == kMoments) {
         const int a0 = parity0 & 1, spare = 1 - ((parity0 + nsteps) & 1);
         auto kept = [](L l) { return *l.moments != 0; };
         pass.pull_phi(a0, [&](L l) { return !kept(l); });
@@ -396,7 +431,7 @@ struct lb_batch {
     int ngroups = 0;
     int bins = 0;                              // lb_batch_set_plan: 0 = a group per lattice, k = k groups
     int reduced = 0;                           // all lattices in the tau_g = 1 reduced form
-    int unread_g = 0;                          // every tau_g = 1
+    int general = lbk::kTwoPass;               // the step of general states
     int *d_moments = nullptr;                  // [n] LatDesc::moments
     lbk::GridBarrier *d_bar = nullptr;         // one per group
     int skip_cta = -1;                         // test hook: first CTA of the largest group
@@ -419,12 +454,14 @@ void drop_graphs(lb_batch *b)
 }
 
 // what a step of the ensemble does now, and its kernel
-int batch_step(const lb_batch *b) { return b->reduced ? lbk::kReduced : b->unread_g ? lbk::kUnreadG : lbk::kTwoPass; }
+int batch_step(const lb_batch *b) { return b->reduced ? lbk::kReduced : b->general; }
 
 template <typename T, bool SH>
 auto batch_kernel(const lb_batch *b)
 {
     const int step = batch_step(b);
+    if constexpr (sizeof(T) == 4)
+        if (step == lbk::kMoments) return lbk::k_batch<T, SH, lbk::kMoments>;
     return step == lbk::kReduced   ? lbk::k_batch<T, SH, lbk::kReduced>
            : step == lbk::kUnreadG ? lbk::k_batch<T, SH, lbk::kUnreadG>
                                    : lbk::k_batch<T, SH, lbk::kTwoPass>;
@@ -489,7 +526,7 @@ int batch_tables(lb_batch *b)
             const size_t w0 = work.size();
             work.resize(w0 + (size_t)nb[k]);
             for (long long j = 0; j < nb[k]; j++) work[w0 + (size_t)j] = make_int2(k, (int)j);
-            if (!b->reduced && !(b->unread_g && sizeof(T) == 4)) continue;
+            if (batch_step(b) != lbk::kReduced && batch_step(b) != lbk::kMoments) continue;
             // the lattice's tiles, their run length for its share of the group's
             // warps.  Tiles go to single warps: a group has some tens of CTAs at
             // most, and whole-CTA tiles of one run length for all left it 1.9
@@ -656,13 +693,9 @@ int lb_batch_create(int n, const lb_params *p, void *cuda_stream, lb_batch **out
     if (!rc) rc = lbk::cuda_status(cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming));
     if (!rc) rc = lbk::cuda_status(cudaMalloc(&b->d_err, sizeof(unsigned int)));
     if (!rc) rc = lbk::cuda_status(cudaMemset(b->d_err, 0, sizeof(unsigned int)));
-    b->unread_g = 1;
-    for (int k = 0; k < n; k++) b->unread_g = b->unread_g && lbk::g_is_equilibrium(p[k]);
-    // CTAs of 128 threads share the lattices out more evenly: 64 lattices of
-    // sides 16..64, 100 steps 17.26 ms at 256 threads, 16.95 at 192, 16.68 at
-    // 128, 17.14 at 96, 17.06 at 64 (FP32); FP64, 61 lattices of 16..55 101.9 /
-    // 97.7 ms at 256 / 128, 53 of 11..27 20.9 / 17.0
-    if (b->unread_g) b->threads = 128;
+    const lbk::BatchDefaults defaults = lbk::batch_defaults(n, p);
+    b->general = defaults.step;
+    b->threads = defaults.threads;
     if (!rc) rc = lbk::cuda_status(cudaMalloc(&b->d_moments, n * sizeof(int)));
     if (!rc) rc = lbk::cuda_status(cudaMemset(b->d_moments, 0, n * sizeof(int)));
     if (!rc)

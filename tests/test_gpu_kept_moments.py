@@ -171,3 +171,58 @@ def test_ensemble_bits_do_not_depend_on_the_runs(launch):
         want = want or got
         for a, w in zip(got, want):
             assert np.array_equal(a[0], w[0]) and np.array_equal(a[1], w[1]), runs
+
+
+def test_an_ensemble_on_many_sites_follows_its_members():
+    """A member written between two runs of an ensemble that keeps moments is
+    followed, one left alone keeps the bits of an undivided run."""
+    from paper_1405_6162_gb300 import Batch
+    dims = [(20, 17, 16), (33, 18, 21), (64, 64, 40), (17, 31, 9), (61, 40, 33)]
+    specs = [dict(P0, nx=x, ny=y, nz=z, tau=0.6 + 0.1 * k) for k, (x, y, z) in enumerate(dims)]
+    start = [_state(d, 960 + k) for k, d in enumerate(dims)]
+    other = _state(dims[1], 970)
+    phi = L.spinodal_phi0(*dims[2], seed=971, amp=0.3)
+    with Batch(specs, precision="fp32_shifted") as b, Batch(specs, precision="fp32_shifted") as c:
+        for x in (b, c):
+            for k, s in enumerate(start):
+                x[k].set_state(*s)
+        b.run(3)
+        b[1].set_state(*other)
+        b[2].init(phi)
+        b.run(2)
+        got = [b[k].get_state() for k in range(len(dims))]
+        c.run(5)
+        want = [c[k].get_state() for k in range(len(dims))]
+        c[1].set_state(*other)
+        c[2].init(phi)
+        c.run(2)
+        want[1], want[2] = c[1].get_state(), c[2].get_state()
+    for k, (a, w) in enumerate(zip(got, want)):
+        assert np.array_equal(a[0], w[0]) and np.array_equal(a[1], w[1]), k
+
+
+# lattices on either side of an ensemble's lines (229376 and 1572864 sites),
+# with tau_g = 1 and not, all alike and mixed
+@pytest.mark.parametrize("precision,tol", [("fp32_shifted", TOL_FP32), ("fp64", 1e-12)])
+@pytest.mark.parametrize("tau_g", [1.0, 0.85, None])
+@pytest.mark.parametrize("dims", [[(13, 7, 5), (1, 1, 9), (32, 32, 32), (20, 33, 17)],
+                                  [(61, 61, 61), (5, 31, 3), (33, 10, 5)], [(61, 61, 61), (5, 31, 3), (33, 10, 6)],
+                                  [(128, 96, 64), (96, 128, 64), (9, 9, 9)]])
+def test_ensemble_steps_match_oracle(dims, tau_g, precision, tol):
+    import oracle
+    from paper_1405_6162_gb300 import Batch
+    from tests.parity import to_oracle
+    oracle.build()
+    specs = [dict(P0, nx=x, ny=y, nz=z, tau=0.7 + 0.1 * k, tau_g=(1.0 if k % 2 else 0.85) if tau_g is None else tau_g)
+             for k, (x, y, z) in enumerate(dims)]
+    start = [nonequilibrium_state(d, P, seed=980 + k) for k, d in enumerate(dims)]
+    with Batch(specs, precision=precision) as b:
+        for k, s in enumerate(start):
+            b[k].set_state(*[to_abi(x) for x in s])
+        b.run(1)
+        b.run(2)
+        got = [b[k].get_state() for k in range(len(dims))]
+    for k, d in enumerate(dims):
+        p = {q: specs[k][q] for q in P0}
+        for a, w in zip(got[k], oracle.step(d, p, *start[k], 3, kind="omp")):
+            assert rel(to_oracle(a), w) <= tol
