@@ -79,8 +79,9 @@ enum { LB_HOST = 0, LB_DEVICE = 1 };
 /* Step kernels selectable with lb_set_kernel(). */
 enum {
     LB_KERNEL_AUTO = 0,     /* library default, the fastest measured on GB300.
-                               FP32-shifted with tau_g = 1, more than 2^18
-                               sites and rows of 12 or more: between steps
+                               FP32-shifted with tau_g = 1 from about 1.25 x
+                               2^18 sites on (more where rows or planes are
+                               few or short: lb_taug1.cu): between steps
                                g is kept as its equilibrium's moments; the
                                last step of a call writes it in full as well.
                                Else LB_KERNEL_BULK (3 slots, clusters of 2,

@@ -296,7 +296,7 @@ int run_t1(lb_ctx *c, int nsteps)
 // y rows a lane of the phi pass in FP32: two from 2^20 sites on (us a step:
 // 128^3 68.2 against 70.1, 256^3 513 / 529, 200x152x136 131.2 / 137.1; below,
 // one: 129x97x65 31.5 / 31.0, 96^3 33.4 / 33.5), one where the lattice has
-// fewer than four rows (1024x1x1024 51 / 43).
+// fewer than four rows.
 int phi_rows(const lb_ctx *c) { return c->N >= (1LL << 20) && c->p.ny >= 4 ? 2 : 1; }
 
 template <typename T, bool SH, int NP>
@@ -423,23 +423,31 @@ static int run_geq_np(lb_ctx *c, int nsteps)
     return run_geq<7, KY>(c, nsteps);
 }
 
-// When the library default takes these steps (microseconds a step over 50
-// steps, against two passes that leave g unread, 78 words a site):
-//   256^3 530 / 770, 200x152x136 140 / 200, 128^3 74 / 103, 80^3 21.1 / 26.8,
-//   72x64x64 14.3 / 14.3, 64^3 13.1 / 13.0, 32^3 7.7 / 4.6 -- below 2^18
-//   sites both passes wait on latency, and the phi pass's walk along z is the
-//   longer chain;
-//   rows of 16 sites 82 / 103, of 12 69 / 79, of 8 56 / 53 (2^20 sites or
-//   so) -- a warp's 30 output columns are mostly idle on short rows.
+// When the library default takes these steps.  The phi pass gains by the words
+// that it saves and loses by its latency -- warps walk along z -- and by the
+// lanes that write nothing: of the positions of a row nx of nx + 2 do, of the
+// rows of a CTA's warps ny of a multiple of them.  Microseconds a step over 50
+// steps and in calls of one, against two passes that leave g unread (78 words
+// a site; with g read, the default until these steps were there, in brackets):
+//   256^3 516 and 713 / 770 (904), 128^3 68.9 and 93.8 / 103 (121), 80^3 19.6
+//   and 27.5 / 25.8 (30.4), 72^3 15.3 and 20.6 / 18.0 (21.5), 68^3 14.1 and 18.3
+//   / 14.9 (17.8), 64^3 12.5 and 15.1 / 12.1 (13.8), 48^3 9.1 and 10.5 / 8.2;
+//   rows of 2, 4, 8 sites (2^20 sites) 44.9, 40.9, 39.9 and 57.4, 53.5, 52.6 /
+//   52.3 (61.4);  600x3x300 22.4 and 30.5 / 27.5 (32.0), 128x5x600 17.0 and 22.6
+//   / 18.4 (21.9), 600x2x300 17.7 and 22.8 / 17.3 (20.7);
+//   1024x1x1024 57.6 and 70.5 / 53.0 (61.0), 16x1x60000 75.6 and 87.6 / 48.0 (56);
+//   one plane, read three times for one written: 600x600 17.3 and 22.1 / 17.3
+//   (20.4), 1200x1200 67.8 and 84.6 / 72.5 (84.3), 2000x2000 173 and 219 / 193
+//   (228), 12x99000 60.3 and 74.5 / 60.6 (69.7).
 // FP64 and double-float steps are bound by arithmetic, of which the reduced
 // form's phi pass has more; they take the two passes.
-constexpr long long kGeqMinSites = (1LL << 18) + 1;
-constexpr int kGeqMinRow = 12;
-
 bool auto_uses_geq(const lb_ctx *c)
 {
-    return c->p.precision == LB_FP32_SHIFTED && g_is_equilibrium(c->p) && c->N >= kGeqMinSites &&
-           c->p.nx >= kGeqMinRow;
+    if (c->p.precision != LB_FP32_SHIFTED || !g_is_equilibrium(c->p)) return false;
+    const int rows = phi_rows(c) * kPhiWarps, nx = c->p.nx, ny = c->p.ny;
+    const double writing = double(nx) / (nx + 2.0) * ny / (double(ny - 1 - (ny - 1) % rows) + rows);
+    const bool plane = c->p.nz == 1;
+    return writing >= (plane ? 0.9 : 0.45) && writing * c->N >= (plane ? 1 << 20 : 5 << 16);
 }
 
 int launch_step_geq(lb_ctx *c, int nsteps)

@@ -21,7 +21,7 @@ TOL_FP32 = 2e-6
 P = dict(P0, tau=0.7, kappa=0.06)
 FORCE = (1e-5, -2e-5, 3e-5)
 # one and two rows a lane (2^20 sites), odd rows, short rows, one plane, few rows
-DIMS = [(72, 73, 72), (31, 97, 130), (128, 128, 64), (13, 170, 160), (2049, 1024, 1), (700, 3, 250), (129, 64, 127)]
+DIMS = [(72, 73, 72), (31, 97, 130), (128, 128, 64), (13, 180, 170), (2049, 1024, 1), (700, 3, 250), (129, 64, 127), (4, 350, 360)]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -171,6 +171,35 @@ def test_ensemble_bits_do_not_depend_on_the_runs(launch):
         want = want or got
         for a, w in zip(got, want):
             assert np.array_equal(a[0], w[0]) and np.array_equal(a[1], w[1]), runs
+
+
+# on either side of the default's lines: sites, rows and planes that leave
+# lanes idle, one plane; and with the wide stencils, several rates and a force
+@pytest.mark.parametrize("dims,npts,rates,force", [(d, 7, None, (0, 0, 0)) for d in [
+    (70, 70, 70), (72, 72, 72), (4, 330, 360), (4, 350, 360), (2, 700, 700), (1, 900, 900), (128, 5, 600), (130, 6, 600), (600, 2, 500),
+    (600, 2, 600), (1024, 1, 512), (1060, 1000, 1), (1024, 1000, 1), (20, 60000, 1), (17, 65000, 1)]] + [
+    ((72, 73, 72), 19, None, (0, 0, 0)), ((72, 73, 72), 27, (1.3, 0.6), FORCE), ((4, 350, 360), 27, None, (0, 0, 0)),
+    ((72, 73, 72), 7, (1.7, 0.55), FORCE), ((72, 73, 72), 7, None, FORCE)])
+def test_default_steps_match_oracle_beside_its_lines(dims, npts, rates, force):
+    import oracle
+    from tests.parity import to_oracle
+    oracle.build()
+    s0 = nonequilibrium_state(dims, P, seed=990)
+    with _lattice(dims) as lat:
+        lat.set_stencil(npts)
+        if rates:
+            lat.set_collision("mrt", *rates)
+        lat.set_force(*force)
+        lat.set_state(*[to_abi(x) for x in s0])
+        lat.step(1)
+        lat.step(2)
+        got = lat.get_state()
+    if npts == 7 and not rates and not any(force):
+        want = oracle.step(dims, P, *s0, 3, kind="omp")
+    else:
+        want = oracle.step_mrt(dims, P, *s0, 3, *(rates or (P["tau"], P["tau"])), force, kind="omp", npts=npts)
+    for a, w in zip(got, want):
+        assert rel(to_oracle(a), w) <= TOL_FP32
 
 
 def test_an_ensemble_on_many_sites_follows_its_members():
