@@ -184,20 +184,13 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b)
 
 // a + b without the renormalisation: the high parts' sum, and its error with
 // the low parts.  Further sums of such values err no more (the parts' errors
-// are relative to the terms, not to the sum); renormalised() before a product
-// or storage.
+// are relative to the terms, not to the sum); not before a product or storage.
 __device__ __forceinline__ df64 sum_term(df64 a, df64 b)
 {
     df64 r;
     float e;
     dfops::two_sum(a.hi, b.hi, r.hi, e);
     r.lo = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-    return r;
-}
-__device__ __forceinline__ df64 renormalised(df64 a)
-{
-    df64 r;
-    dfops::two_sum(a.hi, a.lo, r.hi, r.lo);
     return r;
 }
 // c x, c a power of two (exact, barring underflow)
@@ -325,22 +318,20 @@ __device__ __forceinline__ double widen(double x) { return x; }
 // hi + lo of a double-float is exact in FP64 (|lo| <= ulp(hi) / 2)
 __device__ __forceinline__ double widen(df64 x) { return widen(x.hi) + widen(x.lo); }
 
-// A double as a double-float, to 2^-47, on the integer and FP32 units (the
-// conversions of df64(double) are four instructions of the FP64 pipe): the
-// top 24 bits and the next 23 are cut out of the IEEE 754 layout, the cut-off
-// part as an integer below 2^23 in the fraction of 2^23.  Values that are
-// zero, or too small or large for the parts to be normal floats, are
+// A double as a double-float, to 2^-49 as df64(double), on the integer and FP32
+// units (that conversion is four instructions of the FP64 pipe): the high part
+// is the top 24 bits of the IEEE 754 layout, rounded by the bit after them, and
+// the low part the other 29 bits as a signed integer, rounded to float.  Values
+// that are zero, or too small or large for the parts to be normal floats, are
 // converted (zero by its sign bit).
 __device__ __forceinline__ df64 split_double(double d)
 {
     const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
     const unsigned e = (h >> 20) & 0x7ffu, sign = h & 0x80000000u;
     if (e - 960u < 190u) {   // 2^-63 <= |d| < 2^127
-        const float hi = __uint_as_float(sign | (((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29));
-        const float cut = __fsub_rn(__uint_as_float(0x4b000000u | ((l >> 6) & 0x7fffffu)), 8388608.0f);
-        df64 r;
-        dfops::fast_two_sum(hi, __fmul_rn(__uint_as_float(sign | ((e - 942u) << 23)), cut), r.hi, r.lo);
-        return r;
+        const unsigned top = ((((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29)) + ((l >> 28) & 1u);
+        const float rest = __int2float_rn((int)(l << 3) >> 3);   // units of 2^(e - 1075)
+        return df64(__uint_as_float(sign | top), __fmul_rn(__uint_as_float(sign | ((e - 948u) << 23)), rest));
     }
     if (((h << 1) | l) == 0) return df64(__uint_as_float(sign), 0.0f);
     return df64(d);

@@ -20,66 +20,63 @@ namespace lbk {
 // ------------------------------------------------------------------ init
 
 // A_i(x - c_i) = feq_i(x), so that the first pull yields the equilibrium of
-// phi0 and u0.  Double storage evaluates stencils and equilibria in double.
-// Float and double-float storage evaluate the equilibria in double-float
-// arithmetic on the FP32 units (df64.cuh, ~48 bits; the double pipe runs at
-// 1/64 of the float rate): double-float storage, its stencils in double, keeps
-// the value, float storage its high part -- the float nearest to it, the same
-// float as rounding a double result except at a near tie.  Float storage
-// splits the inputs on the integer units and takes the stencils in
-// double-float too: with them in double, 50 instructions a site of the FP64
-// pipe (120 more at 27 points) bounded this kernel.  Without u0 half the sums
-// are not formed (opposite values are equal).
-// 256^3 float: 1659 -> 639 us without u0 (380 is the copy rate over its
-// bytes), 1959 -> 1247 us with it, bound by the FP32 units; 27 points
-// 129x97x65 197 -> 119 us.
+// phi0 (its stencils taken in double) and u0.  Double storage evaluates the
+// equilibria in double.  Float and double-float storage evaluate them in
+// double-float arithmetic on the FP32 units (df64.cuh, ~48 bits; the double
+// pipe runs at 1/64 of the float rate), with the inputs split on the integer
+// units: double-float storage keeps the value, float storage the float nearest
+// to it, the same float as rounding a double result except at a near tie.
+// Without u0 float storage does not form half of the sums (opposite values are
+// equal).
+// Float, 7 points: 256^3 593 us without u0 (380 is the copy rate over its
+// bytes) and 1109 with it, bound by the FP32 units; 27 points, 129x97x65 147 and
+// 151, bound by the 119 FP64 additions of the stencil.  With the inputs
+// converted on the FP64 pipe and direct sums 1659, 1963, 179 and 201.
 __device__ __forceinline__ void init_store(float *a, size_t o, df64 v) { a[o] = __fadd_rn(v.hi, v.lo); }
-__device__ __forceinline__ void init_store(df64 *a, size_t o, df64 v) { a[o] = renormalised(v); }
-__device__ __forceinline__ void init_store(double *a, size_t o, double v) { a[o] = v; }
-
-// inputs and stencils of storage T: split on the integer units for float
-// storage, else doubles
 template <typename T>
-struct InitArith {
-    using type = double;
-    static __device__ __forceinline__ double in(double v) { return v; }
-};
-template <>
-struct InitArith<float> {
-    using type = df64;
-    static __device__ __forceinline__ df64 in(double v) { return split_double(v); }
-};
-template <>
-__device__ __forceinline__ df64 stencil_value<df64, double>(double v)
+__device__ __forceinline__ void init_store(T *a, size_t o, T v)
 {
-    return split_double(v);
+    a[o] = v;
+}
+template <typename E>
+__device__ __forceinline__ E init_arith(double v)
+{
+    if constexpr (is_df64<E>::value)
+        return split_double(v);
+    else
+        return v;
 }
 
 // p in the arithmetic type E of the equilibria; FLOW: u0 is given
 template <typename T, typename E, bool SH, int NP, bool FLOW>
 __global__ void __launch_bounds__(256) k_init(const double *__restrict__ phi0,
                                               const double *__restrict__ u0,
-                                              T *__restrict__ fa, T *__restrict__ ga,
-                                              Coll<E> p, int nx, int ny, int nz, long long S)
+                                              T *__restrict__ fa, T *__restrict__ ga, Coll<E> p, double rho0, int nx,
+                                              int ny, int nz, long long S)
 {
     const long long N = (long long)nx * ny * nz;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
     const Nbr n(s, nx, ny, nz);
-    using In = InitArith<T>;
-    using R = typename In::type;
-    const R ph = In::in(phi0[s]);
-    R dx, dy, dz, lap;
-    stencil_np<NP, R>(phi0, n, ph, dx, dy, dz, lap);
-    E u[3] = {E(0), E(0), E(0)};
+    const double ph = phi0[s];
+    double dx, dy, dz, lap;
+    stencil_np<NP, double>(phi0, n, ph, dx, dy, dz, lap);
+    E v[3] = {E(0), E(0), E(0)};   // u, or rho0 u
     if (FLOW)
 #pragma unroll
-        for (int a = 0; a < 3; a++) u[a] = E(In::in(u0[a * N + s]));
-    equilibria<E, SH, FLOW>(p, u[0], u[1], u[2], E(ph), E(dx), E(dy), E(dz), E(lap), [&](int i, E fe, E ge) {
+        for (int a = 0; a < 3; a++)
+            v[a] = init_arith<E>(std::is_same<T, float>::value ? u0[a * N + s] : rho0 * u0[a * N + s]);
+    const E q = init_arith<E>(ph), gx = init_arith<E>(dx), gy = init_arith<E>(dy), gz = init_arith<E>(dz);
+    const E l = init_arith<E>(lap);
+    auto sink = [&](int i, E fe, E ge) {
         const size_t o = (size_t)i * S + n.src(i);
         init_store(fa, o, fe);
         init_store(ga, o, ge);
-    });
+    };
+    if constexpr (std::is_same<T, float>::value)
+        equilibria_float<E, SH, FLOW>(p, v[0], v[1], v[2], q, gx, gy, gz, l, sink);
+    else
+        equilibria<E, SH>(p, SH ? E(0) : p.rho0, v[0], v[1], v[2], q, gx, gy, gz, l, sink);
 }
 
 // ------------------------------------------------------------------ moments / state
@@ -345,7 +342,7 @@ static void init_np(lb_ctx *c, const double *phi0_d, const double *u0_d)
     using E = typename std::conditional<std::is_same<T, double>::value, double, df64>::type;
     const auto kernel = u0_d ? k_init<T, E, SH, NP, true> : k_init<T, E, SH, NP, false>;
     kernel<<<grid_for(c->N, 256), 256, 0, c->stream>>>(phi0_d, u0_d, (T *)c->buf.f[cur], (T *)c->buf.g[cur],
-                                                       make_coll<E>(c->p), c->p.nx, c->p.ny, c->p.nz, c->S);
+                                                       make_coll<E>(c->p), c->p.rho0, c->p.nx, c->p.ny, c->p.nz, c->S);
 }
 
 template <typename T, bool SH>

@@ -29,13 +29,6 @@ struct Nbr {
     __device__ __forceinline__ int src(int i) const { return at(-cx(i), -cy(i), -cz(i)); }
 };
 
-// a stored value in the arithmetic type of the stencil
-template <typename R, typename T>
-__device__ __forceinline__ R stencil_value(T v)
-{
-    return R(v);
-}
-
 // The phi stencil of NP points: 7 = nearest faces, d_a phi = (phi(x + e_a) -
 // phi(x - e_a))/2, lap phi = sum of the 6 faces - 6 phi(x); 19 / 27 =
 // the isotropic lattice-weighted differences over the D3Q19 / D3Q27
@@ -50,9 +43,9 @@ __device__ __forceinline__ void stencil_np(const T *__restrict__ phi, const Nbr 
 {
     static_assert(NP == 7 || NP == 19 || NP == 27, "stencil of 7, 19 or 27 points");
     if constexpr (NP == 7) {
-        const R xp = stencil_value<R>(phi[n.at(1, 0, 0)]), xm = stencil_value<R>(phi[n.at(-1, 0, 0)]);
-        const R yp = stencil_value<R>(phi[n.at(0, 1, 0)]), ym = stencil_value<R>(phi[n.at(0, -1, 0)]);
-        const R zp = stencil_value<R>(phi[n.at(0, 0, 1)]), zm = stencil_value<R>(phi[n.at(0, 0, -1)]);
+        const R xp = R(phi[n.at(1, 0, 0)]), xm = R(phi[n.at(-1, 0, 0)]);
+        const R yp = R(phi[n.at(0, 1, 0)]), ym = R(phi[n.at(0, -1, 0)]);
+        const R zp = R(phi[n.at(0, 0, 1)]), zm = R(phi[n.at(0, 0, -1)]);
         dx = D2 ? xp - xm : half(xp - xm);
         dy = D2 ? yp - ym : half(yp - ym);
         dz = D2 ? zp - zm : half(zp - zm);
@@ -69,7 +62,7 @@ __device__ __forceinline__ void stencil_np(const T *__restrict__ phi, const Nbr 
                 for (int c = -1; c <= 1; c++) {
                     const int k = a * a + b * b + c * c;
                     if (k == 0 || (NP == 19 && k == 3)) continue;
-                    const R v = stencil_value<R>(phi[n.at(a, b, c)]);
+                    const R v = R(phi[n.at(a, b, c)]);
                     sum[k] += v;
                     if (a) da[k] += a > 0 ? v : -v;
                     if (b) db[k] += b > 0 ? v : -v;
