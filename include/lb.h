@@ -229,8 +229,8 @@ int lb_set_state_masked(lb_ctx *c, const unsigned char *mask, const double *f, c
  * block_y threads per CTA and z_chunk planes per CTA of the fused, staged
  * and slab kernels (0 = library default for any of the three).  For
  * LB_KERNEL_AUTO and LB_KERNEL_TWO_PASS block_x is the threads per CTA of
- * both passes (a multiple of 32 up to 256; 0 = by size and precision: 32 to
- * 256), block_y the sites per
+ * both passes (a multiple of 32 up to 256; 0 = by size, precision and pass: 32
+ * to 256), block_y the sites per
  * thread of the phi pass (1, 2 or 4; 0 = 1) and z_chunk must be 0.  For
  * LB_KERNEL_LAG block_x must be 0 or 256, block_y 0 or 1, and z_chunk is the
  * lag slack in site blocks beyond the stencil's reach (0 = default 128).

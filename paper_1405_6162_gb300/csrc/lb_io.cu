@@ -30,7 +30,7 @@ namespace lbk {
 // equal).
 // Float, 7 points: 256^3 593 us without u0 (380 is the copy rate over its
 // bytes) and 1109 with it, bound by the FP32 units; 27 points, 129x97x65 147 and
-// 151, bound by the 119 FP64 additions of the stencil.  With the inputs
+// 151, bound by the stencil's FP64 instructions.  With the inputs
 // converted on the FP64 pipe and direct sums 1659, 1963, 179 and 201.
 __device__ __forceinline__ void init_store(float *a, size_t o, df64 v) { a[o] = __fadd_rn(v.hi, v.lo); }
 template <typename T>

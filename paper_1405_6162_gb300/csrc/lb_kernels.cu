@@ -170,18 +170,21 @@ static cudaError_t launch_collide(lb_ctx *c, const T *fa, const T *ga, const T *
 
 // tau_g = 1: the collide pass does not read g, except in double-float with the
 // multiple relaxation times, whose collision does not fit the 96 registers
-// that pay there (144x120x100 338 us a step against 321 with g read)
+// that pay there (144x120x100 338 us a step against 321 with g read), and where
+// the caller asks for more threads than that collision is compiled for (128 in
+// double-float: 222.7 us a step; 240.4 with g read in CTAs of 256)
 template <typename T>
 static bool leaves_g_unread(const lb_ctx *c)
 {
-    return g_is_equilibrium(c->p) && !(is_df64<T>::value && uses_mrt(c));
+    return g_is_equilibrium(c->p) && !(is_df64<T>::value && uses_mrt(c)) && c->block_x <= LBK_K2_MAXT(T, true);
 }
 
 template <typename T, bool SH, int NP>
 static int two_pass(lb_ctx *c, int nsteps)
 {
     // launch shape: threads per CTA of both passes, sites per thread of the
-    // phi pass (lb_set_kernel's block_x, block_y; 0 = default_threads and 1)
+    // phi pass (lb_set_kernel's block_x, block_y; 0 = default_threads, cut to
+    // the collision's limit there, and 1)
     const int tpb = c->block_x ? c->block_x : default_threads<T>(c->N);
     const int vvl = c->block_y ? c->block_y : 1;
     for (int t = 0; t < nsteps; t++) {
