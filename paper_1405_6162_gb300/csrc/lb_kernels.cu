@@ -121,17 +121,27 @@ static inline unsigned grid_for(long long N, int tpb) { return (unsigned)((N + t
 //   192, whichever leaves the busiest of the 152 SMs fewer sites: 64^3 114.5
 //   at 256, 113.6 at 128, 109.8 at 192; 80^3 221.3, 213.6, 214.1; 100^3 407.1,
 //   405.5, 409.2.
-//   FP32: 128 below 2^20 sites -- 16^3 4.28 / 3.64, 64^3 13.05 / 12.33 (tau_g
-//   != 1 14.1 / 13.4), 80^3 26.6 / 25.7, 100^3 51.2 / 50.6 -- and 256 above,
-//   where 128 lose up to 2 % (160^3 234.6 / 239.5).
+//   FP32: 128 below 2^20 sites -- 16^3 4.28 at 256 / 3.55, 64^3 12.97 / 12.23
+//   (tau_g != 1 13.9 / 13.5), 80^3 26.6 / 26.0 (30.3 / 29.9) -- and 256 above,
+//   where 128 lose up to 2 % (160^3 234.6 / 239.5); but where 152 SMs have one
+//   or two CTAs of 128 each the uneven share shows: 32 from 3 x 2^13 to 3 x 2^14
+//   sites -- 30^3 4.48 at 128 / 4.52 (tau_g != 1 4.92 / 4.55), 32^3 4.74 / 4.59
+//   (5.22 / 4.79; 4.75 at 256), 34^3 5.57 / 4.97 (5.64 / 5.41), 36^3 5.73 / 5.09
+//   (6.17 / 5.50) -- and from there to 2^17 160 where g is not read: 38^3 6.28 /
+//   5.40, 40^3 6.75 / 5.68 (at 256, reading g, 6.36), 42^3 6.69 / 6.50, 46^3 8.17 /
+//   7.73; 52^3 8.11 / 8.80 (with g read 42^3 6.27 / 7.49).
 //   Double-float: 64 below 2^18 sites (16^3 to 56x52x60 3 to 8 % with tau_g
 //   != 1, 1 % without), 256 above (128x128x64 152.3 / 155.4).
 template <typename T>
-static int default_threads(long long N)
+static int default_threads(long long N, bool geq = false)
 {
     const bool small = N < (1LL << 18);
     if (is_df64<T>::value) return small ? 64 : 256;
-    if (sizeof(T) == 4) return N < (1LL << 20) ? 128 : 256;
+    if (sizeof(T) == 4) {
+        if (N >= 3 << 13 && N < 3 << 14) return 32;
+        if (geq && N >= 3 << 14 && N <= 1 << 17) return 160;
+        return N < (1LL << 20) ? 128 : 256;
+    }
     if (small) return 32;
     auto busiest = [&](int tpb) { return ((N + tpb - 1) / tpb + 151) / 152 * tpb; };
     return busiest(192) < busiest(128) ? 192 : 128;
@@ -185,7 +195,7 @@ static int two_pass(lb_ctx *c, int nsteps)
     // launch shape: threads per CTA of both passes, sites per thread of the
     // phi pass (lb_set_kernel's block_x, block_y; 0 = default_threads, cut to
     // the collision's limit there, and 1)
-    const int tpb = c->block_x ? c->block_x : default_threads<T>(c->N);
+    const int tpb = c->block_x ? c->block_x : default_threads<T>(c->N, leaves_g_unread<T>(c));
     const int vvl = c->block_y ? c->block_y : 1;
     for (int t = 0; t < nsteps; t++) {
         const int a = c->buf.cur, b = 1 - a;
