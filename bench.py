@@ -38,8 +38,8 @@ BYTES_PER_SITE = {"fp32_shifted": 4 * 19 * 4, "fp64": 4 * 19 * 8}   # read+write
 # tau_g = 1 reduced form: collide reads f (19) + phi, writes f (19) + (gmh, u) (4);
 # the phi pass reads phi + (gmh, u) and writes phi -- 49 words per site
 BYTES_PER_SITE_TAUG1 = {"fp32_shifted": 49 * 4, "fp64": 49 * 8}
-# the library default with tau_g = 1: in FP32 the steps of one call keep g as
-# its moments (49 words); FP64 stores all of it
+# the library default with tau_g = 1: in FP32 the steps keep g as its moments
+# (49 words); FP64 stores all of it
 BYTES_PER_SITE_DEFAULT = {"fp32_shifted": 49 * 4, "fp64": 4 * 19 * 8}
 METRIC = "MLUPS and % of HBM roofline (fused step), FP32-shifted vs FP64 at stated error"
 ORACLE_SAMPLE = (64, 64, 64)
@@ -49,7 +49,8 @@ MRT_RATES = (1.3, 0.6)      # tau_bulk, tau_ghost of the MRT measurement
 MASK_DENSITY = 0.1          # fraction of sites selected in the masked-moments measurement
 FALLBACK_HBM = 6800.0
 # kernels one timestep launches, per lb_set_kernel choice
-STEP_KERNELS = {"auto": "timestep = k_phi_pull + k_collide_pull (two launches)",
+STEP_KERNELS = {"auto": {"fp32_shifted": "timestep = k_geq_phi + k_geq_collide (two launches)",
+                         "fp64": "timestep = k_phi_pull + k_collide_pull (two launches)"},
                 "two_pass": "timestep = k_phi_pull + k_collide_pull (two launches)",
                 "fused": "k_fused", "staged": "k_staged", "slab": "k_slab", "lag": "k_lag", "bulk": "k_bulk",
                 "taug1": "timestep = k_t1_collide + k_t1_phi (two launches)"}
@@ -539,10 +540,10 @@ def run_ours(args):
     tuned = {}
     for prec in ("fp32_shifted", "fp64"):
         t0 = time.perf_counter()
-        cached = tuning.cached_table(DIMS, prec) is not None
+        cached = tuning.cached_table(DIMS, prec, params=params) is not None
         cfg = tuning.ensure_tuned(DIMS, prec, params, phi0)
         tuned[prec] = {"config": list(cfg), "tuned_now": not cached, "seconds": time.perf_counter() - t0,
-                       "table": (tuning.cached_table(DIMS, prec) or {}).get("table")}
+                       "table": (tuning.cached_table(DIMS, prec, params=params) or {}).get("table")}
     results = {}
     for prec in ("fp32_shifted", "fp64"):
         cfg = tuple(tuned[prec]["config"])
@@ -601,10 +602,10 @@ def run_ours(args):
     tuned_t1 = {}
     for prec in ("fp32_shifted", "fp64"):
         t0 = time.perf_counter()
-        cached = tuning.cached_table(DIMS, prec, ("taug1",)) is not None
+        cached = tuning.cached_table(DIMS, prec, ("taug1",), params) is not None
         cfg = tuning.ensure_tuned(DIMS, prec, params, phi0, families=("taug1",))
         tuned_t1[prec] = {"config": list(cfg), "tuned_now": not cached, "seconds": time.perf_counter() - t0,
-                          "table": (tuning.cached_table(DIMS, prec, ("taug1",)) or {}).get("table")}
+                          "table": (tuning.cached_table(DIMS, prec, ("taug1",), params) or {}).get("table")}
     reduced = {prec: timed(prec, tuple(tuned_t1[prec]["config"]), 7) for prec in ("fp32_shifted", "fp64")}
     # masked moments (stream compaction) of a seeded 10 % site mask on the
     # benchmark lattice after the warm-up steps
@@ -705,17 +706,23 @@ def run_ours(args):
     def line_for(prec):
         r = results[prec]
         mlups = ws * n * args.steps / r["wall"] / 1e6
-        kernel = STEP_KERNELS.get(r["cfg"][0], r["cfg"][0])
-        # ncu summary of the kernel that ran (bulk: its own, with its sources listed)
-        prof = f"step_bulk_{prec}_256cubed" if r["cfg"][0] == "bulk" else f"step_{prec}_256cubed"
+        choice = r["cfg"][0]
+        kernel = STEP_KERNELS.get(choice, choice)
+        kernel = kernel[prec] if isinstance(kernel, dict) else kernel
+        # words a site that the kernel cannot do without, and the ncu summary
+        # of the kernel that ran (with its sources listed)
+        bytes_per_site = (BYTES_PER_SITE_DEFAULT if choice == "auto" else BYTES_PER_SITE)[prec]
+        prof = (f"step_bulk_{prec}_256cubed" if choice == "bulk" else
+                "step_default_fp32_256cubed" if (choice, prec) == ("auto", "fp32_shifted") else f"step_{prec}_256cubed")
         if prec == "fp32_shifted":
-            achieved = BYTES_PER_SITE[prec] * n / r["t_step"] / 1e9
+            achieved = bytes_per_site * n / r["t_step"] / 1e9
             roof = {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak, "traffic": _profile_value(prof, "dram_bytes_per_step"),
                     "peak_kind": f"{peak_kind} (copy bandwidth)",
-                    "algorithmic_bytes_per_launch": BYTES_PER_SITE[prec] * n,
+                    "algorithmic_bytes_per_launch": bytes_per_site * n,
                     "launch_seconds": r["t_step"], "timing": TIMING_NOTE,
-                    "frac_single_launches": BYTES_PER_SITE[prec] * n / r["t_launch"] / 1e9 / peak}
+                    # (a call of one default step writes g's 19 words as well)
+                    "frac_single_launches": (bytes_per_site + (19 * 4 if choice == "auto" else 0)) * n / r["t_launch"] / 1e9 / peak}
         else:
             # FP64 is bound by the FP64 pipe: flops per site from ncu counters
             fl = _profile_value(prof, "fp64_flops_per_site")
@@ -856,7 +863,7 @@ def run_ours(args):
                      **{f"{npts}pt": {prec: stencil_for(npts, prec) for prec in ("fp32_shifted", "fp64")}
                         for npts in (19, 27)}},
         "autotune": {"what": "kernel and launch shape of the headline (fp32_shifted) and of the fp64 line, "
-                             "chosen by tuning.autotune over the general-step kernels (two_pass: threads per CTA, "
+                             "chosen by tuning.autotune over the library default (auto) and the general-step kernels (two_pass: threads per CTA, "
                              "phi sites per thread; bulk: g slots, CTAs per y-cluster, planes per CTA; fused: "
                              "tile and z run); table rows are [config, seconds per step]",
                      **tuned},
@@ -1004,7 +1011,7 @@ def main():
     ap.add_argument("--lattice", type=int, nargs="+", default=[128],
                     help="edge of the --only lattice, or its three extents")
     ap.add_argument("--precision", choices=["fp32_shifted", "fp64", "fp64_df"], default="fp32_shifted")
-    ap.add_argument("--kernel", choices=["two_pass", "fused", "staged", "slab", "lag", "taug1", "bulk"], default=None,
+    ap.add_argument("--kernel", choices=["auto", "two_pass", "fused", "staged", "slab", "lag", "taug1", "bulk"], default=None,
                     help="override the tuned launch of the --only lattice")
     ap.add_argument("--block", type=int, nargs=3, default=(0, 0, 0), metavar=("BX", "BY", "ZC"))
     ap.add_argument("--stencil", type=int, choices=[7, 19, 27], default=7,

@@ -6,6 +6,9 @@ per thread) and the threads per block TPB (targetDP Sec. III.C and Sec. IV:
 VVL = 8 on the CPU, VVL = 2 on the K40).  Here the tuner chooses, for one
 lattice, among the step kernels themselves and their launch shapes:
 
+* the library default, ``("auto", 0, 0, 0)``, which no other candidate stands
+  for: FP32 steps with tau_g = 1 that keep g as its moments between steps, and
+  CTA sizes by the number of sites (timed with the ``two_pass`` family);
 * ``two_pass``: threads per CTA of both passes and sites per thread of the
   phi pass (the VVL axis), ``("two_pass", tpb, vvl, 0)``;
 * ``bulk``: shared-memory plane slots of g, CTAs per y-cluster and planes per
@@ -16,9 +19,11 @@ lattice, among the step kernels themselves and their launch shapes:
   warps per CTA and z run of its phi pass, ``("taug1", rows, warps, z_run)``.
 
 ``autotune`` times every candidate on the GPU through the C ABI and keeps the
-fastest in an on-disk cache keyed by GPU name, lattice extents, precision
-and family set; ``bench_config`` returns the cached choice (or the library
-default), ``ensure_tuned`` tunes on first use.  ``autotune_batch`` does the
+fastest in an on-disk cache keyed by GPU name, lattice extents, precision,
+family set and which of tau and tau_g are 1 (the kernels, and with them the
+fastest, depend on that); ``bench_config`` returns the cached choice (or the
+library default), without parameters the last one tuned for the lattice;
+``ensure_tuned`` tunes on first use.  ``autotune_batch`` does the
 same for an ensemble's (threads, CTAs per SM, CTA plan).
 """
 from __future__ import annotations
@@ -41,8 +46,9 @@ def _gpu_name() -> str:
     return torch.cuda.get_device_name() if torch.cuda.is_available() else "none"
 
 
-def _key(dims, precision, families=GENERAL) -> str:
-    return f"{_gpu_name()}|{dims[0]}x{dims[1]}x{dims[2]}|{precision}|{'+'.join(families)}|v4"
+def _key(dims, precision, families=GENERAL, params=None) -> str:
+    times = "any" if params is None else "".join(f"{t}{'=' if params.get(t) == 1.0 else '!='}1" for t in ("tau", "tau_g"))
+    return f"{_gpu_name()}|{dims[0]}x{dims[1]}x{dims[2]}|{precision}|{'+'.join(families)}|{times}|v5"
 
 
 def _load() -> dict:
@@ -63,16 +69,16 @@ def _save(key, entry):
     os.replace(tmp, CACHE)
 
 
-def bench_config(dims, precision, families=GENERAL):
+def bench_config(dims, precision, families=GENERAL, params=None):
     """Launch configuration cached for lattice ``dims`` in ``precision``
-    over ``families``, else the library default."""
-    hit = _load().get(_key(dims, precision, families))
+    over ``families`` (and ``params``), else the library default."""
+    hit = _load().get(_key(dims, precision, families, params))
     return tuple(hit["config"]) if hit else DEFAULT
 
 
-def cached_table(dims, precision, families=GENERAL):
+def cached_table(dims, precision, families=GENERAL, params=None):
     """The timed table behind a cached choice (None if not tuned)."""
-    return _load().get(_key(dims, precision, families))
+    return _load().get(_key(dims, precision, families, params))
 
 
 def _bulk_ok(dims, precision):
@@ -131,7 +137,8 @@ def autotune(dims, precision, params, phi0, configs=None, families=GENERAL, step
     table's rows are (config, seconds per step); configurations the library
     refuses for this lattice are skipped."""
     from .lattice import Lattice
-    configs = configs or candidates(precision, dims, families, params.get("tau_g"))
+    general = [DEFAULT] if "two_pass" in families else []
+    configs = configs or general + candidates(precision, dims, families, params.get("tau_g"))
     table = []
     with Lattice.from_params(dims, params, precision=precision) as lat:
         lat.init(phi0)
@@ -147,16 +154,18 @@ def autotune(dims, precision, params, phi0, configs=None, families=GENERAL, step
                 log(f"{cfg} {t * 1e3:.3f} ms")
     best = min(table, key=lambda r: r[1])
     if save:
-        _save(_key(dims, precision, families),
-              {"config": list(best[0]), "seconds_per_step": best[1], "steps": steps,
-               "table": [[list(c), t] for c, t in table], "when": time.strftime("%Y-%m-%dT%H:%M:%S")})
+        entry = {"config": list(best[0]), "seconds_per_step": best[1], "steps": steps,
+                 "table": [[list(c), t] for c, t in table], "when": time.strftime("%Y-%m-%dT%H:%M:%S")}
+        for p in (params, None):
+            _save(_key(dims, precision, families, p), entry)
     return best[0], table
 
 
 def ensure_tuned(dims, precision, params, phi0, families=GENERAL, log=None):
-    """The cached choice for ``dims``/``precision``/``families``, tuning on
-    first use (the cache lives beside the built library)."""
-    hit = _load().get(_key(dims, precision, families))
+    """The cached choice for ``dims``/``precision``/``families`` and which
+    relaxation times of ``params`` are 1, tuning on first use (the cache lives
+    beside the built library)."""
+    hit = _load().get(_key(dims, precision, families, params))
     if hit:
         return tuple(hit["config"])
     best, _ = autotune(dims, precision, params, phi0, families=families, log=log)
@@ -166,7 +175,7 @@ def ensure_tuned(dims, precision, params, phi0, families=GENERAL, log=None):
 def _batch_key(batch) -> str:
     import hashlib
     h = hashlib.sha256(repr([sorted(d.items()) for d in batch.specs]).encode()).hexdigest()[:12]
-    return f"{_gpu_name()}|batch{len(batch)}:{h}|{batch.precision}|{getattr(batch, 'form', 'general')}|v3"
+    return f"{_gpu_name()}|batch{len(batch)}:{h}|{batch.precision}|{getattr(batch, 'form', 'general')}|v4"
 
 
 def batch_candidates(precision):
