@@ -514,6 +514,30 @@ def _adjoint(torch):
             "dJ_dkappa": g, "dJ_dkappa_fd_richardson": fd_rich, "rel_diff_vs_fd": abs(g - fd_rich) / abs(fd_rich)}
 
 
+def _reduce_line(prec, t, n, fp64_tflops, peak, peak_kind):
+    """lb_reduce of n sites in t seconds.  FP32 storage is summed on the FP32
+    units and bound by the 38 stored words a site, against the copy bandwidth;
+    FP64 storage by the FP64 pipe: additions per site from ncu counters against
+    the measured FP64 FMA-instruction rate (the probe's TFLOP/s over 2)."""
+    hbm = prec == "fp32_shifted"
+    adds = _profile_value("reduce_128cubed", f"fp64_adds_per_site_{prec}")
+    tr = _profile_value("reduce_128cubed", f"dram_bytes_per_site_{prec}")
+    gbs = 38 * (4 if hbm else 8) * n / t / 1e9
+    rate, rate_peak = adds * n / t / 1e12 if adds else None, fp64_tflops / 2 if fp64_tflops else None
+    rate_frac = rate / rate_peak if (rate and rate_peak) else None
+    if hbm:
+        bound = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
+                 "peak_kind": f"{peak_kind} (copy bandwidth)", "fp64_instr_frac": rate_frac}
+    else:
+        bound = {"bound": "alu (FP64 pipe)", "achieved": rate, "peak": rate_peak, "unit": "T FP64 instructions/s",
+                 "frac": rate_frac, "peak_kind": "measured in this run: FMA instructions/s of lb_probe_fp64_fma"}
+    return {"ms_per_call": t * 1e3, "sites_per_s": n / t,
+            "roofline": {**bound, "kernel": "k_reduce", "fp64_adds_per_site": adds,
+                         "achieved_gbs": gbs, "hbm_frac": gbs / peak, "traffic": tr * n if tr else None,
+                         "timing": "median of 10 calls, CUDA events around each (the kernel, the "
+                                   "read-back of its result and the return)"}}
+
+
 def run_ours(args):
     import torch
     ws, rank, local = _dist()
@@ -786,26 +810,7 @@ def run_ours(args):
         return out
 
     def reduce_for(prec):
-        # lb_reduce: FP32 storage is summed on the FP32 units and bound by the
-        # 38 stored words a site; FP64 storage by the FP64 pipe: additions per
-        # site from ncu counters against the measured FP64 FMA-instruction
-        # rate (the probe's TFLOP/s over 2)
-        t = results[prec]["t_reduce"]
-        adds = _profile_value("reduce_128cubed", f"fp64_adds_per_site_{prec}")
-        pk = fp64_peak["tflops"]
-        gbs = 38 * (4 if prec == "fp32_shifted" else 8) * n / t / 1e9
-        ach = adds * n / t / 1e12 if adds else None
-        tr = _profile_value("reduce_128cubed", f"dram_bytes_per_site_{prec}")
-        return {"ms_per_call": t * 1e3, "sites_per_s": n / t,
-                "roofline": {"bound": "hbm" if prec == "fp32_shifted" else "alu (FP64 pipe)", "kernel": "k_reduce",
-                             "achieved": ach,
-                             "peak": pk / 2 if pk else None, "unit": "T FP64 instructions/s",
-                             "frac": ach / (pk / 2) if (ach and pk) else None, "fp64_adds_per_site": adds,
-                             "peak_kind": "measured in this run: FMA instructions/s of lb_probe_fp64_fma",
-                             "achieved_gbs": gbs, "hbm_frac": gbs / peak,
-                             "traffic": tr * n if tr else None,
-                             "timing": "median of 10 calls, CUDA events around each (the kernel, the "
-                                       "48-byte read-back and the return)"}}
+        return _reduce_line(prec, results[prec]["t_reduce"], n, fp64_peak["tflops"], peak, peak_kind)
 
     def df_line():
         r = df
