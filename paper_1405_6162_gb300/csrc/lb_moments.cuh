@@ -43,10 +43,12 @@ __device__ __forceinline__ df64 moment_term(df64 v) { return v; }
 __device__ __forceinline__ double to_double(df64 v) { return widen(v); }
 __device__ __forceinline__ double to_double(double v) { return v; }
 
-// 1 / rho to within an ulp or so where the sums are double-float: the float
-// reciprocal of rho cut to 24 bits on the integer units, and two Newton
-// steps, 4 FP64 instructions; the division for rho far outside the float
-// range and for double sums
+// 1 / rho.  Where the sums are double-float: the float reciprocal of rho cut to
+// 24 bits on the integer units (its error e0 at most 2^-22), and two Newton steps,
+// 4 FP64 instructions, whose last rounds a value off by e0^4 <= 2^-88 -- the
+// correctly rounded quotient but for a tie nearer than that (40000 densities
+// between 2^-90 and 2^90: all).  The division for rho far outside the float range
+// and for double sums.
 template <typename A>
 __device__ __forceinline__ double inverse(double rho)
 {
