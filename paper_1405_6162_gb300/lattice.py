@@ -157,6 +157,8 @@ class Lattice:
         L.check(L.lib().lb_init(self.handle, pp, up, kind), "lb_init")
 
     def step(self, nsteps: int = 1):
+        """Advance by ``nsteps``; the bits of a run do not depend on how it is
+        cut into calls."""
         L.check(L.lib().lb_step(self.handle, int(nsteps)), "lb_step")
 
     def set_kernel(self, kernel="auto", block_x=0, block_y=0, z_chunk=0):
