@@ -111,10 +111,10 @@ struct Coll {
 // Equilibria of f and g at one site.  R is rho (SH = false) or rho - rho0
 // (SH = true: the result is feq_i - w_i rho0).  j = sum f c = rho u.
 // sink(i, feq_i, geq_i) is called once per direction, i a literal after
-// inlining.  Direct sums, the least error of FP64 and double-float storage.
+// inlining.  Direct sums, for double-float storage.
 template <typename T, bool SH, typename Sink>
-__device__ __forceinline__ void equilibria(const Coll<T>& p, T R, T jx, T jy, T jz,
-                                           T phi, T dx, T dy, T dz, T lap, Sink&& sink)
+__device__ __forceinline__ void equilibria_direct(const Coll<T>& p, T R, T jx, T jy, T jz,
+                                                  T phi, T dx, T dy, T dz, T lap, Sink&& sink)
 {
     const T third = T(1.0 / 3.0);
     const T rho = SH ? p.rho0 + R : R;
@@ -189,14 +189,15 @@ __device__ __forceinline__ T scaled(float c, T x)
     return T(c) * x;
 }
 
-// The same for values that are rounded to float storage, at density rho0 and
-// velocity u = (ux, uy, uz), with fewer instructions.  SH: feq_i - w_i rho0 in
-// place of feq_i.  FLOW = false: u = 0, nothing of it is computed and opposite
-// values are equal.  The sums are not renormalised, nor are the values that
-// sink gets.  Kept in double-float they err by up to a quarter more (rms over
-// starts of amplitude 1e-4 to 1), rounded to float by the same to nine digits.
+// The same at density rho0 and velocity u = (ux, uy, uz), with fewer
+// instructions, for float and FP64 storage.  SH: feq_i - w_i rho0 in place of
+// feq_i.  FLOW = false: u = 0, nothing of it is computed and opposite values are
+// equal.  For df64 the sums are not renormalised, nor are the values that sink
+// gets: kept in double-float f errs by up to a quarter more than by the direct
+// sums (rms over starts of amplitude 1e-4 to 1), rounded to float by the same to
+// nine digits.
 template <typename T, bool SH, bool FLOW, typename Sink>
-__device__ __forceinline__ void equilibria_float(const Coll<T>& p, T ux, T uy, T uz, T phi, T dx, T dy, T dz, T lap,
+__device__ __forceinline__ void equilibria(const Coll<T>& p, T ux, T uy, T uz, T phi, T dx, T dy, T dz, T lap,
                                            Sink&& sink)
 {
     const T zero = T(0);

@@ -24,20 +24,62 @@ namespace lbk {
 // equilibria in double.  Float and double-float storage evaluate them in
 // double-float arithmetic on the FP32 units (df64.cuh, ~48 bits; the double
 // pipe runs at 1/64 of the float rate), with the inputs split on the integer
-// units: double-float storage keeps the value, float storage the float nearest
-// to it, the same float as rounding a double result except at a near tie.
-// Without u0 float storage does not form half of the sums (opposite values are
-// equal).
-// Float, 7 points: 256^3 593 us without u0 (380 is the copy rate over its
-// bytes) and 1109 with it, bound by the FP32 units; 27 points, 129x97x65 147 and
-// 151, bound by the stencil's FP64 instructions.  With the inputs
-// converted on the FP64 pipe and direct sums 1659, 1963, 179 and 201.
+// units: double-float storage keeps the value, by direct sums, float storage the
+// float nearest to it, the same float as rounding a double result except at a
+// near tie.  Without u0 float and double storage do not form half of the sums
+// (opposite values are equal).
+// Float, 7 points: 256^3 592 us without u0 (380 is the copy rate over its
+// bytes) and 1102 with it, bound by the FP32 units.  With the inputs converted on
+// the FP64 pipe and direct sums 1657 and 1959.
 __device__ __forceinline__ void init_store(float *a, size_t o, df64 v) { a[o] = __fadd_rn(v.hi, v.lo); }
 template <typename T>
 __device__ __forceinline__ void init_store(T *a, size_t o, T v)
 {
     a[o] = v;
 }
+// The wide stencils in double by opposite pairs (their sums and differences),
+// with fewer of the FP64 instructions that bound the start of float storage than
+// stencil_np: 129x97x65, 27 points, 112 us without u0 and 119 with it, by single
+// values 147 and 151; 19 points 75 and 93, 96 and 105.
+template <int NP>
+__device__ __forceinline__ void stencil_pairs(const double *__restrict__ phi, const Nbr &n, double ph, double (&d)[3],
+                                              double &lap)
+{
+    static_assert(NP == 19 || NP == 27, "the 7-point differences are pairs already");
+    // by class (faces, edges, corners), differences by axis too; the first term
+    // of each is not added to a zero (0 + x is an instruction)
+    double sum[3], dif[3][3];
+    int terms[4][3] = {};
+    auto add = [](double &to, int &n, double x) { to = n++ ? to + x : x; };
+#pragma unroll
+    for (int a = 0; a <= 1; a++)
+#pragma unroll
+        for (int b = -1; b <= 1; b++)
+#pragma unroll
+            for (int c = -1; c <= 1; c++) {
+                // one of each pair: the first component that is not zero is 1
+                if (a == 0 && (b < 0 || (b == 0 && c <= 0))) continue;
+                const int k = a * a + b * b + c * c - 1;
+                if (k == 2 && NP == 19) continue;
+                const double vp = phi[n.at(a, b, c)], vm = phi[n.at(-a, -b, -c)];
+                const double m = vp - vm;
+                add(sum[k], terms[3][k], vp + vm);
+                if (a) add(dif[0][k], terms[0][k], m);
+                if (b) add(dif[1][k], terms[1][k], b > 0 ? m : -m);
+                if (c) add(dif[2][k], terms[2][k], c > 0 ? m : -m);
+            }
+    constexpr double w1 = NP == 19 ? 1.0 / 18.0 : 2.0 / 27.0, w2 = NP == 19 ? 1.0 / 36.0 : 1.0 / 54.0;
+    constexpr double w3 = NP == 19 ? 0.0 : 1.0 / 216.0;
+    constexpr double out = 6.0 * (6.0 * w1 + 12.0 * w2 + 8.0 * w3);   // the weights of all neighbours
+#pragma unroll
+    for (int x = 0; x < 3; x++) {
+        d[x] = 3.0 * w1 * dif[x][0] + 3.0 * w2 * dif[x][1];
+        if constexpr (NP == 27) d[x] += 3.0 * w3 * dif[x][2];
+    }
+    lap = 6.0 * w1 * sum[0] + 6.0 * w2 * sum[1] - out * ph;
+    if constexpr (NP == 27) lap += 6.0 * w3 * sum[2];
+}
+
 template <typename E>
 __device__ __forceinline__ E init_arith(double v)
 {
@@ -59,24 +101,27 @@ __global__ void __launch_bounds__(256) k_init(const double *__restrict__ phi0,
     if (s >= N) return;
     const Nbr n(s, nx, ny, nz);
     const double ph = phi0[s];
-    double dx, dy, dz, lap;
-    stencil_np<NP, double>(phi0, n, ph, dx, dy, dz, lap);
+    double d[3], lap;
+    if constexpr (std::is_same<T, float>::value && NP != 7)
+        stencil_pairs<NP>(phi0, n, ph, d, lap);
+    else
+        stencil_np<NP, double>(phi0, n, ph, d[0], d[1], d[2], lap);
     E v[3] = {E(0), E(0), E(0)};   // u, or rho0 u
     if (FLOW)
 #pragma unroll
         for (int a = 0; a < 3; a++)
-            v[a] = init_arith<E>(std::is_same<T, float>::value ? u0[a * N + s] : rho0 * u0[a * N + s]);
-    const E q = init_arith<E>(ph), gx = init_arith<E>(dx), gy = init_arith<E>(dy), gz = init_arith<E>(dz);
+            v[a] = init_arith<E>(is_df64<T>::value ? rho0 * u0[a * N + s] : u0[a * N + s]);
+    const E q = init_arith<E>(ph), gx = init_arith<E>(d[0]), gy = init_arith<E>(d[1]), gz = init_arith<E>(d[2]);
     const E l = init_arith<E>(lap);
     auto sink = [&](int i, E fe, E ge) {
         const size_t o = (size_t)i * S + n.src(i);
         init_store(fa, o, fe);
         init_store(ga, o, ge);
     };
-    if constexpr (std::is_same<T, float>::value)
-        equilibria_float<E, SH, FLOW>(p, v[0], v[1], v[2], q, gx, gy, gz, l, sink);
+    if constexpr (is_df64<T>::value)
+        equilibria_direct<E, SH>(p, p.rho0, v[0], v[1], v[2], q, gx, gy, gz, l, sink);
     else
-        equilibria<E, SH>(p, SH ? E(0) : p.rho0, v[0], v[1], v[2], q, gx, gy, gz, l, sink);
+        equilibria<E, SH, FLOW>(p, v[0], v[1], v[2], q, gx, gy, gz, l, sink);
 }
 
 // ------------------------------------------------------------------ moments / state
