@@ -233,7 +233,7 @@ int lb_set_state_masked(lb_ctx *c, const unsigned char *mask, const double *f, c
  * to 256), block_y the sites per
  * thread of the phi pass (1, 2 or 4; 0 = 1) and z_chunk must be 0.  For
  * LB_KERNEL_LAG block_x must be 0 or 256, block_y 0 or 1, and z_chunk is the
- * lag slack in site blocks beyond the stencil's reach (0 = default 128).
+ * lag slack in site blocks beyond the stencil's reach (0 = default 608).
  * For LB_KERNEL_BULK block_x is the number of shared-memory plane slots of
  * g (3..8, or 2 in FP32: the lean form, no copies ahead, three CTAs per SM;
  * 0 = 3), block_y the CTAs per cluster along

@@ -108,7 +108,6 @@ inline Mrt<T> make_mrt(const lb_ctx *c)
 }
 
 constexpr int kLagBlock = 256;       // sites per block of the lagged kernel
-constexpr long long kLagSlack = 128;  // extra lag (blocks) beyond the stencil reach
 constexpr int kReduceBlocks = 304;   // 2 x 152 SMs, one wave; fixed so sums are reproducible
 constexpr int kReduceThreads = 256;
 

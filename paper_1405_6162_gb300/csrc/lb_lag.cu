@@ -181,6 +181,13 @@ __global__ void __launch_bounds__(kLagBlock) k_lag(const T *__restrict__ fa, con
     }
 }
 
+// Extra lag (blocks) beyond the stencil's reach: as many as run at a time (152
+// SMs, 4 CTAs of 256), so that a block's neighbours have been finished, not only
+// begun, when it is collided.  With 128 the waits set the pace, and worse the
+// more CTAs fit an SM: FP32 256^3 2504 us a step (1972 when 3 fitted) / 1112, 128^3
+// 314 / 145, 64^3 59 / 24, FP64 256^3 10674 / 8017; 512 to 2048 within 3 %.
+constexpr long long kLagSlack = 608;
+
 template <typename T, bool SH>
 int run_lag(lb_ctx *c, int nsteps)
 {
