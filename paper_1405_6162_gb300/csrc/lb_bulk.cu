@@ -565,8 +565,8 @@ static int run_bulk(lb_ctx *c, int nsteps)
 // CTA (the fastest measured at 256^3 FP32-shifted on GB300), on rows of 256
 // sites (eight warps a CTA; at 128^3, four warps a CTA, the two-pass step is
 // faster: 17.4 against 14.2 GLUPS) and tau_g != 1: with tau_g = 1 g need not
-// be read by the collision, and 50 steps of 256^3 take 530 us each
-// (lb_taug1.cu) against 902 here, a single one 777
+// be read by the collision, and 50 steps of 256^3 take 516 us each
+// (lb_taug1.cu) against 902 here, a single one 713
 constexpr int kAutoSlots = 3, kAutoCluster = 2, kAutoPlanes = 16;
 
 bool auto_uses_bulk(const lb_ctx *c)
