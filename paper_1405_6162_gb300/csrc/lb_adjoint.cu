@@ -16,6 +16,8 @@
 // feeds rho and the stress, its odd part the momentum.
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "d3q19.cuh"
 #include "lb_internal.cuh"
 #include "lb_pdl.cuh"
@@ -27,12 +29,18 @@ namespace {
 
 // Model parameters, and the relaxation rate folded into the factors of the
 // weight sums below (formed on the host): R = w/36, O = w/12 (3 w/36),
-// T = w/8 (9/2 w/36), W = w/24 (3/2 w/36), w the rate of f or of g.
+// T = w/8 (9/2 w/36), W = w/24 (3/2 w/36), w the rate of f or of g.  R and W in two
+// parts: an adjoint that is the same for all velocities is multiplied by 36 R in
+// every step and has no stress, 12 T = 36 W, and with each rounded by itself,
+// 2^-54 off with the same sign, gradients drifted by 1.25e-16 a step (5e-19 now;
+// four instructions more, 64^3 168.0 -> 169.6 us a reverse step).
+struct AdjRate {
+    double R, Rlo, O, T, W, Wlo;
+};
 struct AdjP {
     double rho0, gamma, A, B, B3, kappa, kappa2;   // B3 = 3 B, kappa2 = 2 kappa
     double keep_f, keep_g;                         // 1 - w: the part of f, g that a step keeps
-    double fR, fO, fT, fW;
-    double gR, gO, gT, gW;
+    AdjRate f, g;
 };
 
 // Sums of a distribution's adjoint F over the velocities, weighted in units
@@ -85,10 +93,10 @@ __device__ __forceinline__ void equilibrium_vjp(const AdjP &p, double rinv, cons
 {
     const double third = 1.0 / 3.0;
     // feq_i = w_i [rho + 3 c.j + 9/2 c S c - 3/2 tr S],  S = pb I + kappa d d + j j / rho
-    const double fw = p.fW * mf.W;
-    const double S[3][3] = {{p.fT * mf.Txx - fw, p.fT * mf.Txy, p.fT * mf.Txz},
-                            {p.fT * mf.Txy, p.fT * mf.Tyy - fw, p.fT * mf.Tyz},
-                            {p.fT * mf.Txz, p.fT * mf.Tyz, p.fT * mf.Tzz - fw}};
+    const double fw = fma(p.f.W, mf.W, p.f.Wlo * mf.W);
+    const double S[3][3] = {{p.f.T * mf.Txx - fw, p.f.T * mf.Txy, p.f.T * mf.Txz},
+                            {p.f.T * mf.Txy, p.f.T * mf.Tyy - fw, p.f.T * mf.Tyz},
+                            {p.f.T * mf.Txz, p.f.T * mf.Tyz, p.f.T * mf.Tzz - fw}};
     const double pb_b = S[0][0] + S[1][1] + S[2][2];
     const double kpb = p.kappa * pb_b;
     double dSd = 0.0, uSu = 0.0, Su[3];
@@ -103,13 +111,13 @@ __device__ __forceinline__ void equilibrium_vjp(const AdjP &p, double rinv, cons
         }
     }
     // geq_i = w_i [phi + 3 phi c.u + 9/2 c G c - 3/2 tr G],  G = (Gamma mu - phi/3) I + phi u u
-    const double gw = p.gW * mg.W;
-    const double G[3][3] = {{p.gT * mg.Txx - gw, p.gT * mg.Txy, p.gT * mg.Txz},
-                            {p.gT * mg.Txy, p.gT * mg.Tyy - gw, p.gT * mg.Tyz},
-                            {p.gT * mg.Txz, p.gT * mg.Tyz, p.gT * mg.Tzz - gw}};
+    const double gw = fma(p.g.W, mg.W, p.g.Wlo * mg.W);
+    const double G[3][3] = {{p.g.T * mg.Txx - gw, p.g.T * mg.Txy, p.g.T * mg.Txz},
+                            {p.g.T * mg.Txy, p.g.T * mg.Tyy - gw, p.g.T * mg.Tyz},
+                            {p.g.T * mg.Txz, p.g.T * mg.Tyz, p.g.T * mg.Tzz - gw}};
     const double trG = G[0][0] + G[1][1] + G[2][2];
     const double mu_b = p.gamma * trG;
-    const double o[3] = {p.gO * mg.Ox, p.gO * mg.Oy, p.gO * mg.Oz};
+    const double o[3] = {p.g.O * mg.Ox, p.g.O * mg.Oy, p.g.O * mg.Oz};
     double uo = 0.0, uGu = 0.0, Gu[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -119,17 +127,17 @@ __device__ __forceinline__ void equilibrium_vjp(const AdjP &p, double rinv, cons
     }
     // pb = A/2 phi^2 + 3B/4 phi^4 - kappa phi lap - kappa/2 |d|^2;  mu = A phi + B phi^3 - kappa lap
     const double dmu = p.A + p.B3 * (phi * phi);
-    phi_b = (p.gR * mg.W + uo) + (uGu - third * trG) + pb_b * (phi * dmu - p.kappa * lap) + mu_b * dmu;
+    phi_b = fma(p.g.R, mg.W, fma(p.g.Rlo, mg.W, uo)) + (uGu - third * trG) + pb_b * (phi * dmu - p.kappa * lap) + mu_b * dmu;
     lap_b = -(kpb * phi + p.kappa * mu_b);
     const double dd = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
     kap_b = dSd - pb_b * (phi * lap + 0.5 * dd) - lap * mu_b;
     if (!INIT) {
         // u = j / rho: with v = o + 2 G u, dJ/du = phi v (of g), dJ/dj = dJ/du / rho + 2 S u + direct
         const double pr = phi * rinv;
-        const double fo[3] = {p.fO * mf.Ox, p.fO * mf.Oy, p.fO * mf.Oz};
+        const double fo[3] = {p.f.O * mf.Ox, p.f.O * mf.Oy, p.f.O * mf.Oz};
 #pragma unroll
         for (int a = 0; a < 3; a++) j_b[a] = (fo[a] + 2.0 * Su[a]) + pr * (o[a] + 2.0 * Gu[a]);
-        rho_b = (p.fR * mf.W - uSu) - pr * (uo + 2.0 * uGu);
+        rho_b = fma(p.f.R, mf.W, fma(p.f.Rlo, mf.W, -uSu)) - pr * (uo + 2.0 * uGu);
     }
 }
 
@@ -306,6 +314,20 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_seed(const double *__restri
     }
 }
 
+// the factors of a rate, R and W as what T (rounded) makes them: 2/9 T and T/3,
+// the second parts from the first's exact remainders
+AdjRate adj_rate(double w)
+{
+    AdjRate a;
+    a.O = w / 12.0;
+    a.T = w / 8.0;
+    a.R = 2.0 * a.T / 9.0;
+    a.Rlo = std::fma(-9.0, a.R, 2.0 * a.T) / 9.0;
+    a.W = a.T / 3.0;
+    a.Wlo = std::fma(-3.0, a.W, a.T) / 3.0;
+    return a;
+}
+
 // rates w, w_g: 1 for the equilibria of the initialisation
 AdjP adj_params(const lb_params &q, double w, double wg)
 {
@@ -319,14 +341,8 @@ AdjP adj_params(const lb_params &q, double w, double wg)
     p.kappa2 = 2.0 * q.kappa;
     p.keep_f = 1.0 - w;
     p.keep_g = 1.0 - wg;
-    p.fR = w / 36.0;
-    p.fO = w / 12.0;
-    p.fT = w / 8.0;
-    p.fW = w / 24.0;
-    p.gR = wg / 36.0;
-    p.gO = wg / 12.0;
-    p.gT = wg / 8.0;
-    p.gW = wg / 24.0;
+    p.f = adj_rate(w);
+    p.g = adj_rate(wg);
     return p;
 }
 

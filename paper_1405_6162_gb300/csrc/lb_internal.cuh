@@ -166,7 +166,7 @@ int taug1_g_rows(lb_ctx *c, int i0, int i1, double *out);
 int taug1_phi_out(lb_ctx *c, double *out);
 
 // LB_KERNEL_AUTO with tau_g = 1, FP32-shifted: steps that keep g as its
-// equilibrium's moments within a call
+// equilibrium's moments between steps
 bool auto_uses_geq(const lb_ctx *c);
 int launch_step_geq(lb_ctx *c, int nsteps);
 
